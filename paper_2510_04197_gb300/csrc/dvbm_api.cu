@@ -156,6 +156,13 @@ static void set_step_factors(dvbm_ctx* c) {
       c->P.kyr[k] = c->P.kyv[k] / (4.0 * c->P.lq);
     }
     c->P.kyvf[k] = (float)c->P.kyv[k];
+    // |k| <= 1 (check_dt), so the fractions stay below 2^61
+    int L = 0;
+    while ((1 << L) < c->P.lq) ++L;
+    const double fold = c->P.lq > 0 ? (double)(1 << L) / c->P.lq : 1.0;
+    c->P.kxq[k] = (long long)std::llround(std::ldexp(std::fabs(c->P.kxv[k]) * fold, 60));
+    c->P.kyq[k] = (long long)std::llround(std::ldexp(std::fabs(c->P.kyv[k]) * fold, 60));
+    c->P.advn = 1 + L;
   }
   c->P.dt = c->dt;
   c->P.dt_mu = c->dt / c->mu;

@@ -9,6 +9,7 @@
 //     F_pq = W_p W_q sum_{a+b<=N} A_ab He_a(xi_p) He_b(xi_q) / (a! b!).
 #pragma once
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 namespace dvbm {
@@ -64,6 +65,11 @@ struct Phys {
   double kxr[5], kyr[5]; // kxv / (4 lq), kyv / (4 lq): flux factors of the scaled differences
   double kxv[5], kyv[5]; // dt/dx * c * xi_k and dt/dy * c * xi_k
   float kxvf[5], kyvf[5];
+  // tile advection of FP64 storage: |kxv|, |kyv| as 2^60-fractions with the
+  // limiter's scale folded in (times 2^L / lq, L = ceil(log2 lq); lq counts as 1
+  // for a general beta), and the values' extra shift 1 + L below 60 bits
+  long long kxq[5], kyq[5];
+  int advn;
   double fref0, gref0;   // FP32DEV reference: f_ref = w rho0, g_ref = w rho0 (C_v - R) T0
   double rho_ref_mom;    // unused padding for alignment
 };
@@ -118,6 +124,23 @@ __device__ __forceinline__ EqF eq_f(double rho, double ux, double uy, double s) 
   return e;
 }
 
+// 1/x with one Halley step from the single-precision reciprocal: relative error
+// e = 1 - x r of about 2^-23 becomes e^3 plus rounding (three FP64 instructions;
+// the compiler's division takes about three times as many).  Outside the
+// single-precision range, and for non-finite x, the plain division.
+__device__ __forceinline__ double recip(double x) {
+  const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;
+  if (ex - 903u >= 240u) return 1.0 / x;  // |x| outside [2^-120, 2^120)
+  // x rounded down to 24 bits as a float, and back, by bit manipulation (the
+  // hardware conversions run at the FP64 rate)
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const float f = __uint_as_float((hi & 0x80000000u) | (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29));
+  const unsigned u = __float_as_uint(__frcp_rn(f));
+  const double r = __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // Collision coefficients from the moments (Sec. II.C relaxation times,
 // Table I split-II quasi-equilibria).  PRC selects the Prandtl case at
 // compile time: -1 (Pr < 1), 0 (Pr = 1), +1 (Pr > 1).
@@ -127,79 +150,74 @@ __device__ __forceinline__ EqF eq_f(double rho, double ux, double uy, double s) 
 // with Delta = H_2(f) - A^eq_2, Delta' its traceless part and
 // S(u, A)_abc = [u_a A_bc]_cyc - tr(A)/(D+2) [u_a d_bc]_cyc, the symmetric
 // tensor whose contraction is the heat-flux constraint 2 (A u)_a.
+// FP64 work is what bounds this function's kernels, so k1 = dt/tau1 enters at
+// the zeroth coefficient and runs through the equilibrium recurrences, and
+// k1 A^eq + s1 (A* - A^eq) is written k1 A* + k2 (A^eq - A*) with k2 = Pr k1
+// (Pr <= 1) or s1 = k1 - k2 on the deviations alone (Pr > 1): 84 FP64
+// instructions instead of 114.
 template <int PRC>
 __device__ __forceinline__ Coeffs collision_coeffs(const Moments& m, const Phys& P) {
   Coeffs C;
   const double rho = m.m00;
-  const double irho = 1.0 / rho;
+  const double irho = recip(rho);
   const double ux = m.m10 * irho, uy = m.m01 * irho;
   const double Et = fma(0.5, m.m20 + m.m02, m.g00 * P.inv_c2);        // E / c^2
   const double theta = P.gm1 * fma(-0.5, fma(ux, ux, uy * uy), Et * irho);
   const double s = theta - 1.0;
   C.bad = !(rho > 0.0) || !(theta > 0.0) || !(fabs(Et) < 1e300);
-  const double p = rho * P.c2 * theta;                                   // rho R T
-  double k1, k2;                                                         // dt/tau1, dt/tau2
-  if (PRC <= 0) { k1 = P.dt_mu * p; k2 = k1 * P.Pr; }
-  else          { k2 = P.dt_mu * p; k1 = k2 * P.Pr; }
-  const double s1 = k1 - k2;
+  const double rt = rho * theta;                                         // p / c^2
+  const double kp = (P.dt_mu * P.c2) * rt;                               // dt p / mu
+  const double k1 = PRC <= 0 ? kp : kp * P.Pr;                           // dt/tau1
   C.a1 = 1.0 - k1;
   C.k1 = k1;
-  EqF e = eq_f(rho, ux, uy, s);
-  // deviations dA = A* - A^eq (zero where Table I keeps equilibrium moments)
-  double d20 = 0, d11 = 0, d02 = 0, d30 = 0, d21 = 0, d12 = 0, d03 = 0;
-  double d40 = 0, d31 = 0, d13 = 0, d04 = 0, dg10 = 0, dg01 = 0;
-  const double reps = rho * P.epsf * theta;                               // rho eps / c^2
+  const EqF e = eq_f(k1 * rho, ux, uy, s);                               // k1 A^eq
+  C.f00 = e.a00; C.f10 = e.a10; C.f01 = e.a01;
+  C.f20 = e.a20; C.f11 = e.a11; C.f02 = e.a02;
+  C.f30 = e.a30; C.f21 = e.a21; C.f12 = e.a12; C.f03 = e.a03;
+  C.f40 = e.a40; C.f31 = e.a31; C.f22 = e.a22; C.f13 = e.a13; C.f04 = e.a04;
+  // k1 A^eq of g (split II, physical units): rho eps (1, u, uu + s I)
+  const double kr = e.a00 * (theta * (P.epsf * P.c2));
+  const double krx = kr * ux, kry = kr * uy, krs = kr * s;
+  C.g00 = kr;
+  C.g10 = krx;
+  C.g01 = kry;
+  C.g20 = fma(krx, ux, krs);
+  C.g11 = krx * uy;
+  C.g02 = fma(kry, uy, krs);
   if (PRC != 0) {
-    // Delta = H_2(f) - A^eq_2 with H_20 = mu_20 - rho, H_11 = mu_11, H_02 = mu_02 - rho
-    const double Dxx = (m.m20 - rho) - e.a20;
-    const double Dxy = m.m11 - e.a11;
-    const double Dyy = (m.m02 - rho) - e.a02;
+    // Delta = H_2(f) - A^eq_2: mu_20 - rho theta - rho ux^2, mu_11 - rho ux uy, ...
+    const double Dxx = fma(-m.m10, ux, m.m20 - rt);
+    const double Dxy = fma(-m.m10, uy, m.m11);
+    const double Dyy = fma(-m.m01, uy, m.m02 - rt);
     if (PRC < 0) {
+      const double s1 = fma(-P.Pr, k1, k1);                             // dt/tau1 - dt/tau2
       const double kap = 0.25 * (Dxx + Dyy);                            // tr(Delta)/(D+2)
       const double Px = Dxx - kap, Py = Dyy - kap;
-      // H_3(f): mu_30 - 3 mu_10, mu_21 - mu_01, mu_12 - mu_10, mu_03 - 3 mu_01
-      d30 = (fma(-3.0, m.m10, m.m30) - e.a30) - 3.0 * ux * Px;
-      d21 = ((m.m21 - m.m01) - e.a21) - fma(2.0 * ux, Dxy, uy * Px);
-      d12 = ((m.m12 - m.m10) - e.a12) - fma(2.0 * uy, Dxy, ux * Py);
-      d03 = (fma(-3.0, m.m01, m.m03) - e.a03) - 3.0 * uy * Py;
-      // g*: first moment of g (in units of c^2), minus its equilibrium value
-      dg10 = m.g10 * P.inv_c2 - reps * ux;
-      dg01 = m.g01 * P.inv_c2 - reps * uy;
+      // A*_3 = H_3(f) - S(u, Delta); H_3: mu_30 - 3 mu_10, mu_21 - mu_01, mu_12 - mu_10, mu_03 - 3 mu_01
+      const double x30 = fma(-3.0 * ux, Px, fma(-3.0, m.m10, m.m30));
+      const double x21 = fma(-2.0 * ux, Dxy, fma(-uy, Px, m.m21 - m.m01));
+      const double x12 = fma(-2.0 * uy, Dxy, fma(-ux, Py, m.m12 - m.m10));
+      const double x03 = fma(-3.0 * uy, Py, fma(-3.0, m.m01, m.m03));
+      C.f30 = fma(s1, x30, P.Pr * C.f30);
+      C.f21 = fma(s1, x21, P.Pr * C.f21);
+      C.f12 = fma(s1, x12, P.Pr * C.f12);
+      C.f03 = fma(s1, x03, P.Pr * C.f03);
+      // g*: first moment of g
+      C.g10 = fma(s1, m.g10, P.Pr * krx);
+      C.g01 = fma(s1, m.g01, P.Pr * kry);
     } else {
-      const double Tx = 0.5 * (Dxx - Dyy);                              // Delta'_xx = -Delta'_yy
-      d20 = Tx; d11 = Dxy; d02 = -Tx;
-      d30 = 3.0 * ux * Tx;
-      d21 = fma(uy, Tx, 2.0 * ux * Dxy);
-      d12 = fma(-ux, Tx, 2.0 * uy * Dxy);
-      d03 = -3.0 * uy * Tx;
-      d40 = -6.0 * Tx; d31 = -3.0 * Dxy; d13 = -3.0 * Dxy; d04 = 6.0 * Tx;
+      const double s1 = k1 - kp;
+      const double tx = s1 * (0.5 * (Dxx - Dyy));                       // s1 Delta'_xx = -s1 Delta'_yy
+      const double ty = s1 * Dxy;
+      C.f20 += tx; C.f11 += ty; C.f02 -= tx;
+      C.f30 = fma(3.0 * ux, tx, C.f30);
+      C.f21 = fma(uy, tx, fma(2.0 * ux, ty, C.f21));
+      C.f12 = fma(-ux, tx, fma(2.0 * uy, ty, C.f12));
+      C.f03 = fma(-3.0 * uy, tx, C.f03);
+      C.f40 = fma(-6.0, tx, C.f40); C.f31 = fma(-3.0, ty, C.f31);
+      C.f13 = fma(-3.0, ty, C.f13); C.f04 = fma(6.0, tx, C.f04);
     }
   }
-  C.f00 = k1 * e.a00;
-  C.f10 = k1 * e.a10;
-  C.f01 = k1 * e.a01;
-  C.f20 = fma(s1, d20, k1 * e.a20);
-  C.f11 = fma(s1, d11, k1 * e.a11);
-  C.f02 = fma(s1, d02, k1 * e.a02);
-  C.f30 = fma(s1, d30, k1 * e.a30);
-  C.f21 = fma(s1, d21, k1 * e.a21);
-  C.f12 = fma(s1, d12, k1 * e.a12);
-  C.f03 = fma(s1, d03, k1 * e.a03);
-  C.f40 = fma(s1, d40, k1 * e.a40);
-  C.f31 = fma(s1, d31, k1 * e.a31);
-  C.f22 = k1 * e.a22;
-  C.f13 = fma(s1, d13, k1 * e.a13);
-  C.f04 = fma(s1, d04, k1 * e.a04);
-  // g^eq (split II): A00 = rho eps, A10 = rho eps ux, A20 = rho eps (ux^2 + s) ...
-  // (units of c^2; multiplied back by c^2 for physical g)
-  const double kg = k1 * P.c2;
-  const double sg = s1 * P.c2;
-  C.g00 = kg * reps;
-  C.g10 = fma(sg, dg10, kg * reps * ux);
-  C.g01 = fma(sg, dg01, kg * reps * uy);
-  C.g20 = kg * reps * fma(ux, ux, s);
-  C.g11 = kg * reps * ux * uy;
-  C.g02 = kg * reps * fma(uy, uy, s);
   return C;
 }
 
@@ -385,6 +403,194 @@ __device__ __forceinline__ double ll_to_double_rn(long long F, int scale) {
   const int ex = 1023 + 63 - lz + scale + carry;
   const unsigned hi = (unsigned)(frac >> 32) | ((unsigned)ex << 20) | (F < 0 ? 0x80000000u : 0u);
   return __hiloint2double((int)hi, (int)(unsigned)frac);
+}
+
+// address of a warp-uniform pointer plus a lane's 32-bit byte offset
+template <class T>
+__device__ __forceinline__ T* at(T* base, unsigned off) {
+  typedef typename std::conditional<std::is_const<T>::value, const char, char>::type B;
+  return (T*)((B*)base + off);
+}
+
+// ---- limb products on the integer multiply-add pipe ------------------------
+// A 64-bit by 64-bit high-word product (__mul64hi) runs at 3.8 lanes / clock /
+// SM on GB300 (measured; it is built from half-rate 32-bit high multiplies),
+// a 32 x 32 + 64-bit multiply-add at 62.  Fixed-point factors are therefore
+// kept as two signed 32-bit limbs, x = h 2^32 + l with l in [-2^31, 2^31), and
+// a sum of products x_i k_i / 2^64 is three wide multiply-adds per product: the
+// high products and the two cross products have an accumulator each, the low
+// product (below one unit of the result) is left out.
+__host__ __device__ constexpr int limb_lo(long long x) { return (int)(unsigned)(unsigned long long)x; }
+__host__ __device__ constexpr int limb_hi(long long x) {
+  return (int)((x - (long long)limb_lo(x)) >> 32);
+}
+struct LimbAcc {
+  long long hi = 0, mid = 0;
+  __device__ __forceinline__ void mac(int xh, int xl, int kh, int kl) {
+    // written as the instruction: a compiler's reassociation splits the sums
+    // into separate multiplies and adds
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(hi) : "r"(xh), "r"(kh));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(mid) : "r"(xh), "r"(kl));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(mid) : "r"(xl), "r"(kh));
+  }
+  // the sum / 2^64: rounded to nearest or down, or / 2^61 (down)
+  __device__ __forceinline__ long long value() const { return hi + ((mid + 0x80000000ll) >> 32); }
+  __device__ __forceinline__ long long floor() const { return hi + (mid >> 32); }
+  __device__ __forceinline__ long long value8() const { return (hi << 3) + (mid >> 29); }
+};
+struct Limbs {
+  int h, l;
+  __device__ __forceinline__ explicit Limbs(long long x) : h((int)(x >> 32) + (int)((unsigned)x >> 31)), l((int)x) {}
+};
+// limbs packed into one 64-bit word (high word h, low word l)
+__device__ __forceinline__ long long pack_limbs(long long x) { return x + ((x & 0x80000000ll) << 1); }
+
+// ---- block fixed point ------------------------------------------------------
+// Exponent key of a double: its high word without the sign, so that the largest
+// key of a block has the block's largest exponent in bits 20..30.
+__device__ __forceinline__ unsigned abs_key(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+__device__ __forceinline__ unsigned abs_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+
+// Value v as an integer of 60 - n0 bits at the block exponent E (n0 >= 0):
+// v = X 2^(E - 1082 + n0); magnitudes are truncated, negative values are the
+// ones' complement of theirs (one unit more).  A value of larger exponent than
+// E (only non-finite ones are left out of the block maximum) gives 0.
+__device__ __forceinline__ long long block_fix(double v, int E, int n0) {
+  const int hi = __double2hiint(v);
+  const unsigned lo = (unsigned)__double2loint(v);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
+  const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 7;
+  const unsigned n = min((unsigned)(E - e + n0), 63u);
+  return (long long)(m >> n) ^ (long long)(hi >> 31);
+}
+// the same for a float: v = X 2^(E - 186 + n0)
+__device__ __forceinline__ long long block_fix(float v, int E, int n0) {
+  const int u = __float_as_int(v);
+  const int e = (u >> 23) & 0xff;
+  const unsigned mh = (((unsigned)u & 0x7fffffu) | 0x800000u) << 4;
+  const unsigned n = min((unsigned)(E - e + n0), 63u);
+  return (long long)(((unsigned long long)mh << 32) >> n) ^ (long long)(u >> 31);
+}
+
+// int64 -> double by bit manipulation, value F 2^scale: one count of leading
+// zeros on the word that holds the leading one.  RN rounds to nearest (ties
+// away), otherwise the bits below 2^-52 of the value are dropped; a negative F
+// counts one unit less in magnitude (see block_fix).  The value's exponent must
+// lie in the normal range.
+template <bool RN>
+__device__ __forceinline__ double fix_to_double(long long F, int scale) {
+  const int s = (int)(F >> 63);
+  const unsigned hi = (unsigned)(int)(F >> 32) ^ (unsigned)s, lo = (unsigned)F ^ (unsigned)s;
+  const bool low = hi == 0u;
+  const unsigned top = low ? lo : hi;
+  const int n = __clz((int)top) + (low ? 32 : 0);
+  // leading one at bit 62 (|F| < 2^62); a carry out of the rounded significand
+  // goes into the exponent below, which is exactly right
+  const unsigned long long norm = ((((unsigned long long)hi) << 32) | lo) << ((n - 1) & 63);
+  const unsigned long long r = (norm + (RN ? 0x200u : 0u)) >> 10;
+  const unsigned rh = (unsigned)(r >> 32) + ((unsigned)(1023 + 62 - n + scale) << 20);
+  const double v = __hiloint2double((int)(rh | ((unsigned)s & 0x80000000u)), (int)(unsigned)r);
+  return top == 0u ? 0.0 : v;
+}
+
+// ---- moments in block fixed point -------------------------------------------
+// The 13 moments of a cell (Sec. II.D.1) without FP64 arithmetic: on GB300 an
+// FP64 instruction takes the issue time of 32 integer ones.  The 25 populations
+// of f (of g) are brought to their largest exponent as 58-bit integers
+// (truncated below 2^-57 of the largest, finer than the rounding of a double
+// sum); sums are exact, and the powers of the abscissae are fixed-point factors
+// rounded from their exact values to 2^-62 (factors rounded to double leave a
+// drift of a few 1e-17 a step between the moments and the equilibria built from
+// them).  A non-finite population makes the zeroth moment NaN, which the
+// caller's checks see.
+// XA^n and XB^n times 2^62 / 4, / 16, / 32 (n = 1, 2, 3)
+constexpr long long kXA[4] = {0, 1562930575100362931ll, 529687401272071863ll, 359029054183477437ll};
+constexpr long long kXB[4] = {0, 3293862167010879573ll, 2352616360245045577ll, 3360677197683338703ll};
+// the weighted sum over the two node pairs, (XB^n b + XA^n a) / 16, / 64, / 128 (n = 1, 2, 3)
+template <int n>
+__device__ __forceinline__ long long pair_sum(long long b, long long a) {
+  const Limbs x(b), y(a);
+  LimbAcc s;
+  s.mac(x.h, x.l, limb_hi(kXB[n]), limb_lo(kXB[n]));
+  s.mac(y.h, y.l, limb_hi(kXA[n]), limb_lo(kXA[n]));
+  return s.value();
+}
+
+template <class S>
+__device__ __forceinline__ Moments moments_fix(const S* __restrict__ s, unsigned off, long long PL) {
+  constexpr int kBias = sizeof(S) == 8 ? 1080 : 184;
+  constexpr int kExpBits = sizeof(S) == 8 ? 20 : 23;
+  constexpr unsigned kInf = sizeof(S) == 8 ? 0x7ff00000u : 0x7f800000u;
+  constexpr int kTiny = sizeof(S) == 8 ? 128 : 0;  // blocks below this exponent count as zero
+  Moments m;
+  bool finite = true;
+  {
+    S v[25];
+    unsigned key = 0;
+#pragma unroll
+    for (int i = 0; i < 25; ++i) {
+      v[i] = __ldg(at(s + i * PL, off));
+      key = max(key, abs_key(v[i]));
+    }
+    finite = key < kInf;
+    const int E = (int)(key >> kExpBits);
+    const int n0 = E < kTiny ? 63 : 2;
+    long long M0[5], M1[5], M2[5], M3s = 0;  // y-sums of each x-node, M1, M2, M3 times 1/16, 1/64, 1/128
+#pragma unroll
+    for (int p = 0; p < 5; ++p) {
+      const long long x0 = block_fix(v[5 * p], E, n0), x1 = block_fix(v[5 * p + 1], E, n0),
+                      x2 = block_fix(v[5 * p + 2], E, n0), x3 = block_fix(v[5 * p + 3], E, n0),
+                      x4 = block_fix(v[5 * p + 4], E, n0);
+      const long long sA = x1 + x2, dA = x1 - x2, sB = x3 + x4, dB = x3 - x4;
+      M0[p] = x0 + sA + sB;
+      M1[p] = pair_sum<1>(dB, dA);
+      M2[p] = pair_sum<2>(sB, sA);
+      M3s += pair_sum<3>(dB, dA);
+    }
+    const long long a0 = M0[1] + M0[2], b0 = M0[3] + M0[4], c0 = M0[1] - M0[2], d0 = M0[3] - M0[4];
+    // second factors: the first left four spare bits
+    const long long a1 = M1[1] + M1[2], b1 = M1[3] + M1[4], c1 = M1[1] - M1[2], d1 = M1[3] - M1[4];
+    const long long a2 = M2[1] + M2[2], b2 = M2[3] + M2[4], c2 = M2[1] - M2[2], d2 = M2[3] - M2[4];
+    const int sc = E - kBias;
+    m.m00 = fix_to_double<true>(M0[0] + a0 + b0, sc);
+    m.m01 = fix_to_double<true>(M1[0] + a1 + b1, sc + 4);
+    m.m02 = fix_to_double<true>(M2[0] + a2 + b2, sc + 6);
+    m.m03 = fix_to_double<true>(M3s, sc + 7);
+    m.m10 = fix_to_double<true>(pair_sum<1>(d0, c0), sc + 4);
+    m.m20 = fix_to_double<true>(pair_sum<2>(b0, a0), sc + 6);
+    m.m30 = fix_to_double<true>(pair_sum<3>(d0, c0), sc + 7);
+    m.m11 = fix_to_double<true>(pair_sum<1>(d1 << 4, c1 << 4), sc + 4);
+    m.m21 = fix_to_double<true>(pair_sum<2>(b1 << 4, a1 << 4), sc + 6);
+    m.m12 = fix_to_double<true>(pair_sum<1>(d2 << 4, c2 << 4), sc + 6);
+  }
+  {
+    S v[25];
+    unsigned key = 0;
+#pragma unroll
+    for (int i = 0; i < 25; ++i) {
+      v[i] = __ldg(at(s + (25 + i) * PL, off));
+      key = max(key, abs_key(v[i]));
+    }
+    finite = finite && key < kInf;
+    const int E = (int)(key >> kExpBits);
+    const int n0 = E < kTiny ? 63 : 2;
+    long long N0[5], N1s = 0;
+#pragma unroll
+    for (int p = 0; p < 5; ++p) {
+      const long long x0 = block_fix(v[5 * p], E, n0), x1 = block_fix(v[5 * p + 1], E, n0),
+                      x2 = block_fix(v[5 * p + 2], E, n0), x3 = block_fix(v[5 * p + 3], E, n0),
+                      x4 = block_fix(v[5 * p + 4], E, n0);
+      N0[p] = x0 + (x1 + x2) + (x3 + x4);
+      N1s += pair_sum<1>(x3 - x4, x1 - x2);
+    }
+    const int sc = E - kBias;
+    m.g00 = fix_to_double<true>(N0[0] + (N0[1] + N0[2]) + (N0[3] + N0[4]), sc);
+    m.g01 = fix_to_double<true>(N1s, sc + 4);
+    m.g10 = fix_to_double<true>(pair_sum<1>(N0[3] - N0[4], N0[1] - N0[2]), sc + 4);
+  }
+  if (!finite) m.m00 = __longlong_as_double(0x7ff8000000000000ll);
+  return m;
 }
 
 struct CoeffsFix {
@@ -620,38 +826,200 @@ __device__ __forceinline__ double flux_difference_rat_v(double a0, double a1, do
   return ll_to_double_scaled(F, E - 1074);  // value = F 2^(E - 1074)
 }
 
-// slope_rat together with the minmod branch it took: 0 (a and b differ in
-// sign), 1 (2 lp Da), 2 (lq (Da + Db)), 3 (2 lp Db), ties resolved in that
-// order.  The value equals slope_rat's.
-__device__ __forceinline__ long long slope_rat_code(long long Da, long long Db, long long lp2, long long lq,
-                                                    int& code) {
-  const long long ra = lp2 * Da, rb = lp2 * Db, y = lq * (Da + Db);
-  int br;
-  if (Da >= 0) br = (ra <= y && ra <= rb) ? 1 : (y <= rb ? 2 : 3);
-  else br = (ra >= y && ra >= rb) ? 1 : (y >= rb ? 2 : 3);
-  if ((Da ^ Db) < 0) br = 0;
-  code = br;
-  return br == 0 ? 0ll : (br == 1 ? ra : (br == 2 ? y : rb));
+// ---- advection of one population over a tile (FP64 storage) -----------------
+// The update's flux differences (Sec. III.A.2) of one population over a tile of
+// up to 32 x 8 cells, by one warp, in block fixed point: the tile's cells and
+// its upwind halo share one exponent, so every value is converted once (a
+// per-cell stencil converts eight values per cell), differences are exact, and
+// each limited slope is computed once and handed to the neighbour (along x by
+// a warp shuffle, along y in registers while the warp walks the rows).
+//
+// The scheme is mirror symmetric, so a tile is walked in the population's own
+// direction: stream coordinates i, j run along +v_x and +v_y, and one body
+// serves all signs.  With D_j = F_j - F_{j-1} and sigma_j = minmod3(hb D_j,
+// (D_j + D_{j+1})/4, hb D_{j+1}) the face value downstream of cell j is
+// F_j + sigma_j, and the cell's change is -k ((F_j + sigma_j) - (F_{j-1} + sigma_{j-1})).
+// Everything is kept times 4 lq (beta = lp / lq: candidates 2 lp D and
+// lq (D + D')); a general beta takes lq = 1 and a fixed-point beta.
+constexpr int kTileY = 8;                 // CTA = 32 x kTileY cells
+constexpr int kCta = 32 * kTileY;
+constexpr int kAdvPitch = 36, kAdvRows = kTileY + 3;  // stream columns -2 .. 32, rows -2 .. 8
+
+// x k + y for a small k >= 0: two multiply-adds (a sign-extended 64-bit k takes three)
+__device__ __forceinline__ long long mad_small(long long x, unsigned k, long long y) {
+  unsigned lo, hi;
+  asm("{\n\t.reg .u64 t;\n\tmad.wide.u32 t, %2, %3, %4;\n\tmov.b64 {%0, %1}, t;\n\t}"
+      : "=r"(lo), "=r"(hi)
+      : "r"((unsigned)x), "r"(k), "l"(y));
+  hi += (unsigned)(x >> 32) * k;
+  return (long long)(((unsigned long long)hi << 32) | lo);
 }
 
-// flux_difference_rat_v that also returns the branch code of the cell's own
-// slope sigma_j (first argument its backward, second its forward difference):
-// s_bc for v > 0, s_ab for v < 0.  The adjoint reads these codes instead of
-// re-deriving them from the state.
-__device__ __forceinline__ double flux_difference_rat_code_v(double a0, double a1, double a2, double a3, int lp,
-                                                             int lq, int sgn, int& code) {
-  const int E = max(max(bexp(a0), bexp(a1)), max(bexp(a2), bexp(a3)));
-  const long long x0 = to_block_fixed52(a0, E), x1 = to_block_fixed52(a1, E), x2 = to_block_fixed52(a2, E),
-                  x3 = to_block_fixed52(a3, E);
-  const long long Da = x1 - x0, Db = x2 - x1, Dc = x3 - x2;
-  const long long lp2 = 2 * lp, q4 = 4 * lq;
-  int c_ab, c_bc;
-  const long long s_ab = slope_rat_code(Da, Db, lp2, lq, c_ab);
-  const long long s_bc = slope_rat_code(Db, Dc, lp2, lq, c_bc);
-  code = sgn > 0 ? c_bc : c_ab;
-  const long long F = sgn > 0 ? q4 * Db + s_bc - s_ab : q4 * Db - s_bc + s_ab;
-  if (E < 64) return 0.0;
-  return ll_to_double_scaled(F, E - 1074);
+// scaled limited slope 4 lq sigma(a, b)
+template <bool RAT>
+__device__ __forceinline__ long long slope_fix(long long a, long long b, const Phys& P) {
+  const long long t = a + b;
+  const bool neg = t < 0;
+  const long long m = ((a < b) != neg) ? a : b;  // the smaller in magnitude, where the signs agree
+  const bool differ = (a ^ b) < 0;               // else the slope is zero: the first candidate counts as 0
+  long long r1, r2;
+  if (RAT) {
+    r1 = mad_small(m, differ ? 0u : 2u * (unsigned)P.lp, 0);
+    r2 = mad_small(t, (unsigned)P.lq, 0);
+  } else {
+    const Limbs x(differ ? 0ll : m << 3);
+    const Limbs h(P.hq);
+    LimbAcc s;
+    s.mac(x.h, x.l, h.h, h.l);
+    r1 = s.floor() << 1;  // 2 beta m
+    r2 = t;
+  }
+  return ((r1 < r2) != neg) ? r1 : r2;
+}
+
+// minmod branch of the cell's own slope as the adjoint reads it (backward
+// difference first, in grid direction): 0 signs differ, 1 hb Da, 2 (Da + Db)/4,
+// 3 hb Db, ties in that order; rational limiter
+__device__ __forceinline__ unsigned slope_branch_code(long long a, long long b, bool mirrored, const Phys& P) {
+  const long long Da = mirrored ? -b : a, Db = mirrored ? -a : b;
+  if ((Da ^ Db) < 0) return 0u;
+  const long long ra = Da * (long long)(2 * P.lp), rb = Db * (long long)(2 * P.lp), y = (Da + Db) * (long long)P.lq;
+  if (Da >= 0) return (ra <= y && ra <= rb) ? 1u : (y <= rb ? 2u : 3u);
+  return (ra >= y && ra >= rb) ? 1u : (y >= rb ? 2u : 3u);
+}
+
+struct AdvTile {
+  int W, H;          // cells of the tile (ragged at the grid's upper ends)
+  bool fx, fy;       // walked against x, against y
+  int lane;
+};
+// What a warp reads of one population: its lane's column in stream rows -2 .. 8,
+// and one cell of the x-halo.  Read one population ahead, so that the loads'
+// latency passes during the walk over the previous one.
+struct AdvLoad {
+  double v[kAdvRows], h;
+};
+// plane: the population's plane at the tile's lowest cell.  Every lane and row
+// loads, in ragged tiles the last column and the row after the tile again, so
+// that the loads need no predicates.
+__device__ __forceinline__ void advect_load(AdvLoad& L, const double* __restrict__ plane, long long PT,
+                                            const AdvTile& T) {
+  const int i = min(T.lane, T.W - 1);
+  const unsigned lx = (unsigned)(T.fx ? T.W - 1 - i : i) * 8u;
+  const long long sy = T.fy ? -PT : PT;
+  const double* row0 = plane + (T.fy ? (T.H - 1) * PT : 0);  // stream row 0
+#pragma unroll
+  for (int j = -2; j <= kTileY; ++j) L.v[j + 2] = __ldg(at(row0 + min(j, T.H) * sy, lx));
+  const int hr = min(T.lane & 7, T.H - 1), hc = T.lane >> 3;  // halo cell: row hr, stream column -2, -1, W (or 0)
+  const int h = hc == 3 ? 0 : hc == 2 ? T.W : hc - 2;
+  L.h = __ldg(row0 + hr * sy + (T.fx ? T.W - 1 - h : h));
+}
+
+// out: the plane (at the tile's lowest cell, row pitch PT) where the tile's flux
+// sums go, kx (x-face difference) + ky (y-face difference) as integers W in
+// units of 2^(E - 1079), E the returned block exponent; MX, MY: the population
+// moves along x, along y; kx, ky: flux factors (Phys::kxq, kyq); xs: this warp's
+// [kAdvRows][kAdvPitch] words of shared memory; code: (CODES) this population's
+// branch codes at the tile's lowest cell, row pitch cpitch; next: starts the
+// next population's loads into L.
+template <bool MX, bool MY, bool RAT, bool CODES, class Next>
+__device__ __forceinline__ int advect_tile(AdvLoad& L, const Next& next, long long* out, long long PT, const AdvTile& T,
+                                           const Phys& P, long long kx, long long ky, long long* xs,
+                                           unsigned char* code, long long cpitch) {
+  const int lane = T.lane;
+  const bool in = lane < T.W;
+  const unsigned lx = in ? (unsigned)(T.fx ? T.W - 1 - lane : lane) : 0u;  // this lane's column of the tile
+  const long long sy = T.fy ? -PT : PT;
+  constexpr int J0 = MY ? -2 : 0, J1 = MY ? kTileY : kTileY - 1;  // rows this population needs
+  const double* v = L.v + (J0 + 2);
+  const double vh = L.h;
+  const int hr = lane & 7, hc = lane >> 3;
+  const bool hin = MX && hc < 3 && hr < T.H;
+  // block exponent; non-finite values are left out (their key wraps to 0)
+  unsigned key = 0;
+#pragma unroll
+  for (int j = 0; j <= J1 - J0; ++j) key = max(key, ((unsigned)__double2hiint(v[j]) + 0x100000u) & 0x7fffffffu);
+  if (MX) key = max(key, ((unsigned)__double2hiint(vh) + 0x100000u) & 0x7fffffffu);
+  key = __reduce_max_sync(0xffffffffu, key);
+  const int E = (int)(key >> 20) - 1;
+  const int n0 = E < 128 ? 63 : P.advn;  // a block of negligible values has no flux
+  __syncwarp();                          // the previous population's reads of xs are done
+#pragma unroll
+  for (int j = J0; j <= J1; ++j) xs[(j + 2) * kAdvPitch + lane + 2] = block_fix(v[j - J0], E, n0);
+  if (MX) {
+    __syncwarp();  // column W of a ragged tile is written twice: the halo value last
+    if (hin) xs[(hr + 2) * kAdvPitch + (hc == 2 ? T.W + 2 : hc)] = block_fix(vh, E, n0);
+  }
+  next();
+  __syncwarp();
+  const unsigned q4 = RAT ? 4u * (unsigned)P.lq : 4u;
+  if (MX) {
+    // scaled face value upstream of column 0, one row per lane, kept in column -2
+    if (lane < T.H) {
+      long long* r = xs + (lane + 2) * kAdvPitch;
+      const long long a = r[1] - r[0], b = r[2] - r[1];
+      r[0] = mad_small(r[1], q4, slope_fix<RAT>(a, b, P));
+    }
+    __syncwarp();
+  }
+  const Limbs KX(kx), KY(ky);
+  const long long* own = xs + 2 * kAdvPitch + lane + 2;  // (row 0, this column)
+  long long c = own[0], dy = 0, gy = 0;
+  if (MY) {
+    const long long b = own[-kAdvPitch], a = own[-2 * kAdvPitch];
+    dy = c - b;
+    gy = mad_small(b, q4, slope_fix<RAT>(b - a, dy, P));
+  }
+  long long* orow = out + (T.fy ? (T.H - 1) * PT : 0);
+  unsigned char* crow = CODES ? code + (T.fy ? (T.H - 1) * cpitch : 0) : nullptr;
+  const long long csy = T.fy ? -cpitch : cpitch;
+#pragma unroll 1
+  for (int j = 0; j < T.H; ++j) {
+    LimbAcc w;
+    unsigned bits = 0;
+    if (MX) {
+      const long long a = c - own[-1], b = own[1] - c;
+      const long long g = mad_small(c, q4, slope_fix<RAT>(a, b, P));
+      const long long e = xs[(j + 2) * kAdvPitch];
+      long long gl = __shfl_up_sync(0xffffffffu, g, 1);
+      if (lane == 0) gl = e;
+      const Limbs f(g - gl);
+      w.mac(f.h, f.l, KX.h, KX.l);
+      if (CODES) bits = slope_branch_code(a, b, T.fx, P);
+    }
+    const long long cn = own[kAdvPitch];
+    if (MY) {
+      const long long dn = cn - c;
+      const long long g = mad_small(c, q4, slope_fix<RAT>(dy, dn, P));
+      const Limbs f(g - gy);
+      w.mac(f.h, f.l, KY.h, KY.l);
+      if (CODES) bits |= slope_branch_code(dy, dn, T.fy, P) << 2;
+      gy = g;
+      dy = dn;
+    }
+    if (in) {
+      *at(orow, lx * 8) = w.floor();
+      if (CODES) crow[lx] = (unsigned char)bits;
+    }
+    c = cn;
+    own += kAdvPitch;
+    orow += sy;
+    if (CODES) crow += csy;
+  }
+  return E;
+}
+
+// a1 F + target - flux sum of one population: the target t 2^(st - 1079) and
+// the flux sum w 2^(sw - 1079) are subtracted as integers at the larger of
+// their scales, so that one conversion and one FMA are left.  Both are rounded
+// down, so the mean errors cancel in the difference.  The conversion is the
+// hardware's: it takes one slot of the FP64 pipe, which the kernel does not
+// fill, for about twenty integer instructions.
+__device__ __forceinline__ double collide_advect(double a1, double F, long long t, int st, long long w, int sw) {
+  const int d = sw - st;
+  const double z = __ll2double_rn((t >> min(max(d, 0), 63)) - (w >> min(max(-d, 0), 63)));
+  const int zh = __double2hiint(z);
+  return fma(a1, F, __hiloint2double(zh == 0 ? 0 : zh + ((max(sw, st) - 1079) << 20), __double2loint(z)));
 }
 
 // Flux difference F_{j+1/2} - F_{j-1/2} of the upwind-limited face values
