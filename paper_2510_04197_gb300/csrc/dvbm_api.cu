@@ -342,10 +342,24 @@ static dvbm_status fill_ghosts(dvbm_ctx* c, void* b) {
   return DVBM_OK;
 }
 
+// the ghost layers that a step's kernel left (storage, bc: the step's) in b
+static cudaError_t ghosts_after_step(int lattice, int storage, void* b, const Geom& G, const Phys& P, const Macro& M,
+                                     BCDev bc, cudaStream_t st) {
+  if (step_writes_images(storage, G)) {
+    bool any = false;
+    for (int s = 0; s < 4; ++s) {
+      if (bc.kind[s] == DVBM_BC_WALL) any = true;
+      else bc.kind[s] = DVBM_BC_EXTERNAL;
+    }
+    if (!any) return cudaSuccess;
+  }
+  return launch_ghost(lattice, storage, b, G, P, M, bc, st);
+}
+
 // lattice dispatch of the per-step and diagnostic kernels
 static cudaError_t l_step(dvbm_ctx* c, const void* src, void* dst) {
-  return c->lattice == DVBM_D2Q16_SPLIT_I ? launch_step16(src, dst, c->G, c->P, c->flag, c->stream)
-                                          : launch_step(c->storage, src, dst, c->G, c->P, c->flag, c->stream);
+  return c->lattice == DVBM_D2Q16_SPLIT_I ? launch_step16(src, dst, c->G, c->P, c->bc, c->flag, c->stream)
+                                          : launch_step(c->storage, src, dst, c->G, c->P, c->bc, c->flag, c->stream);
 }
 static cudaError_t l_init(dvbm_ctx* c, void* dst, const double* const* F) {
   return launch_init(c->lattice, c->storage, dst, F[0], F[1], F[2], F[3], c->G, c->P, c->M, c->stream);
@@ -496,8 +510,8 @@ extern "C" dvbm_status dvbm_step(dvbm_ctx* c, int n) {
     void* src = c->buf[c->cur];
     void* dst = c->buf[1 - c->cur];
     CUDA_TRY(c, l_step(c, src, dst));
-    dvbm_status s = fill_ghosts(c, dst);
-    if (s != DVBM_OK) return s;
+    CUDA_TRY(c, ghosts_after_step(c->lattice, c->storage, dst, c->G, c->P, c->M, c->bc, c->stream));
+    dvbm_status s = DVBM_OK;
     c->cur = 1 - c->cur;
     ++c->steps;
     c->halo_fresh = false;
@@ -755,10 +769,11 @@ extern "C" dvbm_status dvbm_adjoint(dvbm_ctx* c, const double* dL_drho, const do
     const long long nrec = coded ? E - S : E - S - 1;
     for (long long t = 0; t < nrec && e == cudaSuccess; ++t) {
       if (coded)
-        e = launch_step_codes(seg[t], seg[t + 1], c->G, c->P, c->flag, codes + t * code_step,
+        e = launch_step_codes(seg[t], seg[t + 1], c->G, c->P, c->bc, c->flag, codes + t * code_step,
                               moms ? moms + t * mom_step : nullptr, c->stream);
-      else e = launch_step(0, seg[t], seg[t + 1], c->G, c->P, c->flag, c->stream);
-      if (e == cudaSuccess && t + 1 < E - S) e = launch_ghost(DVBM_D2Q25_SPLIT_II, 0, seg[t + 1], c->G, c->P, c->M, c->bc, c->stream);
+      else e = launch_step(0, seg[t], seg[t + 1], c->G, c->P, c->bc, c->flag, c->stream);
+      if (e == cudaSuccess && t + 1 < E - S)
+        e = ghosts_after_step(DVBM_D2Q25_SPLIT_II, 0, seg[t + 1], c->G, c->P, c->M, c->bc, c->stream);
     }
     for (long long t = E - S - 1; t >= 0 && e == cudaSuccess; --t) {
       e = launch_adjoint_step((const double*)seg[t], (const double*)lam[a], (double*)lam[1 - a],
@@ -903,12 +918,12 @@ extern "C" dvbm_status dvbm_adjoint_advance(dvbm_ctx* c, int* halo) {
       break;
     case AdjRecompute:  // one forward step of the segment
       if (coded)
-        e = launch_step_codes(A.seg[A.t], A.seg[A.t + 1], c->G, c->P, c->flag, A.codes + A.t * code_step,
+        e = launch_step_codes(A.seg[A.t], A.seg[A.t + 1], c->G, c->P, c->bc, c->flag, A.codes + A.t * code_step,
                               A.moms + A.t * mom_step, c->stream);
       else
-        e = launch_step(0, A.seg[A.t], A.seg[A.t + 1], c->G, c->P, c->flag, c->stream);
+        e = launch_step(0, A.seg[A.t], A.seg[A.t + 1], c->G, c->P, c->bc, c->flag, c->stream);
       if (e == cudaSuccess)
-        e = launch_ghost(DVBM_D2Q25_SPLIT_II, 0, A.seg[A.t + 1], c->G, c->P, c->M, c->bc, c->stream);
+        e = ghosts_after_step(DVBM_D2Q25_SPLIT_II, 0, A.seg[A.t + 1], c->G, c->P, c->M, c->bc, c->stream);
       A.code_t = A.t;
       ++A.t;
       A.halo = A.seg[A.t];

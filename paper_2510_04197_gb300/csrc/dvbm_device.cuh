@@ -741,64 +741,6 @@ __device__ __forceinline__ void write_equilibrium_fix(S* d, long long PL, Coeffs
   write_node_fix<S, 4>(d, PL, X, F.Ef, F.Eg);
 }
 
-// float -> double by bit manipulation (exact; the hardware conversion runs on
-// the FP64 pipe on GB300).  Zero and subnormal floats give a signed zero;
-// infinities and NaNs keep their class.
-__device__ __forceinline__ double f2d_bits(float v) {
-  const unsigned u = __float_as_uint(v);
-  const unsigned e = (u >> 23) & 0xffu;
-  const unsigned sign = u & 0x80000000u;
-  const unsigned m = u & 0x7fffffu;
-  unsigned hi = sign | ((e + 896u) << 20) | (m >> 3);
-  unsigned lo = m << 29;
-  if (e == 0u) { hi = sign; lo = 0u; }
-  if (e == 255u) hi = sign | 0x7ff00000u | (m >> 3);
-  return __hiloint2double((int)hi, (int)lo);
-}
-
-// value of integer F at block exponent E: F 2^(E - 1082)
-__device__ __forceinline__ double from_block_fixed(long long F, int E) {
-  if (E < 64) return 0.0;
-  return ll_to_double_scaled(F, E - 1082);
-}
-
-// limited slope on integers: minmod3(hb Da, (Da + Db)/4, hb Db); Hq = hb 2^62
-__device__ __forceinline__ long long slope_int(long long Da, long long Db, long long ra, long long rb) {
-  const long long y = (Da + Db) >> 2;
-  const long long mn = min(min(ra, y), rb), mx = max(max(ra, y), rb);
-  const bool same = (Da ^ Db) >= 0;
-  return same ? (Da >= 0 ? mn : mx) : 0ll;
-}
-
-// F_{j+1/2} - F_{j-1/2} (general beta) from the stencil values a0..a3 (v > 0:
-// cells j-2..j+1; v < 0: cells j-1..j+2)
-__device__ __forceinline__ double flux_difference_int_v(double a0, double a1, double a2, double a3, long long Hq,
-                                                        int sgn) {
-  const int E = max(max(bexp(a0), bexp(a1)), max(bexp(a2), bexp(a3)));
-  const long long x0 = to_block_fixed(a0, E), x1 = to_block_fixed(a1, E), x2 = to_block_fixed(a2, E),
-                  x3 = to_block_fixed(a3, E);
-  const long long Da = x1 - x0, Db = x2 - x1, Dc = x3 - x2;
-  const long long ra = __mul64hi(Da << 2, Hq), rb = __mul64hi(Db << 2, Hq), rc = __mul64hi(Dc << 2, Hq);
-  const long long s_ab = slope_int(Da, Db, ra, rb);  // slope of the cell between a and b faces
-  const long long s_bc = slope_int(Db, Dc, rb, rc);
-  // v > 0 (cells j-2..j+1): dF = D_j + sigma_j - sigma_{j-1} = Db + s_bc - s_ab
-  // v < 0 (cells j-1..j+2): dF = D_{j+1} - sigma_{j+1} + sigma_j = Db - s_bc + s_ab
-  const long long F = sgn > 0 ? Db + s_bc - s_ab : Db - s_bc + s_ab;
-  return from_block_fixed(F, E);
-}
-
-
-// Rational limiter: with beta = lp/lq the scaled slope 4 lq sigma equals
-// minmod3(2 lp Da, lq (Da + Db), 2 lp Db) exactly, so the flux difference
-// scaled by 4 lq needs only small-integer multiplies.  Values enter with a
-// 52-bit significand (X = value 2^(1074 - E)) to leave headroom for the
-// factors (lp <= 128, lq <= 64).
-__device__ __forceinline__ long long slope_rat(long long Da, long long Db, long long lp2, long long lq) {
-  const long long ra = lp2 * Da, rb = lp2 * Db, y = lq * (Da + Db);
-  const long long mn = min(min(ra, y), rb), mx = max(max(ra, y), rb);
-  return ((Da ^ Db) >= 0) ? (Da >= 0 ? mn : mx) : 0ll;
-}
-
 // 52-bit variant: value = X 2^(E - 1074); the magnitude is truncated (toward
 // zero) in one shift of the significand
 __device__ __forceinline__ long long to_block_fixed52(double v, int E) {
@@ -810,25 +752,9 @@ __device__ __forceinline__ long long to_block_fixed52(double v, int E) {
   return hi < 0 ? -(long long)mag : (long long)mag;
 }
 
-// 4 lq (F_{j+1/2} - F_{j-1/2}) as a double (the caller folds 1/(4 lq)) from
-// the stencil values a0..a3 (v > 0: cells j-2..j+1; v < 0: cells j-1..j+2)
-__device__ __forceinline__ double flux_difference_rat_v(double a0, double a1, double a2, double a3, int lp, int lq,
-                                                        int sgn) {
-  const int E = max(max(bexp(a0), bexp(a1)), max(bexp(a2), bexp(a3)));
-  const long long x0 = to_block_fixed52(a0, E), x1 = to_block_fixed52(a1, E), x2 = to_block_fixed52(a2, E),
-                  x3 = to_block_fixed52(a3, E);
-  const long long Da = x1 - x0, Db = x2 - x1, Dc = x3 - x2;
-  const long long lp2 = 2 * lp, q4 = 4 * lq;
-  const long long s_ab = slope_rat(Da, Db, lp2, lq);
-  const long long s_bc = slope_rat(Db, Dc, lp2, lq);
-  const long long F = sgn > 0 ? q4 * Db + s_bc - s_ab : q4 * Db - s_bc + s_ab;
-  if (E < 64) return 0.0;
-  return ll_to_double_scaled(F, E - 1074);  // value = F 2^(E - 1074)
-}
-
 // ---- advection of one population over a tile (FP64 storage) -----------------
 // The update's flux differences (Sec. III.A.2) of one population over a tile of
-// up to 32 x 8 cells, by one warp, in block fixed point: the tile's cells and
+// up to 32 x R cells, by one warp, in block fixed point: the tile's cells and
 // its upwind halo share one exponent, so every value is converted once (a
 // per-cell stencil converts eight values per cell), differences are exact, and
 // each limited slope is computed once and handed to the neighbour (along x by
@@ -841,9 +767,8 @@ __device__ __forceinline__ double flux_difference_rat_v(double a0, double a1, do
 // F_j + sigma_j, and the cell's change is -k ((F_j + sigma_j) - (F_{j-1} + sigma_{j-1})).
 // Everything is kept times 4 lq (beta = lp / lq: candidates 2 lp D and
 // lq (D + D')); a general beta takes lq = 1 and a fixed-point beta.
-constexpr int kTileY = 8;                 // CTA = 32 x kTileY cells
-constexpr int kCta = 32 * kTileY;
-constexpr int kAdvPitch = 36, kAdvRows = kTileY + 3;  // stream columns -2 .. 32, rows -2 .. 8
+constexpr int kCta = 256;                 // threads of a step kernel's CTA
+constexpr int kAdvPitch = 36;             // stream columns -2 .. 32 of a tile's row
 
 // x k + y for a small k >= 0: two multiply-adds (a sign-extended 64-bit k takes three)
 __device__ __forceinline__ long long mad_small(long long x, unsigned k, long long y) {
@@ -893,25 +818,27 @@ struct AdvTile {
   bool fx, fy;       // walked against x, against y
   int lane;
 };
-// What a warp reads of one population: its lane's column in stream rows -2 .. 8,
+// What a warp reads of one population: its lane's column in stream rows -2 .. R,
 // and one cell of the x-halo.  Read one population ahead, so that the loads'
 // latency passes during the walk over the previous one.
+template <int R>
 struct AdvLoad {
-  double v[kAdvRows], h;
+  double v[R + 3], h;
 };
 // plane: the population's plane at the tile's lowest cell.  Every lane and row
 // loads, in ragged tiles the last column and the row after the tile again, so
 // that the loads need no predicates.
-__device__ __forceinline__ void advect_load(AdvLoad& L, const double* __restrict__ plane, long long PT,
+template <int R>
+__device__ __forceinline__ void advect_load(AdvLoad<R>& L, const double* __restrict__ plane, long long PT,
                                             const AdvTile& T) {
   const int i = min(T.lane, T.W - 1);
   const unsigned lx = (unsigned)(T.fx ? T.W - 1 - i : i) * 8u;
   const long long sy = T.fy ? -PT : PT;
   const double* row0 = plane + (T.fy ? (T.H - 1) * PT : 0);  // stream row 0
 #pragma unroll
-  for (int j = -2; j <= kTileY; ++j) L.v[j + 2] = __ldg(at(row0 + min(j, T.H) * sy, lx));
-  const int hr = min(T.lane & 7, T.H - 1), hc = T.lane >> 3;  // halo cell: row hr, stream column -2, -1, W (or 0)
-  const int h = hc == 3 ? 0 : hc == 2 ? T.W : hc - 2;
+  for (int j = -2; j <= R; ++j) L.v[j + 2] = __ldg(at(row0 + min(j, T.H) * sy, lx));
+  const int hr = min(T.lane % R, T.H - 1), hc = T.lane / R;  // halo cell: row hr, stream column -2, -1, W (or 0)
+  const int h = hc > 2 ? 0 : hc == 2 ? T.W : hc - 2;
   L.h = __ldg(row0 + hr * sy + (T.fx ? T.W - 1 - h : h));
 }
 
@@ -919,21 +846,21 @@ __device__ __forceinline__ void advect_load(AdvLoad& L, const double* __restrict
 // sums go, kx (x-face difference) + ky (y-face difference) as integers W in
 // units of 2^(E - 1079), E the returned block exponent; MX, MY: the population
 // moves along x, along y; kx, ky: flux factors (Phys::kxq, kyq); xs: this warp's
-// [kAdvRows][kAdvPitch] words of shared memory; code: (CODES) this population's
+// [R + 3][kAdvPitch] words of shared memory; code: (CODES) this population's
 // branch codes at the tile's lowest cell, row pitch cpitch; next: starts the
 // next population's loads into L.
-template <bool MX, bool MY, bool RAT, bool CODES, class Next>
-__device__ __forceinline__ int advect_tile(AdvLoad& L, const Next& next, long long* out, long long PT, const AdvTile& T,
+template <int R, bool MX, bool MY, bool RAT, bool CODES, class Next>
+__device__ __forceinline__ int advect_tile(AdvLoad<R>& L, const Next& next, long long* out, long long PT, const AdvTile& T,
                                            const Phys& P, long long kx, long long ky, long long* xs,
                                            unsigned char* code, long long cpitch) {
   const int lane = T.lane;
   const bool in = lane < T.W;
   const unsigned lx = in ? (unsigned)(T.fx ? T.W - 1 - lane : lane) : 0u;  // this lane's column of the tile
   const long long sy = T.fy ? -PT : PT;
-  constexpr int J0 = MY ? -2 : 0, J1 = MY ? kTileY : kTileY - 1;  // rows this population needs
+  constexpr int J0 = MY ? -2 : 0, J1 = MY ? R : R - 1;  // rows this population needs
   const double* v = L.v + (J0 + 2);
   const double vh = L.h;
-  const int hr = lane & 7, hc = lane >> 3;
+  const int hr = lane % R, hc = lane / R;
   const bool hin = MX && hc < 3 && hr < T.H;
   // block exponent; non-finite values are left out (their key wraps to 0)
   unsigned key = 0;
@@ -1020,6 +947,332 @@ __device__ __forceinline__ double collide_advect(double a1, double F, long long 
   const double z = __ll2double_rn((t >> min(max(d, 0), 63)) - (w >> min(max(-d, 0), 63)));
   const int zh = __double2hiint(z);
   return fma(a1, F, __hiloint2double(zh == 0 ? 0 : zh + ((max(sw, st) - 1079) << 20), __double2loint(z)));
+}
+
+// node constants W_k He_n(xi_k)/n! 2^(61 + kd(k)) (below 2^61), rounded from their
+// exact values; nodes 0, +-sqrt(5 - sqrt 10), +-sqrt(5 + sqrt 10)
+constexpr long long kKF[3][5] = {
+    {1229782938247303441ll, 0ll, -614891469123651721ll, 0ll, 153722867280912930ll},
+    {1024144424542654913ll, 1388356993984702056ll, 428974331826690775ll, -268942719741157367ll, -198390030905321379ll},
+    {415325171389884787ll, 1186571560667484526ll, 1487337098375687568ll, 1020901976637480698ll, 357337308995267594ll}};
+__host__ __device__ constexpr long long kf(int k, int n) {
+  return sgn_of(k) < 0 && n % 2 == 1 ? -kKF[(k + 1) / 2][n] : kKF[(k + 1) / 2][n];
+}
+// as limbs, a constant-bank table for the node loop: [node][n] = {high, low}
+static __constant__ int c_kf[5][5][2] = {
+#define KF(k, n) {limb_hi(kf(k, n)), limb_lo(kf(k, n))}
+#define KROW(k) {KF(k, 0), KF(k, 1), KF(k, 2), KF(k, 3), KF(k, 4)}
+    KROW(0), KROW(1), KROW(2), KROW(3), KROW(4)};
+
+// This thread's collision coefficients in block fixed point (60 bits, one
+// exponent for f, one for g) as limb pairs in shared memory: field k of thread
+// t at [k * kCta + t] (consecutive threads, consecutive words; registers would
+// hold 42 words across the node loop).  Field order f00, f10, f01, f20, f11,
+// f02, f30, f21, f12, f03, f40, f31, f22, f13, f04, g00, g10, g01, g20, g11, g02.
+struct FixView {
+  const long long* b;
+  __device__ __forceinline__ void mac(LimbAcc& s, int field, const int (&k)[2]) const {
+    const long long x = b[field * kCta];
+    s.mac((int)(x >> 32), (int)x, k[0], k[1]);
+  }
+};
+template <int N>
+__device__ __forceinline__ void fields_to_smem(const double (&f)[N], long long* b, int& E) {
+  unsigned key = 0;
+#pragma unroll
+  for (int k = 0; k < N; ++k) key = max(key, abs_key(f[k]));
+  E = (int)(key >> 20);
+  const int n0 = E < 128 ? 63 : 0;  // negligible coefficients: target 0
+#pragma unroll
+  for (int k = 0; k < N; ++k) b[k * kCta] = pack_limbs(block_fix(f[k], E, n0));
+}
+__device__ __forceinline__ void coeffs_to_smem(const Coeffs& C, long long* b, int& Ef, int& Eg) {
+  const double f[15] = {C.f00, C.f10, C.f01, C.f20, C.f11, C.f02, C.f30, C.f21,
+                        C.f12, C.f03, C.f40, C.f31, C.f22, C.f13, C.f04};
+  const double g[6] = {C.g00, C.g10, C.g01, C.g20, C.g11, C.g02};
+  fields_to_smem<15>(f, b, Ef);
+  fields_to_smem<6>(g, b + 15 * kCta, Eg);
+}
+
+// h^b of x-node p: W_p sum_a C_ab He_a(xi_p)/a! (value h 2^(E - 1082 - kd(p)))
+__device__ __forceinline__ void hf_node(const FixView& X, const int (&K)[5][2], long long (&h)[5]) {
+  LimbAcc a, b, c, d, e;
+  X.mac(a, 0, K[0]); X.mac(a, 1, K[1]); X.mac(a, 3, K[2]); X.mac(a, 6, K[3]); X.mac(a, 10, K[4]);
+  X.mac(b, 2, K[0]); X.mac(b, 4, K[1]); X.mac(b, 7, K[2]); X.mac(b, 11, K[3]);
+  X.mac(c, 5, K[0]); X.mac(c, 8, K[1]); X.mac(c, 12, K[2]);
+  X.mac(d, 9, K[0]); X.mac(d, 13, K[1]);
+  X.mac(e, 14, K[0]);
+  h[0] = a.value8(); h[1] = b.value8(); h[2] = c.value8(); h[3] = d.value8(); h[4] = e.value8();
+}
+__device__ __forceinline__ void hg_node(const FixView& X, const int (&K)[5][2], long long (&h)[3]) {
+  LimbAcc a, b, c;
+  X.mac(a, 15, K[0]); X.mac(a, 16, K[1]); X.mac(a, 18, K[2]);
+  X.mac(b, 17, K[0]); X.mac(b, 19, K[1]);
+  X.mac(c, 20, K[0]);
+  h[0] = a.value8(); h[1] = b.value8(); h[2] = c.value8();
+}
+template <int k, int n>
+__device__ __forceinline__ void kmac(LimbAcc& s, const Limbs& x) {
+  s.mac(x.h, x.l, limb_hi(kf(k, n)), limb_lo(kf(k, n)));
+}
+// t_q = W_q sum_b h^b He_b(xi_q)/b! of the five y-nodes with the +-xi symmetry:
+// value t_q 2^(E - 1079 - kd(p) - kd(q))
+__device__ __forceinline__ void expand_node(const long long (&h)[5], long long (&t)[5]) {
+  const Limbs h0(h[0]), h1(h[1]), h2(h[2]), h3(h[3]), h4(h[4]);
+  LimbAcc c, ea, oa, eb, ob;
+  kmac<0, 0>(c, h0); kmac<0, 2>(c, h2); kmac<0, 4>(c, h4);
+  kmac<1, 0>(ea, h0); kmac<1, 2>(ea, h2); kmac<1, 4>(ea, h4);
+  kmac<1, 1>(oa, h1); kmac<1, 3>(oa, h3);
+  kmac<3, 0>(eb, h0); kmac<3, 2>(eb, h2); kmac<3, 4>(eb, h4);
+  kmac<3, 1>(ob, h1); kmac<3, 3>(ob, h3);
+  t[0] = c.value();
+  t[1] = ea.value() + oa.value(); t[2] = ea.value() - oa.value();
+  t[3] = eb.value() + ob.value(); t[4] = eb.value() - ob.value();
+}
+__device__ __forceinline__ void expand_node(const long long (&h)[3], long long (&t)[5]) {
+  const Limbs h0(h[0]), h1(h[1]), h2(h[2]);
+  LimbAcc c, ea, oa, eb, ob;
+  kmac<0, 0>(c, h0); kmac<0, 2>(c, h2);
+  kmac<1, 0>(ea, h0); kmac<1, 2>(ea, h2);
+  kmac<1, 1>(oa, h1);
+  kmac<3, 0>(eb, h0); kmac<3, 2>(eb, h2);
+  kmac<3, 1>(ob, h1);
+  t[0] = c.value();
+  t[1] = ea.value() + oa.value(); t[2] = ea.value() - oa.value();
+  t[3] = eb.value() + ob.value(); t[4] = eb.value() - ob.value();
+}
+__device__ __forceinline__ void load_kf(int p, int (&K)[5][2]) {
+#pragma unroll
+  for (int n = 0; n < 5; ++n) {
+    K[n][0] = c_kf[p][n][0];
+    K[n][1] = c_kf[p][n][1];
+  }
+}
+
+struct Lat25 {
+  static constexpr int NQ = 5, POPS = 50, FIELDS = 21;
+  typedef Moments Mom;
+  typedef int NodeK[5][2];
+  __device__ static __forceinline__ bool backward(int k) { return k != 0 && (k & 1) == 0; }
+  __device__ static __forceinline__ int kdp(int k) { return k == 0 ? 0 : (k <= 2 ? kd(1) : kd(3)); }
+  __device__ static __forceinline__ Mom moments(const double* s, unsigned off, long long PL) {
+    return moments_fix<double>(s, off, PL);
+  }
+  template <int PRC>
+  __device__ static __forceinline__ Coeffs coeffs(const Mom& m, const Phys& P) { return collision_coeffs<PRC>(m, P); }
+  __device__ static __forceinline__ void to_smem(const Coeffs& C, long long* b, int& Ef, int& Eg) {
+    coeffs_to_smem(C, b, Ef, Eg);
+  }
+  __device__ static __forceinline__ void load_k(int p, NodeK& K) { load_kf(p, K); }
+  __device__ static __forceinline__ void target_f(const FixView& X, const NodeK& K, long long (&t)[5]) {
+    long long h[5];
+    hf_node(X, K, h);
+    expand_node(h, t);
+  }
+  __device__ static __forceinline__ void target_g(const FixView& X, const NodeK& K, long long (&t)[5]) {
+    long long h[3];
+    hg_node(X, K, h);
+    expand_node(h, t);
+  }
+};
+
+// ---- the FP64 step over tiles --------------------------------------------------
+// Two phases per 32 x R tile, 256 threads.  Advection, one population per warp:
+// the warp walks the tile and writes the flux sums (advect_tile) as integers into
+// the new state's space, from where they come back out of L2.  Collision, one
+// cell per thread: moments, combined coefficients, the collision target of each
+// population in fixed point, and the update with the flux sum (collide_advect).
+// Low tiles (R < 8, small grids) also write the periodic and zero-gradient ghost
+// images of the cells next to the grid's edge, so that a step without walls is
+// one launch (64^2: 25 -> 21 us).  In the 8-row kernel the same code costs 6 %: its
+// divergent tail keeps the compiler off the uniform registers for addresses.
+//  * Advection: warp w does f (w < 4) or g.  D2Q25: x-node p = 1 + w % 4, its four
+//    populations that move along both axes, (p, 0) along x only and (0, p) along
+//    y only, so that all eight warps have the same work; the resting population
+//    needs none.  D2Q16: the four populations of x-node w % 4.
+//  * Collision with R < 8: a cell has 8 / R threads, which all form its
+//    coefficients and share the populations (in units of an x-node's f or g).
+struct GhostKinds {
+  int k[4];  // xlo, xhi, ylo, yhi: 0 periodic, 1 zero gradient, else not written here
+};
+// is the cell the source of a ghost image?
+__device__ __forceinline__ bool on_edge(int x, int y, const Geom& G, const GhostKinds& B) {
+  return ((x < 2 && B.k[0] < 2) || (x >= G.Nx - 2 && B.k[1] < 2) || (y < 2 && B.k[2] < 2) || (y >= G.Ny - 2 && B.k[3] < 2));
+}
+// copies N planes' values of cell (x, y) to the cell's ghost images; p: the cell in
+// the first of them
+template <int N, class S>
+__device__ __forceinline__ void write_images(S* p, long long PL, int x, int y, const Geom& G, const GhostKinds& B) {
+  S v[N];
+#pragma unroll
+  for (int q = 0; q < N; ++q) v[q] = p[q * PL];
+  auto put = [&](long long o) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) p[q * PL + o] = v[q];
+  };
+  const long long PT = G.pitch;
+  if (B.k[0] == 0) {
+    if (x < 2) put(G.Nx);
+    if (x >= G.Nx - 2) put(-G.Nx);
+  }
+  if (B.k[0] == 1 && x == 0) put(-1), put(-2);
+  if (B.k[1] == 1 && x == G.Nx - 1) put(1), put(2);
+  if (B.k[2] == 0) {
+    if (y < 2) put(G.Ny * PT);
+    if (y >= G.Ny - 2) put(-G.Ny * PT);
+  }
+  if (B.k[2] == 1 && y == 0) put(-PT), put(-2 * PT);
+  if (B.k[3] == 1 && y == G.Ny - 1) put(PT), put(2 * PT);
+}
+
+// What bounds it: the integer ALU (about two thirds busy) beside the FP64 pipe
+// (about half) and the latency between them; DRAM is at a fifth of its rate.
+// D2Q25: 12.4 k instructions and 186 FP64 ones a cell, against 26.8 k and 407 of a
+// thread per cell with its own stencils: 15.5 -> 8.4 ms a step at 4096^2, 1.02 ->
+// 0.54 ms at 1024^2.  D2Q16: 10.5 -> 6.0 ms and 0.70 -> 0.39 ms.  Three CTAs of 80
+// registers; four of 64 measured 1 % slower.
+// L: the lattice (Lat25, Lat16).  PRC: Prandtl branch; RAT: rational limiter;
+// CODES: also the branch codes of every population's slopes (one byte x | y << 2
+// at codes[pop][y][x]) and, unless moms is null, the cells' moments.
+template <class L, int R, int PRC, bool RAT, bool CODES>
+__global__ void __launch_bounds__(kCta, 3) k_step_tile(const double* __restrict__ src, double* dst, Geom G, Phys P,
+                                                       GhostKinds B, unsigned int* __restrict__ flag,
+                                                       unsigned char* codes, double* __restrict__ moms) {
+  __shared__ long long s_buf[L::FIELDS * kCta];  // the advection's tiles, then the collision coefficients
+  __shared__ int s_exp[L::POPS];                 // block exponents of the flux sums
+  static_assert(8 * (R + 3) * kAdvPitch <= L::FIELDS * kCta, "the advection tiles fit the coefficients' space");
+  constexpr int NQ = L::NQ, NF = NQ * NQ;
+  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * R;
+  const long long PL = G.plane;
+  const long long PT = G.pitch;
+  const long long cplane = (long long)G.Nx * G.Ny;
+  const double* stile = src + cell_index(G, y0, x0);
+  double* dtile = dst + cell_index(G, y0, x0);
+  {
+    const int w = __shfl_sync(0xffffffffu, (int)threadIdx.y, 0), c0 = NF * (w >> 2);
+    AdvTile T;
+    T.W = min(32, G.Nx - x0);
+    T.H = min(R, G.Ny - y0);
+    T.lane = threadIdx.x;
+    long long* xs = s_buf + w * ((R + 3) * kAdvPitch);
+    unsigned char* ctile = CODES ? codes + (long long)y0 * G.Nx + x0 : nullptr;
+    int E;
+    AdvLoad<R> V;
+    // the walk directions of population (p, q): sign of each velocity component
+    auto tile = [&](int p, int q) {
+      AdvTile t = T;
+      t.fx = L::backward(p);
+      t.fy = L::backward(q);
+      return t;
+    };
+    auto load = [&](int p, int q) { advect_load<R>(V, stile + (c0 + NQ * p + q) * PL, PT, tile(p, q)); };
+    auto out = [&](int c) { return (long long*)(dtile + c * PL); };
+    auto code = [&](int c) { return CODES ? ctile + c * cplane : nullptr; };
+    if constexpr (NQ == 5) {
+      const int p = 1 + (w & 3);
+      load(p, 0);
+      {
+        const int c = c0 + 5 * p;
+        E = advect_tile<R, true, false, RAT, CODES>(V, [&] { load(p, 1); }, out(c), PT, tile(p, 0), P, P.kxq[p], 0, xs,
+                                                    code(c), G.Nx);
+        if (T.lane == 0) s_exp[c] = E;
+      }
+#pragma unroll 1
+      for (int q = 1; q < 5; ++q) {
+        const int c = c0 + 5 * p + q;
+        E = advect_tile<R, true, true, RAT, CODES>(V, [&] { load(q < 4 ? p : 0, q < 4 ? q + 1 : p); }, out(c), PT,
+                                                   tile(p, q), P, P.kxq[p], P.kyq[q], xs, code(c), G.Nx);
+        if (T.lane == 0) s_exp[c] = E;
+      }
+      {
+        const int c = c0 + p;
+        E = advect_tile<R, false, true, RAT, CODES>(V, [] {}, out(c), PT, tile(0, p), P, 0, P.kyq[p], xs, code(c), G.Nx);
+        if (T.lane == 0) s_exp[c] = E;
+      }
+      if (p == 1) {  // the resting population: no flux, and no slopes the adjoint uses
+        if (T.lane == 0) s_exp[c0] = 0;
+        if (T.lane < T.W)
+          for (int j = 0; j < T.H; ++j) {
+            ((long long*)dtile)[c0 * PL + j * PT + T.lane] = 0;
+            if (CODES) ctile[c0 * cplane + (long long)j * G.Nx + T.lane] = 0;
+          }
+      }
+    } else {
+      const int p = w & 3;
+      load(p, 0);
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {
+        const int c = c0 + 4 * p + q;
+        E = advect_tile<R, true, true, RAT, CODES>(V, [&] { load(p, min(q + 1, 3)); }, out(c), PT, tile(p, q), P, P.kxq[p],
+                                                   P.kyq[q], xs, code(c), G.Nx);
+        if (T.lane == 0) s_exp[c] = E;
+      }
+    }
+  }
+  __syncthreads();
+  constexpr int NG = 8 / R;  // threads of a cell
+  const int row = threadIdx.y % R, group = threadIdx.y / R;
+  const int x = x0 + threadIdx.x, y = y0 + row;
+  if (x >= G.Nx || y >= G.Ny) return;
+  const unsigned off = (row * (unsigned)PT + threadIdx.x) * 8u;  // this cell's byte offset in the tile
+  const typename L::Mom m = L::moments(stile, off, PL);
+  if constexpr (CODES) {
+    // the recomputing adjoint also keeps the cell's moments (13 planes of
+    // Nx * Ny doubles, Moments field order) for its collision part
+    if (moms && group == 0) {
+      const long long ci = (long long)y * G.Nx + x;
+      const double v[13] = {m.m00, m.m10, m.m01, m.m20, m.m11, m.m02, m.m30,
+                            m.m21, m.m12, m.m03, m.g00, m.g10, m.g01};
+#pragma unroll
+      for (int k = 0; k < 13; ++k) moms[k * cplane + ci] = v[k];
+    }
+  }
+  int Ef, Eg;
+  double a1;
+  const int tid = threadIdx.y * 32 + threadIdx.x;
+  const FixView X{s_buf + tid};
+  {
+    const auto C = L::template coeffs<PRC>(m, P);
+    if (C.bad) atomicOr(flag, 1u);
+    L::to_smem(C, s_buf + tid, Ef, Eg);
+    a1 = C.a1;
+  }
+#pragma unroll 1
+  for (int p0 = 0; p0 < NQ; p0 += NG > 2 ? NG / 2 : 1) {
+    // NG = 1: an x-node's f and g in turn; NG = 2: one of them; NG = 4: of every second x-node
+    const int p = NG > 2 ? p0 + (group >> 1) : p0;
+    if (NG > 2 && p >= NQ) break;
+    typename L::NodeK K;
+    L::load_k(p, K);
+    const int dp = L::kdp(p);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      if (NG > 1 && k != (group & 1)) continue;
+      const double* sp = stile + (NF * k + NQ * p) * PL;
+      double* dp_ = dtile + (NF * k + NQ * p) * PL;
+      double F[NQ];
+      long long W[NQ], t[NQ];
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        F[q] = __ldg(at(sp + q * PL, off));
+        W[q] = *at((const long long*)dp_ + q * PL, off);
+      }
+      if (k == 0) L::target_f(X, K, t);
+      else L::target_g(X, K, t);
+      const int st = (k == 0 ? Ef : Eg) - dp;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        *at(dp_ + q * PL, off) = collide_advect(a1, F[q], t[q], st - L::kdp(q), W[q], s_exp[NF * k + NQ * p + q]);
+      }
+    }
+  }
+  if constexpr (R < 8) {
+    if (on_edge(x, y, G, B)) {
+      // of the units this thread has written
+      for (int p = NG > 2 ? group >> 1 : 0; p < NQ; p += NG > 2 ? NG / 2 : 1)
+        write_images<NQ>(at(dtile + (NF * (group & 1) + NQ * p) * PL, off), PL, x, y, G, B);
+    }
+  }
 }
 
 // Flux difference F_{j+1/2} - F_{j-1/2} of the upwind-limited face values

@@ -15,14 +15,32 @@ struct Macro {          // constants needed to turn moments into physical fields
   double c, T_ref, R, gamma;
 };
 
-cudaError_t launch_step(int storage, const void* src, void* dst, const Geom& G, const Phys& P,
+// ghost layers the step kernels write themselves: periodic and zero-gradient sides
+inline GhostKinds ghost_kinds(const BCDev& bc) {
+  GhostKinds B;
+  for (int s = 0; s < 4; ++s) B.k[s] = bc.kind[s];
+  return B;
+}
+// Tile height of the FP64 step.  8 rows share their halo best (2.2 times the rate of
+// 2 rows on a full chip); while the grid's tiles are fewer than the SMs, lower
+// tiles shorten the step by spreading it over more of them, as long as each
+// SM gets no more than one.  Measured, D2Q25, us a step with 8 / 4 / 2 rows: 64^2
+// 41 / 29 / 23, 128^2 41 / 31 / 33, 192^2 42 / 41 / 54, 256^2 60 / 69 / 84.
+inline int tile_rows(const Geom& G) {
+  const long long tiles = (long long)((G.Nx + 31) / 32) * ((G.Ny + 7) / 8);
+  return 4 * tiles <= 152 ? 2 : 2 * tiles <= 152 ? 4 : 8;
+}
+// Does the step kernel write the ghost layers of periodic and zero-gradient sides?
+// Then only wall sides are left for launch_ghost, else all.
+inline bool step_writes_images(int storage, const Geom& G) { return storage == 0 && tile_rows(G) < 8; }
+cudaError_t launch_step(int storage, const void* src, void* dst, const Geom& G, const Phys& P, const BCDev& bc,
                         unsigned int* flag, cudaStream_t st);
 // FP64 step with the rational limiter that also records the minmod branch
 // codes of every population's x and y slopes: codes[pop][y][x] = x | y << 2
 // moms (nullable): also store the 13 moments of each cell of the input state,
 // moms[k][y][x] in Moments field order
-cudaError_t launch_step_codes(const void* src, void* dst, const Geom& G, const Phys& P, unsigned int* flag,
-                              unsigned char* codes, double* moms, cudaStream_t st);
+cudaError_t launch_step_codes(const void* src, void* dst, const Geom& G, const Phys& P, const BCDev& bc,
+                              unsigned int* flag, unsigned char* codes, double* moms, cudaStream_t st);
 // auxiliary kernels, written once for both models: lattice 0 = D2Q25 / split II
 // (storage 0 FP64, 1 FP32-deviation), lattice 1 = D2Q16 / split I (FP64)
 cudaError_t launch_init(int lattice, int storage, void* dst, const double* rho, const double* ux, const double* uy,
@@ -47,7 +65,7 @@ cudaError_t launch_pack(int storage, const void* buf, void* packed, int to_packe
                         cudaStream_t st);
 
 // D2Q16, total-energy split (I), FP64 storage
-cudaError_t launch_step16(const void* src, void* dst, const Geom& G, const Phys& P, unsigned int* flag,
+cudaError_t launch_step16(const void* src, void* dst, const Geom& G, const Phys& P, const BCDev& bc, unsigned int* flag,
                           cudaStream_t st);
 
 // adjoint (FP64 storage, periodic)

@@ -277,4 +277,138 @@ __device__ __forceinline__ void write_equilibrium_fix16(double* d, long long PL,
 }
 }  // namespace q16
 
+// ---- the step over tiles (k_step_tile) -----------------------------------------
+namespace q16 {
+
+// node constants W_k He_n(xi_k)/n! 2^(61 + kdq(k)), rounded from their exact values
+constexpr long long kKQ[2][4] = {
+    {1047138985598193535ll, 776939204445353226ll, -235339116647385024ll, -317184102009169216ll},
+    {423130076034613764ll, 987760865702054896ll, 941356466589540094ll, 403251684809969295ll}};
+__host__ __device__ constexpr long long kqf(int k, int n) {
+  return sgn(k) < 0 && n % 2 == 1 ? -kKQ[k / 2][n] : kKQ[k / 2][n];
+}
+static __constant__ int c_kqf[4][4][2] = {
+#define KQ(k, n) {limb_hi(kqf(k, n)), limb_lo(kqf(k, n))}
+#define KQROW(k) {KQ(k, 0), KQ(k, 1), KQ(k, 2), KQ(k, 3)}
+    KQROW(0), KQROW(1), KQROW(2), KQROW(3)};
+#undef KQROW
+#undef KQ
+
+// YA^n and YB^n times 2^62 / 4, / 8 (n = 1, 2): pair sums / 16, / 32
+constexpr long long kYA[3] = {0, 855426002562088766ll, 317347557025960323ll};
+constexpr long long kYB[3] = {0, 2691396352982990230ll, 3141416956794580605ll};
+template <int n>
+__device__ __forceinline__ long long pair_sum16(long long b, long long a) {
+  const Limbs x(b), y(a);
+  LimbAcc s;
+  s.mac(x.h, x.l, limb_hi(kYB[n]), limb_lo(kYB[n]));
+  s.mac(y.h, y.l, limb_hi(kYA[n]), limb_lo(kYA[n]));
+  return s.value();
+}
+
+// moments in block fixed point, as moments_fix for D2Q25
+__device__ __forceinline__ Mom moments_fix16(const double* __restrict__ s, unsigned off, long long PL) {
+  Mom m;
+  bool finite = true;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    double v[16];
+    unsigned key = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      v[i] = __ldg(at(s + (16 * k + i) * PL, off));
+      key = max(key, abs_key(v[i]));
+    }
+    finite = finite && key < 0x7ff00000u;
+    const int E = (int)(key >> 20);
+    const int n0 = E < 128 ? 63 : 2;
+    const int sc = E - 1080;
+    long long M0[4], M1[4], M2s = 0;  // y-sums of each x-node, M1 and M2 times 1/16, 1/32
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const long long x0 = block_fix(v[4 * p], E, n0), x1 = block_fix(v[4 * p + 1], E, n0),
+                      x2 = block_fix(v[4 * p + 2], E, n0), x3 = block_fix(v[4 * p + 3], E, n0);
+      const long long sA = x0 + x1, dA = x0 - x1, sB = x2 + x3, dB = x2 - x3;
+      M0[p] = sA + sB;
+      M1[p] = pair_sum16<1>(dB, dA);
+      if (k == 0) M2s += pair_sum16<2>(sB, sA);
+    }
+    const long long a0 = M0[0] + M0[1], b0 = M0[2] + M0[3], c0 = M0[0] - M0[1], d0 = M0[2] - M0[3];
+    const double s00 = fix_to_double<true>(a0 + b0, sc);
+    const double s10 = fix_to_double<true>(pair_sum16<1>(d0, c0), sc + 4);
+    const double s01 = fix_to_double<true>((M1[0] + M1[1]) + (M1[2] + M1[3]), sc + 4);
+    if (k == 0) {
+      m.m00 = s00; m.m10 = s10; m.m01 = s01;
+      m.m20 = fix_to_double<true>(pair_sum16<2>(b0, a0), sc + 5);
+      m.m02 = fix_to_double<true>(M2s, sc + 5);
+      m.m11 = fix_to_double<true>(pair_sum16<1>((M1[2] - M1[3]) << 4, (M1[0] - M1[1]) << 4), sc + 4);
+    } else {
+      m.g00 = s00; m.g10 = s10; m.g01 = s01;
+    }
+  }
+  if (!finite) m.m00 = __longlong_as_double(0x7ff8000000000000ll);
+  return m;
+}
+template <int k, int n>
+__device__ __forceinline__ void kqmac(LimbAcc& s, const Limbs& x) {
+  s.mac(x.h, x.l, limb_hi(kqf(k, n)), limb_lo(kqf(k, n)));
+}
+}  // namespace q16
+
+struct Lat16 {
+  static constexpr int NQ = 4, POPS = 32, FIELDS = 16;
+  typedef q16::Mom Mom;
+  typedef int NodeK[4][2];
+  __device__ static __forceinline__ bool backward(int k) { return (k & 1) != 0; }
+  __device__ static __forceinline__ int kdp(int k) { return k < 2 ? 0 : 2; }
+  __device__ static __forceinline__ Mom moments(const double* s, unsigned off, long long PL) {
+    return q16::moments_fix16(s, off, PL);
+  }
+  template <int PRC>
+  __device__ static __forceinline__ q16::Co coeffs(const Mom& m, const Phys& P) { return q16::coeffs<PRC>(m, P); }
+  // fields f00, f10, f01, f20, f11, f02, f30, f21, f12, f03, g00, g10, g01, g20, g11, g02
+  __device__ static __forceinline__ void to_smem(const q16::Co& C, long long* b, int& Ef, int& Eg) {
+    const double f[10] = {C.f00, C.f10, C.f01, C.f20, C.f11, C.f02, C.f30, C.f21, C.f12, C.f03};
+    const double g[6] = {C.g00, C.g10, C.g01, C.g20, C.g11, C.g02};
+    fields_to_smem<10>(f, b, Ef);
+    fields_to_smem<6>(g, b + 10 * kCta, Eg);
+  }
+  __device__ static __forceinline__ void load_k(int p, NodeK& K) {
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      K[n][0] = q16::c_kqf[p][n][0];
+      K[n][1] = q16::c_kqf[p][n][1];
+    }
+  }
+  __device__ static __forceinline__ void target_f(const FixView& X, const NodeK& K, long long (&t)[4]) {
+    LimbAcc a, b, c, d;
+    X.mac(a, 0, K[0]); X.mac(a, 1, K[1]); X.mac(a, 3, K[2]); X.mac(a, 6, K[3]);
+    X.mac(b, 2, K[0]); X.mac(b, 4, K[1]); X.mac(b, 7, K[2]);
+    X.mac(c, 5, K[0]); X.mac(c, 8, K[1]);
+    X.mac(d, 9, K[0]);
+    const Limbs h0(a.value8()), h1(b.value8()), h2(c.value8()), h3(d.value8());
+    LimbAcc ea, oa, eb, ob;
+    q16::kqmac<0, 0>(ea, h0); q16::kqmac<0, 2>(ea, h2);
+    q16::kqmac<0, 1>(oa, h1); q16::kqmac<0, 3>(oa, h3);
+    q16::kqmac<2, 0>(eb, h0); q16::kqmac<2, 2>(eb, h2);
+    q16::kqmac<2, 1>(ob, h1); q16::kqmac<2, 3>(ob, h3);
+    t[0] = ea.value() + oa.value(); t[1] = ea.value() - oa.value();
+    t[2] = eb.value() + ob.value(); t[3] = eb.value() - ob.value();
+  }
+  __device__ static __forceinline__ void target_g(const FixView& X, const NodeK& K, long long (&t)[4]) {
+    LimbAcc a, b, c;
+    X.mac(a, 10, K[0]); X.mac(a, 11, K[1]); X.mac(a, 13, K[2]);
+    X.mac(b, 12, K[0]); X.mac(b, 14, K[1]);
+    X.mac(c, 15, K[0]);
+    const Limbs h0(a.value8()), h1(b.value8()), h2(c.value8());
+    LimbAcc ea, oa, eb, ob;
+    q16::kqmac<0, 0>(ea, h0); q16::kqmac<0, 2>(ea, h2);
+    q16::kqmac<0, 1>(oa, h1);
+    q16::kqmac<2, 0>(eb, h0); q16::kqmac<2, 2>(eb, h2);
+    q16::kqmac<2, 1>(ob, h1);
+    t[0] = ea.value() + oa.value(); t[1] = ea.value() - oa.value();
+    t[2] = eb.value() + ob.value(); t[3] = eb.value() - ob.value();
+  }
+};
+
 }  // namespace dvbm
