@@ -387,10 +387,6 @@ __device__ __forceinline__ double ll_to_double_scaled(long long F, int scale) {
 // when it goes back to double, so the collision target carries no
 // systematic bias into the conserved sums.
 __host__ __device__ constexpr int kd(int k) { return k == 0 ? 0 : (k <= 2 ? 1 : 4); }
-__host__ __device__ constexpr long long khfix(int k, int n) {
-  return (long long)(kh(k, n) * 9223372036854775808.0 * (double)(1 << kd(k)));  // exact power-of-two scaling
-}
-
 // int64 -> double rounded to nearest (ties away from zero), value F 2^scale
 __device__ __forceinline__ double ll_to_double_rn(long long F, int scale) {
   if (F == 0) return 0.0;
@@ -502,8 +498,8 @@ __device__ __forceinline__ double fix_to_double(long long F, int scale) {
 // sum); sums are exact, and the powers of the abscissae are fixed-point factors
 // rounded from their exact values to 2^-62 (factors rounded to double leave a
 // drift of a few 1e-17 a step between the moments and the equilibria built from
-// them).  A non-finite population makes the zeroth moment NaN, which the
-// caller's checks see.
+// them).  A non-finite population makes its family's zeroth moment NaN, which
+// the caller's checks see.
 // XA^n and XB^n times 2^62 / 4, / 16, / 32 (n = 1, 2, 3)
 constexpr long long kXA[4] = {0, 1562930575100362931ll, 529687401272071863ll, 359029054183477437ll};
 constexpr long long kXB[4] = {0, 3293862167010879573ll, 2352616360245045577ll, 3360677197683338703ll};
@@ -524,7 +520,7 @@ __device__ __forceinline__ Moments moments_fix(const S* __restrict__ s, unsigned
   constexpr unsigned kInf = sizeof(S) == 8 ? 0x7ff00000u : 0x7f800000u;
   constexpr int kTiny = sizeof(S) == 8 ? 128 : 0;  // blocks below this exponent count as zero
   Moments m;
-  bool finite = true;
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
   {
     S v[25];
     unsigned key = 0;
@@ -533,7 +529,6 @@ __device__ __forceinline__ Moments moments_fix(const S* __restrict__ s, unsigned
       v[i] = __ldg(at(s + i * PL, off));
       key = max(key, abs_key(v[i]));
     }
-    finite = key < kInf;
     const int E = (int)(key >> kExpBits);
     const int n0 = E < kTiny ? 63 : 2;
     long long M0[5], M1[5], M2[5], M3s = 0;  // y-sums of each x-node, M1, M2, M3 times 1/16, 1/64, 1/128
@@ -563,6 +558,7 @@ __device__ __forceinline__ Moments moments_fix(const S* __restrict__ s, unsigned
     m.m11 = fix_to_double<true>(pair_sum<1>(d1 << 4, c1 << 4), sc + 4);
     m.m21 = fix_to_double<true>(pair_sum<2>(b1 << 4, a1 << 4), sc + 6);
     m.m12 = fix_to_double<true>(pair_sum<1>(d2 << 4, c2 << 4), sc + 6);
+    if (key >= kInf) m.m00 = nan;
   }
   {
     S v[25];
@@ -572,7 +568,6 @@ __device__ __forceinline__ Moments moments_fix(const S* __restrict__ s, unsigned
       v[i] = __ldg(at(s + (25 + i) * PL, off));
       key = max(key, abs_key(v[i]));
     }
-    finite = finite && key < kInf;
     const int E = (int)(key >> kExpBits);
     const int n0 = E < kTiny ? 63 : 2;
     long long N0[5], N1s = 0;
@@ -588,97 +583,18 @@ __device__ __forceinline__ Moments moments_fix(const S* __restrict__ s, unsigned
     m.g00 = fix_to_double<true>(N0[0] + (N0[1] + N0[2]) + (N0[3] + N0[4]), sc);
     m.g01 = fix_to_double<true>(N1s, sc + 4);
     m.g10 = fix_to_double<true>(pair_sum<1>(N0[3] - N0[4], N0[1] - N0[2]), sc + 4);
+    if (key >= kInf) m.g00 = nan;
   }
-  if (!finite) m.m00 = __longlong_as_double(0x7ff8000000000000ll);
   return m;
 }
-
-struct CoeffsFix {
-  long long f00, f10, f01, f20, f11, f02, f30, f21, f12, f03, f40, f31, f22, f13, f04;
-  long long g00, g10, g01, g20, g11, g02;
-  int Ef, Eg;  // block exponents: value = X 2^(E - 1082)
-};
-
-__device__ __forceinline__ CoeffsFix coeffs_to_fix(const Coeffs& C) {
-  CoeffsFix X;
-  const int Ef = max(max(max(max(bexp(C.f00), bexp(C.f10)), max(bexp(C.f01), bexp(C.f20))),
-                         max(max(bexp(C.f11), bexp(C.f02)), max(bexp(C.f30), bexp(C.f21)))),
-                     max(max(max(bexp(C.f12), bexp(C.f03)), max(bexp(C.f40), bexp(C.f31))),
-                         max(max(bexp(C.f22), bexp(C.f13)), bexp(C.f04))));
-  const int Eg = max(max(max(bexp(C.g00), bexp(C.g10)), max(bexp(C.g01), bexp(C.g20))),
-                     max(bexp(C.g11), bexp(C.g02)));
-  X.f00 = to_block_fixed(C.f00, Ef); X.f10 = to_block_fixed(C.f10, Ef); X.f01 = to_block_fixed(C.f01, Ef);
-  X.f20 = to_block_fixed(C.f20, Ef); X.f11 = to_block_fixed(C.f11, Ef); X.f02 = to_block_fixed(C.f02, Ef);
-  X.f30 = to_block_fixed(C.f30, Ef); X.f21 = to_block_fixed(C.f21, Ef); X.f12 = to_block_fixed(C.f12, Ef);
-  X.f03 = to_block_fixed(C.f03, Ef); X.f40 = to_block_fixed(C.f40, Ef); X.f31 = to_block_fixed(C.f31, Ef);
-  X.f22 = to_block_fixed(C.f22, Ef); X.f13 = to_block_fixed(C.f13, Ef); X.f04 = to_block_fixed(C.f04, Ef);
-  X.g00 = to_block_fixed(C.g00, Eg); X.g10 = to_block_fixed(C.g10, Eg); X.g01 = to_block_fixed(C.g01, Eg);
-  X.g20 = to_block_fixed(C.g20, Eg); X.g11 = to_block_fixed(C.g11, Eg); X.g02 = to_block_fixed(C.g02, Eg);
-  X.Ef = Ef;
-  X.Eg = Eg;
-  return X;
+// moments of the FP32-deviation reference populations w rho0 (f) and w G0 (g):
+// sum w = 1, sum w xi^2 = 1 per axis, odd moments vanish
+__device__ __forceinline__ void add_reference(Moments& m, const Phys& P) {
+  m.m00 += P.fref0; m.m20 += P.fref0; m.m02 += P.fref0;
+  m.g00 += P.gref0;
 }
 
 __device__ __forceinline__ long long mhk(long long x, long long k) { return __mul64hi(x, k); }
-
-// shift the N values so that the largest magnitude has its top bit at 2^60;
-// returns the shift (value of h after the call = h 2^(-sh) of its old scale)
-template <int N>
-__device__ __forceinline__ int renorm_fix(long long (&h)[N]) {
-  unsigned long long m = 0;
-#pragma unroll
-  for (int i = 0; i < N; ++i) m |= (unsigned long long)(h[i] < 0 ? -h[i] : h[i]);
-  const int sh = m == 0ull ? 0 : __clzll((long long)m) - 3;
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-    h[i] = sh >= 0 ? (long long)((unsigned long long)h[i] << sh) : (h[i] >> (-sh));
-  return sh;
-}
-
-// y-expansion of one x-node in fixed point, with the +-xi symmetry as in
-// expand_q5 / expand_q3 (value of t_q = t_q 2^(E - 1080 - kd(p) - sh - kd(q)))
-__device__ __forceinline__ void expand_q5_fix(const long long (&h)[5], long long (&t)[5]) {
-  t[0] = mhk(h[0], khfix(0, 0)) + mhk(h[2], khfix(0, 2)) + mhk(h[4], khfix(0, 4));
-  const long long EA = mhk(h[0], khfix(1, 0)) + mhk(h[2], khfix(1, 2)) + mhk(h[4], khfix(1, 4));
-  const long long OA = mhk(h[1], khfix(1, 1)) + mhk(h[3], khfix(1, 3));
-  const long long EB = mhk(h[0], khfix(3, 0)) + mhk(h[2], khfix(3, 2)) + mhk(h[4], khfix(3, 4));
-  const long long OB = mhk(h[1], khfix(3, 1)) + mhk(h[3], khfix(3, 3));
-  t[1] = EA + OA; t[2] = EA - OA; t[3] = EB + OB; t[4] = EB - OB;
-}
-__device__ __forceinline__ void expand_q3_fix(const long long (&h)[3], long long (&t)[5]) {
-  t[0] = mhk(h[0], khfix(0, 0)) + mhk(h[2], khfix(0, 2));
-  const long long EA = mhk(h[0], khfix(1, 0)) + mhk(h[2], khfix(1, 2));
-  const long long OA = mhk(h[1], khfix(1, 1));
-  const long long EB = mhk(h[0], khfix(3, 0)) + mhk(h[2], khfix(3, 2));
-  const long long OB = mhk(h[1], khfix(3, 1));
-  t[1] = EA + OA; t[2] = EA - OA; t[3] = EB + OB; t[4] = EB - OB;
-}
-
-// h^b of x-node p (f: N = 4, g: N = 2) from fixed-point coefficients X, any
-// view with X(k) = field k in CoeffsFix order (f00, f10, f01, f20, f11, f02,
-// f30, f21, f12, f03, f40, f31, f22, f13, f04, g00, g10, g01, g20, g11, g02);
-// k0..k4 = khfix(p, 0..4) (value of h = h 2^(E - 1081 - kd(p)))
-template <class V>
-__device__ __forceinline__ void hf_fix(const V& X, long long k0, long long k1, long long k2, long long k3,
-                                       long long k4, long long (&hf)[5]) {
-  hf[0] = mhk(X(0), k0) + mhk(X(1), k1) + mhk(X(3), k2) + mhk(X(6), k3) + mhk(X(10), k4);
-  hf[1] = mhk(X(2), k0) + mhk(X(4), k1) + mhk(X(7), k2) + mhk(X(11), k3);
-  hf[2] = mhk(X(5), k0) + mhk(X(8), k1) + mhk(X(12), k2);
-  hf[3] = mhk(X(9), k0) + mhk(X(13), k1);
-  hf[4] = mhk(X(14), k0);
-}
-template <class V>
-__device__ __forceinline__ void hg_fix(const V& X, long long k0, long long k1, long long k2, long long (&hg)[3]) {
-  hg[0] = mhk(X(15), k0) + mhk(X(16), k1) + mhk(X(18), k2);
-  hg[1] = mhk(X(17), k0) + mhk(X(19), k1);
-  hg[2] = mhk(X(20), k0);
-}
-template <class V>
-__device__ __forceinline__ void hfg_fix(const V& X, long long k0, long long k1, long long k2, long long k3,
-                                        long long k4, long long (&hf)[5], long long (&hg)[3]) {
-  hf_fix(X, k0, k1, k2, k3, k4, hf);
-  hg_fix(X, k0, k1, k2, hg);
-}
 
 // int64 -> float rounded to nearest (ties away from zero), value F 2^scale;
 // results below the normal float range flush to zero
@@ -693,52 +609,6 @@ __device__ __forceinline__ float ll_to_float_rn(long long F, int scale) {
   const int ex = 127 + 63 - lz + scale + carry;
   if (ex <= 0) return 0.0f;
   return __uint_as_float((unsigned)min(ex, 255) << 23 | (ex >= 255 ? 0u : frac) | (F < 0 ? 0x80000000u : 0u));
-}
-
-// Populations of coefficient set C (a pure equilibrium: a1 = 0, k1 = 1) at one
-// padded offset, by the step kernel's fixed-point expansion instead of FP64
-// arithmetic: initial conditions (Sec. III.A.3) at FP64-or-better precision.
-// FP32-deviation storage: the reference populations w rho0 and w G0 carry
-// only a zeroth Hermite coefficient, so they are taken off C first and the
-// deviations come straight out of the expansion.
-struct RegView {
-  const long long* v;
-  __device__ __forceinline__ long long operator()(int k) const { return v[k]; }
-};
-template <class S, int p>
-__device__ __forceinline__ void write_node_fix(S* d, long long PL, const RegView& X, int Ef, int Eg) {
-  long long hf[5], hg[3], xf[5], xg[5];
-  hfg_fix(X, khfix(p, 0), khfix(p, 1), khfix(p, 2), khfix(p, 3), khfix(p, 4), hf, hg);
-  const int sf = renorm_fix(hf), sg = renorm_fix(hg);
-  expand_q5_fix(hf, xf);
-  expand_q3_fix(hg, xg);
-  const int scf = Ef - 1080 - sf - kd(p), scg = Eg - 1080 - sg - kd(p);
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    if constexpr (sizeof(S) == 8) {
-      d[(5 * p + q) * PL] = Ef >= 100 ? ll_to_double_rn(xf[q], scf - kd(q)) : 0.0;
-      d[(25 + 5 * p + q) * PL] = Eg >= 100 ? ll_to_double_rn(xg[q], scg - kd(q)) : 0.0;
-    } else {
-      d[(5 * p + q) * PL] = Ef >= 100 ? ll_to_float_rn(xf[q], scf - kd(q)) : 0.0f;
-      d[(25 + 5 * p + q) * PL] = Eg >= 100 ? ll_to_float_rn(xg[q], scg - kd(q)) : 0.0f;
-    }
-  }
-}
-template <class S>
-__device__ __forceinline__ void write_equilibrium_fix(S* d, long long PL, Coeffs C, const Phys& P) {
-  if constexpr (sizeof(S) == 4) {
-    C.f00 -= P.fref0;
-    C.g00 -= P.gref0;
-  }
-  const CoeffsFix F = coeffs_to_fix(C);
-  const long long v[21] = {F.f00, F.f10, F.f01, F.f20, F.f11, F.f02, F.f30, F.f21, F.f12, F.f03, F.f40,
-                           F.f31, F.f22, F.f13, F.f04, F.g00, F.g10, F.g01, F.g20, F.g11, F.g02};
-  const RegView X{v};
-  write_node_fix<S, 0>(d, PL, X, F.Ef, F.Eg);
-  write_node_fix<S, 1>(d, PL, X, F.Ef, F.Eg);
-  write_node_fix<S, 2>(d, PL, X, F.Ef, F.Eg);
-  write_node_fix<S, 3>(d, PL, X, F.Ef, F.Eg);
-  write_node_fix<S, 4>(d, PL, X, F.Ef, F.Eg);
 }
 
 // 52-bit variant: value = X 2^(E - 1074); the magnitude is truncated (toward

@@ -47,9 +47,11 @@ __device__ __forceinline__ void write_expansion(S* d, long long PL, const Coeffs
 
 struct L25 {
   static constexpr int NPOP = 50;
+  typedef Lat25 Tile;
   template <class S>
   __device__ static CellState state(const S* p, long long PL, const Phys& P, const Macro& M) {
-    const Moments m = cell_moments<S>(p, PL, P);
+    Moments m = moments_fix<S>(p, 0u, PL);
+    if constexpr (sizeof(S) == 4) add_reference(m, P);
     CellState c;
     macro_from_moments(m, P, M.c, M.T_ref, c.rho, c.ux, c.uy, c.T);
     c.jx = m.m10 * M.c;
@@ -57,11 +59,9 @@ struct L25 {
     c.E = m.g00 + 0.5 * P.c2 * (m.m20 + m.m02);  // split II: E = sum g + sum v^2/2 f
     return c;
   }
-  // equilibrium populations of (rho, u, T) (Sec. III.A.3 initial conditions)
-  template <class S>
-  __device__ static void write_equilibrium(S* d, long long PL, double rho, double ux, double uy, double T,
-                                           const Phys& P, const Macro& M) {
-    write_equilibrium_fix<S>(d, PL, equilibrium_coeffs(rho, ux / M.c, uy / M.c, T / M.T_ref, P), P);
+  // equilibrium coefficients of (rho, u, T) (Sec. III.A.3 initial conditions)
+  __device__ static Coeffs equilibrium(double rho, double ux, double uy, double T, const Phys& P, const Macro& M) {
+    return equilibrium_coeffs(rho, ux / M.c, uy / M.c, T / M.T_ref, P);
   }
   // wall ghost g mirroring interior cell b (Sec. III.E): equilibrium at
   // rho_B, 2 u_W - u_B, 2 T_W - T_B plus the non-equilibrium part of b
@@ -94,10 +94,11 @@ struct L25 {
 
 struct L16 {
   static constexpr int NPOP = 32;
+  typedef Lat16 Tile;
   template <class S>
   __device__ static CellState state(const S* p, long long PL, const Phys& P, const Macro& M) {
     static_assert(sizeof(S) == 8, "the D2Q16 / split I model has FP64 storage only");
-    const q16::Mom m = q16::cell_moments(p, PL);
+    const q16::Mom m = q16::moments_fix16(p, 0u, PL);
     CellState c;
     q16::macro(m, P, M.c, M.T_ref, c.rho, c.ux, c.uy, c.T);
     c.jx = m.m10 * M.c;
@@ -105,10 +106,8 @@ struct L16 {
     c.E = m.g00;  // split I: E = sum g
     return c;
   }
-  template <class S>
-  __device__ static void write_equilibrium(S* d, long long PL, double rho, double ux, double uy, double T,
-                                           const Phys& P, const Macro& M) {
-    q16::write_equilibrium_fix16(d, PL, q16::equilibrium(rho, ux / M.c, uy / M.c, T / M.T_ref, P));
+  __device__ static q16::Co equilibrium(double rho, double ux, double uy, double T, const Phys& P, const Macro& M) {
+    return q16::equilibrium(rho, ux / M.c, uy / M.c, T / M.T_ref, P);
   }
   template <class S>
   __device__ static void wall_ghost(S* g, const S* b, long long PL, const Phys& P, const Macro& M, double uwx,

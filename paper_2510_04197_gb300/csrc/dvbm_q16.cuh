@@ -201,86 +201,14 @@ __device__ __forceinline__ void write_expansion(double* d, long long PL, const C
 #undef Q16_EXP
 }
 
-// ---- fixed-point expansion (as in dvbm_device.cuh for D2Q25) -------------
-// node constants khq(k, n) 2^(63 + kdq(k)) (|khq| < 0.46; the +-sqrt(3 + sqrt 6)
-// nodes carry the small weight and gain two bits)
-__host__ __device__ constexpr int kdq(int k) { return k < 2 ? 0 : 2; }
-__host__ __device__ constexpr long long khqfix(int k, int n) {
-  return (long long)(khq(k, n) * 9223372036854775808.0 * (double)(1 << kdq(k)));
-}
-struct CoFix {
-  long long f00, f10, f01, f20, f11, f02, f30, f21, f12, f03;
-  long long g00, g10, g01, g20, g11, g02;
-  int Ef, Eg;  // value = X 2^(E - 1082)
-};
-__device__ __forceinline__ CoFix to_fix(const Co& C) {
-  CoFix X;
-  const int Ef = max(max(max(max(bexp(C.f00), bexp(C.f10)), max(bexp(C.f01), bexp(C.f20))),
-                         max(max(bexp(C.f11), bexp(C.f02)), max(bexp(C.f30), bexp(C.f21)))),
-                     max(bexp(C.f12), bexp(C.f03)));
-  const int Eg = max(max(max(bexp(C.g00), bexp(C.g10)), max(bexp(C.g01), bexp(C.g20))),
-                     max(bexp(C.g11), bexp(C.g02)));
-  X.f00 = to_block_fixed(C.f00, Ef); X.f10 = to_block_fixed(C.f10, Ef); X.f01 = to_block_fixed(C.f01, Ef);
-  X.f20 = to_block_fixed(C.f20, Ef); X.f11 = to_block_fixed(C.f11, Ef); X.f02 = to_block_fixed(C.f02, Ef);
-  X.f30 = to_block_fixed(C.f30, Ef); X.f21 = to_block_fixed(C.f21, Ef); X.f12 = to_block_fixed(C.f12, Ef);
-  X.f03 = to_block_fixed(C.f03, Ef);
-  X.g00 = to_block_fixed(C.g00, Eg); X.g10 = to_block_fixed(C.g10, Eg); X.g01 = to_block_fixed(C.g01, Eg);
-  X.g20 = to_block_fixed(C.g20, Eg); X.g11 = to_block_fixed(C.g11, Eg); X.g02 = to_block_fixed(C.g02, Eg);
-  X.Ef = Ef;
-  X.Eg = Eg;
-  return X;
-}
-// t_q = sum_b h^b khq(q, b) with the +-xi symmetry (nodes +a, -a, +b, -b)
-__device__ __forceinline__ void expand_fix(const long long (&h)[4], long long (&t)[4]) {
-  const long long EA = mhk(h[0], khqfix(0, 0)) + mhk(h[2], khqfix(0, 2));
-  const long long OA = mhk(h[1], khqfix(0, 1)) + mhk(h[3], khqfix(0, 3));
-  const long long EB = mhk(h[0], khqfix(2, 0)) + mhk(h[2], khqfix(2, 2));
-  const long long OB = mhk(h[1], khqfix(2, 1)) + mhk(h[3], khqfix(2, 3));
-  t[0] = EA + OA; t[1] = EA - OA; t[2] = EB + OB; t[3] = EB - OB;
-}
-__device__ __forceinline__ void expand3_fix(const long long (&h)[3], long long (&t)[4]) {
-  const long long EA = mhk(h[0], khqfix(0, 0)) + mhk(h[2], khqfix(0, 2));
-  const long long OA = mhk(h[1], khqfix(0, 1));
-  const long long EB = mhk(h[0], khqfix(2, 0)) + mhk(h[2], khqfix(2, 2));
-  const long long OB = mhk(h[1], khqfix(2, 1));
-  t[0] = EA + OA; t[1] = EA - OA; t[2] = EB + OB; t[3] = EB - OB;
-}
-
-}  // namespace q16
-
-namespace q16 {
-// populations of the equilibrium coefficient set C (a1 = 0) by the step
-// kernel's fixed-point expansion (FP64-or-better precision): initial conditions
-__device__ __forceinline__ void write_equilibrium_fix16(double* d, long long PL, const Co& C) {
-  const CoFix X = to_fix(C);
-#pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    const long long k0 = khqfix(p, 0), k1 = khqfix(p, 1), k2 = khqfix(p, 2), k3 = khqfix(p, 3);
-    long long h[4], hh[3], xf[4], xg[4];
-    h[0] = mhk(X.f00, k0) + mhk(X.f10, k1) + mhk(X.f20, k2) + mhk(X.f30, k3);
-    h[1] = mhk(X.f01, k0) + mhk(X.f11, k1) + mhk(X.f21, k2);
-    h[2] = mhk(X.f02, k0) + mhk(X.f12, k1);
-    h[3] = mhk(X.f03, k0);
-    hh[0] = mhk(X.g00, k0) + mhk(X.g10, k1) + mhk(X.g20, k2);
-    hh[1] = mhk(X.g01, k0) + mhk(X.g11, k1);
-    hh[2] = mhk(X.g02, k0);
-    const int sf = renorm_fix(h), sg = renorm_fix(hh);
-    expand_fix(h, xf);
-    expand3_fix(hh, xg);
-    const int dp = kdq(p);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      d[(4 * p + q) * PL] = X.Ef >= 100 ? ll_to_double_rn(xf[q], X.Ef - 1080 - dp - sf - kdq(q)) : 0.0;
-      d[(16 + 4 * p + q) * PL] = X.Eg >= 100 ? ll_to_double_rn(xg[q], X.Eg - 1080 - dp - sg - kdq(q)) : 0.0;
-    }
-  }
-}
 }  // namespace q16
 
 // ---- the step over tiles (k_step_tile) -----------------------------------------
 namespace q16 {
 
 // node constants W_k He_n(xi_k)/n! 2^(61 + kdq(k)), rounded from their exact values
+// (the +-sqrt(3 + sqrt 6) nodes carry the small weight and gain two bits)
+__host__ __device__ constexpr int kdq(int k) { return k < 2 ? 0 : 2; }
 constexpr long long kKQ[2][4] = {
     {1047138985598193535ll, 776939204445353226ll, -235339116647385024ll, -317184102009169216ll},
     {423130076034613764ll, 987760865702054896ll, 941356466589540094ll, 403251684809969295ll}};
@@ -309,7 +237,6 @@ __device__ __forceinline__ long long pair_sum16(long long b, long long a) {
 // moments in block fixed point, as moments_fix for D2Q25
 __device__ __forceinline__ Mom moments_fix16(const double* __restrict__ s, unsigned off, long long PL) {
   Mom m;
-  bool finite = true;
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     double v[16];
@@ -319,7 +246,6 @@ __device__ __forceinline__ Mom moments_fix16(const double* __restrict__ s, unsig
       v[i] = __ldg(at(s + (16 * k + i) * PL, off));
       key = max(key, abs_key(v[i]));
     }
-    finite = finite && key < 0x7ff00000u;
     const int E = (int)(key >> 20);
     const int n0 = E < 128 ? 63 : 2;
     const int sc = E - 1080;
@@ -334,7 +260,7 @@ __device__ __forceinline__ Mom moments_fix16(const double* __restrict__ s, unsig
       if (k == 0) M2s += pair_sum16<2>(sB, sA);
     }
     const long long a0 = M0[0] + M0[1], b0 = M0[2] + M0[3], c0 = M0[0] - M0[1], d0 = M0[2] - M0[3];
-    const double s00 = fix_to_double<true>(a0 + b0, sc);
+    const double s00 = key < 0x7ff00000u ? fix_to_double<true>(a0 + b0, sc) : __longlong_as_double(0x7ff8000000000000ll);
     const double s10 = fix_to_double<true>(pair_sum16<1>(d0, c0), sc + 4);
     const double s01 = fix_to_double<true>((M1[0] + M1[1]) + (M1[2] + M1[3]), sc + 4);
     if (k == 0) {
@@ -346,7 +272,6 @@ __device__ __forceinline__ Mom moments_fix16(const double* __restrict__ s, unsig
       m.g00 = s00; m.g10 = s10; m.g01 = s01;
     }
   }
-  if (!finite) m.m00 = __longlong_as_double(0x7ff8000000000000ll);
   return m;
 }
 template <int k, int n>
@@ -360,7 +285,7 @@ struct Lat16 {
   typedef q16::Mom Mom;
   typedef int NodeK[4][2];
   __device__ static __forceinline__ bool backward(int k) { return (k & 1) != 0; }
-  __device__ static __forceinline__ int kdp(int k) { return k < 2 ? 0 : 2; }
+  __device__ static __forceinline__ int kdp(int k) { return q16::kdq(k); }
   __device__ static __forceinline__ Mom moments(const double* s, unsigned off, long long PL) {
     return q16::moments_fix16(s, off, PL);
   }

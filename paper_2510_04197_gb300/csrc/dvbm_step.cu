@@ -77,10 +77,7 @@ __global__ void __launch_bounds__(kCta, 1024 / kCta) k_step32(const float* __res
   float* d = dst + off;
   const long long PL = G.plane;
   Moments m = moments_fix<float>(s, 0u, PL);
-  // moments of the reference populations w rho0 (f) and w G0 (g):
-  // sum w = 1, sum w xi^2 = 1 per axis, odd moments vanish
-  m.m00 += P.fref0; m.m20 += P.fref0; m.m02 += P.fref0;
-  m.g00 += P.gref0;
+  add_reference(m, P);
   Coeffs C = collision_coeffs<PRC>(m, P);
   if (C.bad) atomicOr(flag, 1u);
   // the expansion then yields t - (dt/tau1) F_ref directly: the reference
