@@ -5,9 +5,9 @@
 //
 //  k_init     equilibrium populations of given (rho, u, T) fields (Sec. III.A.3),
 //             by the step kernels' block-fixed-point Grad expansion
-//  k_ghost    two ghost layers per non-... side: periodic wrap, zero-gradient copy,
-//             or no-slip isothermal wall by ghost node + non-equilibrium
-//             extrapolation (Sec. III.E): rho_G = rho_B, u_G = 2 u_W - u_B,
+//  k_ghost    two ghost layers per side: periodic wrap or zero-gradient copy
+//  k_wall     the ghost layers of no-slip isothermal walls by ghost node +
+//             non-equilibrium extrapolation (Sec. III.E): rho_G = rho_B, u_G = 2 u_W - u_B,
 //             T_G = 2 T_W - T_B, F_G = F^eq(G) + (F_B - F^eq(B)); ghost k
 //             mirrors interior cell k (k = 1, 2)
 //  k_moments  rho, u, T fields
@@ -68,40 +68,80 @@ __global__ void __launch_bounds__(kCta, 3) k_init(S* __restrict__ dst, const dou
   }
 }
 
-// one thread per (side, layer k, position along the side, population);
-// sides 0..3 = xlo, xhi, ylo, yhi, blockIdx.z = population.  Periodic and
-// zero-gradient sides copy one population per thread; a wall side needs all
-// populations of its mirror cell and is done by the blockIdx.z = 0 slice.
-template <class L, class S>
-__global__ void k_ghost(S* __restrict__ buf, Geom G, Phys P, Macro M, BCDev bc) {
-  const int side = blockIdx.y;
-  const int kind = bc.kind[side];
-  const int pop = blockIdx.z;
-  if (kind == 3) return;  // external: the caller supplies these rows (dvbm_halo_unpack)
-  if (kind == 2 && pop != 0) return;
+// Ghost layer k (1 or 2) of position j along a side: the ghost cell (gx, gy) and its
+// source, by kind: periodic wrap, zero gradient, or a wall's mirror cell (ghost k
+// mirrors interior cell k).  Sides 0..3 = xlo, xhi, ylo, yhi.
+__device__ __forceinline__ void ghost_cells(int side, int kind, int k, int j, const Geom& G, int& gx, int& gy, int& bx,
+                                            int& by) {
+  const bool lo = (side % 2) == 0;
+  const int n = side < 2 ? G.Nx : G.Ny;
+  const int gi = lo ? -k : n - 1 + k;  // coordinate along the normal
+  int bi;
+  if (kind == 0) bi = lo ? n - k : k - 1;
+  else if (kind == 1) bi = lo ? 0 : n - 1;
+  else bi = lo ? k - 1 : n - k;
+  if (side < 2) { gx = gi; gy = j; bx = bi; by = j; }
+  else          { gx = j; gy = gi; bx = j; by = bi; }
+}
+
+// periodic and zero-gradient sides, one thread per (side, layer, position, population)
+template <class S>
+__global__ void k_ghost(S* __restrict__ buf, Geom G, BCDev bc) {
+  const int side = blockIdx.y, kind = bc.kind[side], pop = blockIdx.z;
+  if (kind > 1) return;
   const int len = side < 2 ? G.Ny : G.Nx;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= 2 * len) return;
-  const int k = 1 + t / len;        // ghost layer 1 or 2
-  const int j = t % len;            // position along the side
-  int gx, gy, bx, by;               // ghost cell and source/mirror cell
-  const bool lo = (side % 2) == 0;
-  const int n = side < 2 ? G.Nx : G.Ny;
-  int gi = lo ? -k : n - 1 + k;     // ghost coordinate along the normal
-  int bi;
-  if (kind == 0) bi = lo ? n - k : k - 1;            // periodic wrap
-  else if (kind == 1) bi = lo ? 0 : n - 1;           // zero gradient
-  else bi = lo ? k - 1 : n - k;                      // wall: mirror cell
-  if (side < 2) { gx = gi; gy = j; bx = bi; by = j; }
-  else          { gx = j; gy = gi; bx = j; by = bi; }
+  int gx, gy, bx, by;
+  ghost_cells(side, kind, 1 + t / len, t % len, G, gx, gy, bx, by);
+  buf[pop * G.plane + cell_index(G, gy, gx)] = buf[pop * G.plane + cell_index(G, by, bx)];
+}
+
+// Isothermal no-slip walls: F_G = F^eq(rho_B, 2 u_W - u_B, 2 T_W - T_B) + (F_B - F^eq(B)),
+// i.e. F_B plus the expansion of the difference of the two equilibria's
+// coefficients, in the step kernels' fixed point.  The kernel's work is small
+// and all latency, so a ghost cell has eight threads, which all form the
+// coefficients and share the populations (units of an x-node's f or g): one
+// thread a cell took 33 us of a 55 us step at 4 x 256, this takes 21.
+template <class L, class S>
+__global__ void __launch_bounds__(kCta, 2) k_wall(S* __restrict__ buf, Geom G, Phys P, Macro M, BCDev bc) {
+  typedef typename L::Tile LT;
+  constexpr int NQ = LT::NQ, NF = NQ * NQ;
+  __shared__ long long s_buf[LT::FIELDS * kCta];
+  const int side = blockIdx.y;
+  if (bc.kind[side] != 2) return;
+  const int len = side < 2 ? G.Ny : G.Nx;
+  const int t = blockIdx.x * 32 + threadIdx.x;
+  if (t >= 2 * len) return;
+  int gx, gy, bx, by;
+  ghost_cells(side, 2, 1 + t / len, t % len, G, gx, gy, bx, by);
   const long long PL = G.plane;
-  S* gptr = buf + cell_index(G, gy, gx);
-  const S* bptr = buf + cell_index(G, by, bx);
-  if (kind != 2) {
-    gptr[pop * PL] = bptr[pop * PL];
-    return;
+  S* g = buf + cell_index(G, gy, gx);
+  const S* b = buf + cell_index(G, by, bx);
+  long long* slot = s_buf + threadIdx.y * 32 + threadIdx.x;
+  int Ef, Eg;
+  {
+    const CellState c = L::template state<S>(b, PL, P, M);
+    auto D = L::equilibrium(c.rho, 2.0 * bc.uw[side][0] - c.ux, 2.0 * bc.uw[side][1] - c.uy, 2.0 * bc.Tw[side] - c.T, P, M);
+    L::subtract(D, L::equilibrium(c.rho, c.ux, c.uy, c.T, P, M));
+    LT::to_smem(D, slot, Ef, Eg);
   }
-  L::template wall_ghost<S>(gptr, bptr, PL, P, M, bc.uw[side][0], bc.uw[side][1], bc.Tw[side]);
+  const FixView X{slot};
+#pragma unroll 1
+  for (int u = threadIdx.y; u < 2 * NQ; u += 8) {
+    const int p = u >> 1, k = u & 1;
+    typename LT::NodeK K;
+    LT::load_k(p, K);
+    long long v[NQ];
+    if (k == 0) LT::target_f(X, K, v);
+    else LT::target_g(X, K, v);
+    const int sc = (k == 0 ? Ef : Eg) - 1079 - LT::kdp(p);
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const long long o = (NF * k + NQ * p + q) * PL;
+      g[o] = (S)((double)b[o] + fix_to_double<true>(v[q], sc - LT::kdp(q)));
+    }
+  }
 }
 
 template <class L, class S>
@@ -265,10 +305,22 @@ cudaError_t launch_init(int lattice, int storage, void* dst, const double* rho, 
 cudaError_t launch_ghost(int lattice, int storage, void* buf, const Geom& G, const Phys& P, const Macro& M,
                          const BCDev& bc, cudaStream_t st) {
   const int len = G.Nx > G.Ny ? G.Nx : G.Ny;
-  dim3 b(128), g((2 * len + 127) / 128, 4, lattice == 1 ? L16::NPOP : L25::NPOP);
-  if (lattice == 1) k_ghost<L16, double><<<g, b, 0, st>>>((double*)buf, G, P, M, bc);
-  else if (storage == 0) k_ghost<L25, double><<<g, b, 0, st>>>((double*)buf, G, P, M, bc);
-  else k_ghost<L25, float><<<g, b, 0, st>>>((float*)buf, G, P, M, bc);
+  bool copies = false, walls = false;
+  for (int k = 0; k < 4; ++k) {
+    copies = copies || bc.kind[k] < 2;
+    walls = walls || bc.kind[k] == 2;
+  }
+  if (copies) {
+    const dim3 b(128), g((2 * len + 127) / 128, 4, lattice == 1 ? L16::NPOP : L25::NPOP);
+    if (storage == 0) k_ghost<double><<<g, b, 0, st>>>((double*)buf, G, bc);
+    else k_ghost<float><<<g, b, 0, st>>>((float*)buf, G, bc);
+  }
+  if (walls) {
+    const dim3 b(32, 8), g((2 * len + 31) / 32, 4);
+    if (lattice == 1) k_wall<L16, double><<<g, b, 0, st>>>((double*)buf, G, P, M, bc);
+    else if (storage == 0) k_wall<L25, double><<<g, b, 0, st>>>((double*)buf, G, P, M, bc);
+    else k_wall<L25, float><<<g, b, 0, st>>>((float*)buf, G, P, M, bc);
+  }
   return cudaGetLastError();
 }
 

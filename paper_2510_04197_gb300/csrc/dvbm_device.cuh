@@ -277,53 +277,6 @@ __device__ __forceinline__ void accumulate_moments(Moments& m, const double (&f)
   }
 }
 
-// ---- sum-factorised Grad expansion ----------------------------------------
-// h^b_p = W_p sum_a C_ab He_a(xi_p)/a!  for the f expansion (N = 4).
-template <int p>
-__device__ __forceinline__ void hf_of(const Coeffs& C, double (&h)[5]) {
-  if (p != 0) {
-    h[0] = fma(kh(p, 4), C.f40, fma(kh(p, 3), C.f30, fma(kh(p, 2), C.f20, fma(kh(p, 1), C.f10, kh(p, 0) * C.f00))));
-    h[1] = fma(kh(p, 3), C.f31, fma(kh(p, 2), C.f21, fma(kh(p, 1), C.f11, kh(p, 0) * C.f01)));
-    h[2] = fma(kh(p, 2), C.f22, fma(kh(p, 1), C.f12, kh(p, 0) * C.f02));
-    h[3] = fma(kh(p, 1), C.f13, kh(p, 0) * C.f03);
-  } else {  // He_1(0) = He_3(0) = 0
-    h[0] = fma(kh(p, 4), C.f40, fma(kh(p, 2), C.f20, kh(p, 0) * C.f00));
-    h[1] = fma(kh(p, 2), C.f21, kh(p, 0) * C.f01);
-    h[2] = fma(kh(p, 2), C.f22, kh(p, 0) * C.f02);
-    h[3] = kh(p, 0) * C.f03;
-  }
-  h[4] = kh(p, 0) * C.f04;
-}
-template <int p>
-__device__ __forceinline__ void hg_of(const Coeffs& C, double (&h)[3]) {
-  if (p != 0) {
-    h[0] = fma(kh(p, 2), C.g20, fma(kh(p, 1), C.g10, kh(p, 0) * C.g00));
-    h[1] = fma(kh(p, 1), C.g11, kh(p, 0) * C.g01);
-  } else {
-    h[0] = fma(kh(p, 2), C.g20, kh(p, 0) * C.g00);
-    h[1] = kh(p, 0) * C.g01;
-  }
-  h[2] = kh(p, 0) * C.g02;
-}
-// t_q = W_q sum_b h^b He_b(xi_q)/b! for the five y-nodes, using the +-xi
-// symmetry: even part E and odd part O, t(+xi) = E + O, t(-xi) = E - O.
-__device__ __forceinline__ void expand_q5(const double (&h)[5], double (&t)[5]) {
-  t[0] = fma(kh(0, 4), h[4], fma(kh(0, 2), h[2], kh(0, 0) * h[0]));
-  const double EA = fma(kh(1, 4), h[4], fma(kh(1, 2), h[2], kh(1, 0) * h[0]));
-  const double OA = fma(kh(1, 3), h[3], kh(1, 1) * h[1]);
-  const double EB = fma(kh(3, 4), h[4], fma(kh(3, 2), h[2], kh(3, 0) * h[0]));
-  const double OB = fma(kh(3, 3), h[3], kh(3, 1) * h[1]);
-  t[1] = EA + OA; t[2] = EA - OA; t[3] = EB + OB; t[4] = EB - OB;
-}
-__device__ __forceinline__ void expand_q3(const double (&h)[3], double (&t)[5]) {
-  t[0] = fma(kh(0, 2), h[2], kh(0, 0) * h[0]);
-  const double EA = fma(kh(1, 2), h[2], kh(1, 0) * h[0]);
-  const double OA = kh(1, 1) * h[1];
-  const double EB = fma(kh(3, 2), h[2], kh(3, 0) * h[0]);
-  const double OB = kh(3, 1) * h[1];
-  t[1] = EA + OA; t[2] = EA - OA; t[3] = EB + OB; t[4] = EB - OB;
-}
-
 // ---- limited slope of the NND reconstruction (Sec. III.A.2) --------------
 // sigma(a, b) = (b/2) phi(a/b) = 1/2 minmod3(beta a, (a+b)/2, beta b)
 //             = minmod3(hb a, (a+b)/4, hb b),  hb = beta/2,

@@ -17,34 +17,6 @@ struct CellState {
   double rho, jx, jy, E, ux, uy, T;
 };
 
-// write the expansion of coefficient set C (pure equilibrium: a1 = 0, k1 = 1)
-// at one padded offset in double arithmetic; addf/addg (nullable) add
-// per-population values (the wall closure's non-equilibrium parts)
-template <class S>
-__device__ __forceinline__ void write_expansion(S* d, long long PL, const Coeffs& C, const Phys& P,
-                                                const double* addf, const double* addg) {
-#define DVBM_EXP(p)                                                              \
-  {                                                                              \
-    double hf[5], tf[5], hg[3], tg[5];                                           \
-    hf_of<p>(C, hf); expand_q5(hf, tf);                                          \
-    hg_of<p>(C, hg); expand_q3(hg, tg);                                          \
-    _Pragma("unroll") for (int q = 0; q < 5; ++q) {                              \
-      double vf = tf[q], vg = tg[q];                                             \
-      if (addf) { vf += addf[5 * p + q]; vg += addg[5 * p + q]; }                \
-      if constexpr (sizeof(S) == 8) {                                            \
-        d[(5 * p + q) * PL] = vf;                                                \
-        d[(25 + 5 * p + q) * PL] = vg;                                           \
-      } else {                                                                   \
-        const double w = w_of(p) * w_of(q);                                      \
-        d[(5 * p + q) * PL] = __double2float_rn(vf - P.fref0 * w);               \
-        d[(25 + 5 * p + q) * PL] = __double2float_rn(vg - P.gref0 * w);          \
-      }                                                                          \
-    }                                                                            \
-  }
-  DVBM_EXP(0) DVBM_EXP(1) DVBM_EXP(2) DVBM_EXP(3) DVBM_EXP(4)
-#undef DVBM_EXP
-}
-
 struct L25 {
   static constexpr int NPOP = 50;
   typedef Lat25 Tile;
@@ -63,32 +35,11 @@ struct L25 {
   __device__ static Coeffs equilibrium(double rho, double ux, double uy, double T, const Phys& P, const Macro& M) {
     return equilibrium_coeffs(rho, ux / M.c, uy / M.c, T / M.T_ref, P);
   }
-  // wall ghost g mirroring interior cell b (Sec. III.E): equilibrium at
-  // rho_B, 2 u_W - u_B, 2 T_W - T_B plus the non-equilibrium part of b
-  template <class S>
-  __device__ static void wall_ghost(S* g, const S* b, long long PL, const Phys& P, const Macro& M, double uwx,
-                                    double uwy, double Tw) {
-    const Moments m = cell_moments<S>(b, PL, P);
-    double rho, ux, uy, T;
-    macro_from_moments(m, P, M.c, M.T_ref, rho, ux, uy, T);
-    const Coeffs CB = equilibrium_coeffs(rho, ux / M.c, uy / M.c, T / M.T_ref, P);
-    const Coeffs CG = equilibrium_coeffs(rho, (2.0 * uwx - ux) / M.c, (2.0 * uwy - uy) / M.c,
-                                         (2.0 * Tw - T) / M.T_ref, P);
-    double neqf[25], neqg[25];
-    {
-      double hf[5], tf[5], hg[3], tg[5];
-#define DVBM_NEQ(p)                                                                   \
-      hf_of<p>(CB, hf); expand_q5(hf, tf); hg_of<p>(CB, hg); expand_q3(hg, tg);       \
-      _Pragma("unroll") for (int q = 0; q < 5; ++q) {                                 \
-        double w = 0.0;                                                               \
-        if constexpr (sizeof(S) == 4) w = w_of(p) * w_of(q);                          \
-        neqf[5 * p + q] = ((double)b[(5 * p + q) * PL] + P.fref0 * w) - tf[q];        \
-        neqg[5 * p + q] = ((double)b[(25 + 5 * p + q) * PL] + P.gref0 * w) - tg[q];   \
-      }
-      DVBM_NEQ(0) DVBM_NEQ(1) DVBM_NEQ(2) DVBM_NEQ(3) DVBM_NEQ(4)
-#undef DVBM_NEQ
-    }
-    write_expansion<S>(g, PL, CG, P, neqf, neqg);
+  __device__ static void subtract(Coeffs& A, const Coeffs& B) {
+    A.f00 -= B.f00; A.f10 -= B.f10; A.f01 -= B.f01; A.f20 -= B.f20; A.f11 -= B.f11; A.f02 -= B.f02; A.f30 -= B.f30;
+    A.f21 -= B.f21; A.f12 -= B.f12; A.f03 -= B.f03; A.f40 -= B.f40; A.f31 -= B.f31; A.f22 -= B.f22; A.f13 -= B.f13;
+    A.f04 -= B.f04;
+    A.g00 -= B.g00; A.g10 -= B.g10; A.g01 -= B.g01; A.g20 -= B.g20; A.g11 -= B.g11; A.g02 -= B.g02;
   }
 };
 
@@ -109,28 +60,10 @@ struct L16 {
   __device__ static q16::Co equilibrium(double rho, double ux, double uy, double T, const Phys& P, const Macro& M) {
     return q16::equilibrium(rho, ux / M.c, uy / M.c, T / M.T_ref, P);
   }
-  template <class S>
-  __device__ static void wall_ghost(S* g, const S* b, long long PL, const Phys& P, const Macro& M, double uwx,
-                                    double uwy, double Tw) {
-    const q16::Mom m = q16::cell_moments(b, PL);
-    double rho, ux, uy, T;
-    q16::macro(m, P, M.c, M.T_ref, rho, ux, uy, T);
-    const q16::Co CB = q16::equilibrium(rho, ux / M.c, uy / M.c, T / M.T_ref, P);
-    const q16::Co CG = q16::equilibrium(rho, (2.0 * uwx - ux) / M.c, (2.0 * uwy - uy) / M.c,
-                                        (2.0 * Tw - T) / M.T_ref, P);
-    double neqf[16], neqg[16];
-#define Q16_NEQ(p)                                                                     \
-    {                                                                                  \
-      double h[4], tf[4], hh[4], tg[4];                                                \
-      q16::hf<p>(CB, h); q16::expand(h, tf); q16::hg<p>(CB, hh); q16::expand(hh, tg);  \
-      _Pragma("unroll") for (int q = 0; q < 4; ++q) {                                  \
-        neqf[4 * p + q] = b[(4 * p + q) * PL] - tf[q];                                 \
-        neqg[4 * p + q] = b[(16 + 4 * p + q) * PL] - tg[q];                            \
-      }                                                                                \
-    }
-    Q16_NEQ(0) Q16_NEQ(1) Q16_NEQ(2) Q16_NEQ(3)
-#undef Q16_NEQ
-    q16::write_expansion(g, PL, CG, neqf, neqg);
+  __device__ static void subtract(q16::Co& A, const q16::Co& B) {
+    A.f00 -= B.f00; A.f10 -= B.f10; A.f01 -= B.f01; A.f20 -= B.f20; A.f11 -= B.f11; A.f02 -= B.f02;
+    A.f30 -= B.f30; A.f21 -= B.f21; A.f12 -= B.f12; A.f03 -= B.f03;
+    A.g00 -= B.g00; A.g10 -= B.g10; A.g01 -= B.g01; A.g20 -= B.g20; A.g11 -= B.g11; A.g02 -= B.g02;
   }
 };
 

@@ -40,23 +40,6 @@ struct Co {
   bool bad;
 };
 
-template <int p>
-__device__ __forceinline__ void accumulate(Mom& m, const double (&f)[4], const double (&g)[4]) {
-  const double sA = f[0] + f[1], dA = f[0] - f[1], sB = f[2] + f[3], dB = f[2] - f[3];
-  const double m0 = sA + sB;
-  const double m1 = fma(YA, dA, YB * dB);
-  const double m2 = fma(YA * YA, sA, (YB * YB) * sB);
-  const double n0 = (g[0] + g[1]) + (g[2] + g[3]);
-  const double n1 = fma(YA, g[0] - g[1], YB * (g[2] - g[3]));
-  constexpr double x = xi(p);
-  m.m00 += m0; m.m01 += m1; m.m02 += m2;
-  m.m10 = fma(x, m0, m.m10);
-  m.m11 = fma(x, m1, m.m11);
-  m.m20 = fma(x * x, m0, m.m20);
-  m.g00 += n0; m.g01 += n1;
-  m.g10 = fma(x, n0, m.g10);
-}
-
 struct Eq3 { double a00, a10, a01, a20, a11, a02, a30, a21, a12, a03; };
 struct EqG { double A00, A10, A01, A20, A11, A02; };
 
@@ -137,43 +120,6 @@ __device__ __forceinline__ Co equilibrium(double rho, double ux, double uy, doub
   return C;
 }
 
-template <int p>
-__device__ __forceinline__ void hf(const Co& C, double (&h)[4]) {
-  h[0] = fma(khq(p, 3), C.f30, fma(khq(p, 2), C.f20, fma(khq(p, 1), C.f10, khq(p, 0) * C.f00)));
-  h[1] = fma(khq(p, 2), C.f21, fma(khq(p, 1), C.f11, khq(p, 0) * C.f01));
-  h[2] = fma(khq(p, 1), C.f12, khq(p, 0) * C.f02);
-  h[3] = khq(p, 0) * C.f03;
-}
-template <int p>
-__device__ __forceinline__ void hg(const Co& C, double (&h)[4]) {
-  h[0] = fma(khq(p, 2), C.g20, fma(khq(p, 1), C.g10, khq(p, 0) * C.g00));
-  h[1] = fma(khq(p, 1), C.g11, khq(p, 0) * C.g01);
-  h[2] = khq(p, 0) * C.g02;
-  h[3] = 0.0;
-}
-// t_q = W_q sum_b h^b He_b(xi_q)/b!, nodes (+a, -a, +b, -b)
-__device__ __forceinline__ void expand(const double (&h)[4], double (&t)[4]) {
-  const double EA = fma(khq(0, 2), h[2], khq(0, 0) * h[0]);
-  const double OA = fma(khq(0, 3), h[3], khq(0, 1) * h[1]);
-  const double EB = fma(khq(2, 2), h[2], khq(2, 0) * h[0]);
-  const double OB = fma(khq(2, 3), h[3], khq(2, 1) * h[1]);
-  t[0] = EA + OA; t[1] = EA - OA; t[2] = EB + OB; t[3] = EB - OB;
-}
-
-__device__ __forceinline__ Mom cell_moments(const double* s, long long PL) {
-  Mom m = {};
-  double f[4], g[4];
-#define Q16_MOM(p)                                                     \
-  _Pragma("unroll") for (int q = 0; q < 4; ++q) {                     \
-    f[q] = __ldg(s + (4 * p + q) * PL);                                \
-    g[q] = __ldg(s + (16 + 4 * p + q) * PL);                           \
-  }                                                                    \
-  accumulate<p>(m, f, g);
-  Q16_MOM(0) Q16_MOM(1) Q16_MOM(2) Q16_MOM(3)
-#undef Q16_MOM
-  return m;
-}
-
 __device__ __forceinline__ void macro(const Mom& m, const Phys& P, double c, double T_ref, double& rho, double& ux,
                                       double& uy, double& T) {
   rho = m.m00;
@@ -185,26 +131,7 @@ __device__ __forceinline__ void macro(const Mom& m, const Phys& P, double c, dou
   T = theta * T_ref;
 }
 
-// write the expansion of C (plus optional per-population additions)
-__device__ __forceinline__ void write_expansion(double* d, long long PL, const Co& C, const double* addf,
-                                                const double* addg) {
-#define Q16_EXP(p)                                                     \
-  {                                                                    \
-    double h[4], t[4], hh[4], tt[4];                                   \
-    hf<p>(C, h); expand(h, t); hg<p>(C, hh); expand(hh, tt);           \
-    _Pragma("unroll") for (int q = 0; q < 4; ++q) {                    \
-      d[(4 * p + q) * PL] = t[q] + (addf ? addf[4 * p + q] : 0.0);     \
-      d[(16 + 4 * p + q) * PL] = tt[q] + (addg ? addg[4 * p + q] : 0.0); \
-    }                                                                  \
-  }
-  Q16_EXP(0) Q16_EXP(1) Q16_EXP(2) Q16_EXP(3)
-#undef Q16_EXP
-}
-
-}  // namespace q16
-
 // ---- the step over tiles (k_step_tile) -----------------------------------------
-namespace q16 {
 
 // node constants W_k He_n(xi_k)/n! 2^(61 + kdq(k)), rounded from their exact values
 // (the +-sqrt(3 + sqrt 6) nodes carry the small weight and gain two bits)
