@@ -20,6 +20,17 @@ namespace dvbm {
 // this body serves the four moving x-nodes and the kernel's code stays small
 // enough for the instruction cache.  The y-node loop stays unrolled (1754 vs
 // 1722 MLUPS rolled at 4096^2).
+// the five targets t_q 2^(scale - kd(q)) of an x-node as floats: the hardware's
+// conversion (one slot of the FP64 pipe, which this kernel does not fill, for
+// about fifteen integer instructions) and two exact power-of-two factors
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float(min(max(e + 127, 0), 254) << 23); }
+__device__ __forceinline__ void to_floats(const long long (&t)[5], int scale, float (&f)[5]) {
+  const int s1 = scale >> 1;
+  const float m1 = pow2f(s1), m2 = pow2f(scale - s1);
+#pragma unroll
+  for (int q = 0; q < 5; ++q) f[q] = (__ll2float_rn(t[q]) * m1) * (m2 * (1.0f / (float)(1 << kd(q))));
+}
+
 template <bool CENTER>
 __device__ __forceinline__ void node_update32(int p, const float* __restrict__ s, float* __restrict__ d, const Geom& G,
                                               const FixView& X, int Ef, int Eg, const Phys& P, float a1f) {
@@ -32,12 +43,10 @@ __device__ __forceinline__ void node_update32(int p, const float* __restrict__ s
     long long hf[5], hg[3], t[5];
     hf_node(X, K, hf);
     expand_node(hf, t);
-#pragma unroll
-    for (int q = 0; q < 5; ++q) tf[q] = ll_to_float_rn(t[q], Ef - 1079 - dp - kd(q));
+    to_floats(t, Ef - 1079 - dp, tf);
     hg_node(X, K, hg);
     expand_node(hg, t);
-#pragma unroll
-    for (int q = 0; q < 5; ++q) tg[q] = ll_to_float_rn(t[q], Eg - 1079 - dp - kd(q));
+    to_floats(t, Eg - 1079 - dp, tg);
   }
   // x-node sign and flux factor (p = 1, 3: +xi; p = 2, 4: -xi); warp-uniform selects
   const int sx = (p & 1) ? 1 : -1;
