@@ -522,17 +522,453 @@ __device__ __forceinline__ double advection_adjoint_rat(const double* __restrict
   return adjoint_combine_rat(L, stride, bm, b0, bp, lp, lq, sgn);
 }
 
+// ------------------------------------------------- the coded adjoint step over tiles
+// One adjoint step in one launch, with the branch codes of the recomputed forward
+// step, in the forward step's two phases (k_step_tile): first one population per
+// warp over a 32 x 8 tile, then one cell per thread.  512^2: 0.47 ms for the two
+// kernels it replaces (one thread per cell and population in the advection, 64-bit
+// high products in the projection) -> 0.36 ms.  Bound by the FP64 pipe (54 % busy, about
+// 460 instructions a cell, half of them the reverse pass over the collision
+// coefficients) and by latency at 16 warps an SM.
+
+// a code's multipliers 4 lq d(sigma)/d(first argument), /d(second), as a byte table
+// indexed by the code (lp and lq are coprime and lq <= 64, so 2 lp <= 254 fits)
+__device__ __forceinline__ unsigned code_factor(unsigned table, unsigned code) {
+  return __byte_perm(table, 0u, (code & 3u) | 0x4440u);
+}
+
+// What a warp reads of one population: the adjoint state at its lane's column in
+// stream rows -1 .. R + 1, one cell of the x-halo, the branch codes of its
+// column in rows -1 .. R (packed: x bits of rows 0 .., y bits of rows -1 ..)
+// and, lanes 0 .. 15, of the cells before and behind row lane % 8.
+constexpr int kAdjR = 8;
+struct AdjointLoad {
+  double v[kAdjR + 3], h;
+  unsigned char code[kAdjR + 2], edge;
+};
+struct CodePlane {
+  const unsigned char *own, *lo, *hi;  // [Ny][Nx]; the rows below y = 0 and above y = Ny - 1
+  int Nx, Ny;
+  __device__ __forceinline__ const unsigned char* row(int y) const {
+    return y < 0 ? lo : y >= Ny ? hi : own + (long long)y * Nx;
+  }
+};
+__device__ __forceinline__ void adjoint_load(AdjointLoad& L, const double* __restrict__ plane, long long PT,
+                                             const CodePlane& C, int x0, int y0, const AdvTile& T) {
+  const int i = min(T.lane, T.W - 1);
+  const int cx = T.fx ? T.W - 1 - i : i;
+  const long long sy = T.fy ? -PT : PT;
+  const double* row0 = plane + (T.fy ? (T.H - 1) * PT : 0);
+#pragma unroll
+  for (int j = -1; j <= kAdjR + 1; ++j) L.v[j + 1] = __ldg(at(row0 + min(j, T.H + 1) * sy, (unsigned)cx * 8u));
+  const int hr = min(T.lane & 7, T.H - 1), hc = T.lane >> 3;  // stream columns -1, W, W + 1 (or 0)
+  const int h = hc == 0 ? -1 : hc == 3 ? 0 : T.W - 1 + hc;
+  L.h = __ldg(row0 + hr * sy + (T.fx ? T.W - 1 - h : h));
+#pragma unroll
+  for (int j = -1; j <= kAdjR; ++j) {
+    const int y = y0 + (T.fy ? T.H - 1 - min(j, T.H) : min(j, T.H));
+    L.code[j + 1] = __ldg(C.row(y) + x0 + cx);
+  }
+  const int he = T.lane < 8 ? -1 : T.W;
+  int xe = x0 + (T.fx ? T.W - 1 - he : he);
+  xe = xe < 0 ? C.Nx - 1 : xe >= C.Nx ? 0 : xe;
+  L.edge = __ldg(C.own + (long long)(y0 + (T.fy ? T.H - 1 - hr : hr)) * C.Nx + xe);
+}
+
+// The transpose of advect_tile, gathered: with sb_i = l_i - l_{i+1} along the
+// stream and the slopes' partial derivatives d1, d2,
+//     Dbar_i = l_i + d1(sigma_i) sb_i + d2(sigma_{i-1}) sb_{i-1},
+// cell i gets k (Dbar_i - Dbar_{i+1}), subtracted from its adjoint.  Writes the
+// sums over both axes as integers in units of 2^(E - 1076), returns E.  Walked
+// against an axis, the codes' arguments are swapped (tables t1, t2).
+template <bool MX, bool MY, class Next>
+__device__ __forceinline__ int adjoint_walk(const AdjointLoad& L, const Next& next, long long* out, long long PT,
+                                            const AdvTile& T, const Phys& P, long long kx, long long ky, long long* xs) {
+  constexpr int R = kAdjR;
+  const int lane = T.lane;
+  const bool in = lane < T.W;
+  const unsigned lx = in ? (unsigned)(T.fx ? T.W - 1 - lane : lane) : 0u;
+  const long long sy = T.fy ? -PT : PT;
+  constexpr int J0 = MY ? -1 : 0, J1 = MY ? R + 1 : R - 1;
+  unsigned key = 0;
+#pragma unroll
+  for (int j = J0; j <= J1; ++j) key = max(key, ((unsigned)__double2hiint(L.v[j + 1]) + 0x100000u) & 0x7fffffffu);
+  if (MX) key = max(key, ((unsigned)__double2hiint(L.h) + 0x100000u) & 0x7fffffffu);
+  key = __reduce_max_sync(0xffffffffu, key);
+  const int E = (int)(key >> 20) - 1;
+  const int n0 = E < 128 ? 63 : P.advn + 3;
+  __syncwarp();
+#pragma unroll
+  for (int j = J0; j <= J1; ++j) xs[(j + 1) * kAdvPitch + lane + 1] = block_fix(L.v[j + 1], E, n0);
+  const int hr = lane & 7, hc = lane >> 3;
+  if (MX) {
+    __syncwarp();
+    if (hc < 3 && hr < T.H) xs[(hr + 1) * kAdvPitch + (hc == 0 ? 0 : T.W + hc)] = block_fix(L.h, E, n0);
+  }
+  unsigned xb = 0, yb = 0;  // codes of rows 0 .. R - 1 (x), -1 .. R (y), two bits each
+#pragma unroll
+  for (int j = 0; j < R; ++j) xb |= (unsigned)(L.code[j + 1] & 3) << (2 * j);
+#pragma unroll
+  for (int j = -1; j <= R; ++j) yb |= (unsigned)(L.code[j + 1] >> 2) << (2 * (j + 1));
+  const unsigned edge = L.edge & 3u;
+  next();
+  __syncwarp();
+  const unsigned q4 = 4u * (unsigned)P.lq;
+  const unsigned f1 = (2u * (unsigned)P.lp) << 8 | (unsigned)P.lq << 16, f3 = (2u * (unsigned)P.lp) << 24 | (unsigned)P.lq << 16;
+  const unsigned x1 = T.fx ? f3 : f1, x2 = T.fx ? f1 : f3, y1 = T.fy ? f3 : f1, y2 = T.fy ? f1 : f3;
+  if (MX) {
+    // Dbar of column W, one row per lane, kept in column W + 1
+    const unsigned last = __shfl_sync(0xffffffffu, xb, T.W - 1);  // codes of column W - 1
+    const unsigned be = __shfl_sync(0xffffffffu, edge, 8 + (lane & 7));
+    if (lane < T.H) {
+      long long* r = xs + (lane + 1) * kAdvPitch + T.W;  // column W - 1
+      const long long a = r[0] - r[1], b = r[1] - r[2];
+      r[2] = mad_small(r[1], q4, mad_small(b, code_factor(x1, be), mad_small(a, code_factor(x2, last >> (2 * lane)), 0)));
+    }
+    __syncwarp();
+  }
+  const Limbs KX(kx), KY(ky);
+  const long long* own = xs + kAdvPitch + lane + 1;  // (row 0, this column)
+  long long c = own[0], sb = 0, dy = 0;
+  if (MY) {
+    const long long n = own[kAdvPitch], sm = own[-kAdvPitch] - c;
+    sb = c - n;
+    dy = mad_small(c, q4, mad_small(sb, code_factor(y1, yb >> 2), mad_small(sm, code_factor(y2, yb), 0)));
+    yb >>= 2;
+  }
+  long long* orow = out + (T.fy ? (T.H - 1) * PT : 0);
+#pragma unroll 1
+  for (int j = 0; j < T.H; ++j) {
+    LimbAcc w;
+    if (MX) {
+      const unsigned b0 = xb & 3u;
+      unsigned bm = __shfl_up_sync(0xffffffffu, b0, 1);
+      const unsigned e0 = __shfl_sync(0xffffffffu, edge, j);
+      if (lane == 0) bm = e0;
+      const long long s0 = c - own[1], sm = own[-1] - c;
+      const long long d = mad_small(c, q4, mad_small(s0, code_factor(x1, b0), mad_small(sm, code_factor(x2, bm), 0)));
+      long long dn = __shfl_down_sync(0xffffffffu, d, 1);
+      const long long de = xs[(j + 1) * kAdvPitch + T.W + 2];
+      if (lane == T.W - 1) dn = de;
+      const Limbs f(d - dn);
+      w.mac(f.h, f.l, KX.h, KX.l);
+      xb >>= 2;
+    }
+    const long long n = own[kAdvPitch];
+    if (MY) {
+      const long long s1 = n - own[2 * kAdvPitch];
+      const long long d = mad_small(n, q4, mad_small(s1, code_factor(y1, yb >> 2), mad_small(sb, code_factor(y2, yb), 0)));
+      const Limbs f(dy - d);
+      w.mac(f.h, f.l, KY.h, KY.l);
+      dy = d;
+      sb = s1;
+      yb >>= 2;
+    }
+    if (in) *at(orow, lx * 8) = w.floor();
+    c = n;
+    own += kAdvPitch;
+    orow += sy;
+  }
+  return E;
+}
+
+// node constants W_k He_n(xi_k)/n! 2^61 without a node's own scale: the projection
+// sums over nodes
+constexpr long long kK0[3][5] = {
+    {1229782938247303441ll, 0ll, -614891469123651721ll, 0ll, 153722867280912930ll},
+    {512072212271327456ll, 694178496992351028ll, 214487165913345387ll, -134471359870578684ll, -99195015452660690ll},
+    {25957823211867799ll, 74160722541717783ll, 92958568648480473ll, 63806373539842544ll, 22333581812204225ll}};
+template <int cls, int n>
+__device__ __forceinline__ void k0mac(LimbAcc& s, const Limbs& x) {
+  s.mac(x.h, x.l, limb_hi(kK0[cls][n]), limb_lo(kK0[cls][n]));
+}
+
+// The projection Cbar_ab = sum lambda W W He_a He_b / (a! b!) of one family in block
+// fixed point (the transpose of the forward expansion): N = 4 (f) or 2 (g), 58-bit
+// values at the block exponent E; also a1b += sum lambda X.  cb: fields in Coeffs order.
+template <int N>
+__device__ __forceinline__ void project(const double* __restrict__ lam, const double* __restrict__ X, unsigned off,
+                                        long long PL, double (&cb)[N == 4 ? 15 : 6], double& a1b) {
+  double v[25];
+  unsigned key = 0;
+#pragma unroll
+  for (int i = 0; i < 25; ++i) {
+    v[i] = __ldg(at(lam + i * PL, off));
+    key = max(key, ((unsigned)__double2hiint(v[i]) + 0x100000u) & 0x7fffffffu);
+  }
+  const int E = (int)(key >> 20) - 1;
+  const int n0 = E < 128 ? 63 : 2;
+  long long c[N + 1], s[2][N + 1], d[2][N + 1];  // y-projections: centre node, sums and differences of the node pairs
+#pragma unroll
+  for (int p = 0; p < 5; ++p) {
+    long long h[N + 1];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) a1b = fma(v[5 * p + q], __ldg(at(X + (5 * p + q) * PL, off)), a1b);
+    const long long l0 = block_fix(v[5 * p], E, n0), l1 = block_fix(v[5 * p + 1], E, n0),
+                    l2 = block_fix(v[5 * p + 2], E, n0), l3 = block_fix(v[5 * p + 3], E, n0),
+                    l4 = block_fix(v[5 * p + 4], E, n0);
+    const Limbs z(l0), sA(l1 + l2), dA(l1 - l2), sB(l3 + l4), dB(l3 - l4);
+    LimbAcc a0, a1, a2;
+    k0mac<0, 0>(a0, z); k0mac<1, 0>(a0, sA); k0mac<2, 0>(a0, sB);
+    k0mac<1, 1>(a1, dA); k0mac<2, 1>(a1, dB);
+    k0mac<0, 2>(a2, z); k0mac<1, 2>(a2, sA); k0mac<2, 2>(a2, sB);
+    h[0] = a0.value8(); h[1] = a1.value8(); h[2] = a2.value8();
+    if constexpr (N == 4) {
+      LimbAcc a3, a4;
+      k0mac<1, 3>(a3, dA); k0mac<2, 3>(a3, dB);
+      k0mac<0, 4>(a4, z); k0mac<1, 4>(a4, sA); k0mac<2, 4>(a4, sB);
+      h[3] = a3.value8(); h[4] = a4.value8();
+    }
+#pragma unroll
+    for (int b = 0; b <= N; ++b) {
+      if (p == 0) c[b] = h[b];
+      else if (p & 1) s[p >> 1][b] = h[b];
+      else {
+        const long long t = s[(p >> 1) - 1][b];
+        s[(p >> 1) - 1][b] = t + h[b];
+        d[(p >> 1) - 1][b] = t - h[b];
+      }
+    }
+  }
+  const int sc = E - 1080;
+#define DVBM_EVEN(a, b)                                                                         \
+  [&] {                                                                                         \
+    LimbAcc t;                                                                                  \
+    k0mac<0, a>(t, Limbs(c[b])); k0mac<1, a>(t, Limbs(s[0][b])); k0mac<2, a>(t, Limbs(s[1][b])); \
+    return fix_to_double<true>(t.value8(), sc);                                                 \
+  }()
+#define DVBM_ODD(a, b)                                                \
+  [&] {                                                               \
+    LimbAcc t;                                                        \
+    k0mac<1, a>(t, Limbs(d[0][b])); k0mac<2, a>(t, Limbs(d[1][b]));   \
+    return fix_to_double<true>(t.value8(), sc);                       \
+  }()
+  if constexpr (N == 4) {
+    // f00, f10, f01, f20, f11, f02, f30, f21, f12, f03, f40, f31, f22, f13, f04
+    cb[0] = DVBM_EVEN(0, 0); cb[1] = DVBM_ODD(1, 0); cb[2] = DVBM_EVEN(0, 1); cb[3] = DVBM_EVEN(2, 0);
+    cb[4] = DVBM_ODD(1, 1); cb[5] = DVBM_EVEN(0, 2); cb[6] = DVBM_ODD(3, 0); cb[7] = DVBM_EVEN(2, 1);
+    cb[8] = DVBM_ODD(1, 2); cb[9] = DVBM_EVEN(0, 3); cb[10] = DVBM_EVEN(4, 0); cb[11] = DVBM_ODD(3, 1);
+    cb[12] = DVBM_EVEN(2, 2); cb[13] = DVBM_ODD(1, 3); cb[14] = DVBM_EVEN(0, 4);
+  } else {
+    // g00, g10, g01, g20, g11, g02
+    cb[0] = DVBM_EVEN(0, 0); cb[1] = DVBM_ODD(1, 0); cb[2] = DVBM_EVEN(0, 1);
+    cb[3] = DVBM_EVEN(2, 0); cb[4] = DVBM_ODD(1, 1); cb[5] = DVBM_EVEN(0, 2);
+  }
+#undef DVBM_EVEN
+#undef DVBM_ODD
+}
+
+// (XA / XB)^n 2^61
+constexpr long long kR61[4] = {0, 1094117591372063814ll, 519156464237355984ll, 246338635339406942ll};
+template <int n>
+__device__ __forceinline__ void rmac(LimbAcc& s, long long x) {
+  const Limbs l(x);
+  s.mac(l.h, l.l, limb_hi(kR61[n]), limb_lo(kR61[n]));
+}
+// the moment adjoints of one family as 58-bit integers times XB^(a + b) at one
+// exponent: polynomials in xi / XB, whose outer nodes are +-1
+template <int N>
+__device__ __forceinline__ int scale_moments(const double (&m)[N], long long (&Q)[N]) {
+  unsigned key = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) key = max(key, abs_key(m[i]));
+  const int E = (int)(key >> 20);
+  const int n0 = E < 128 ? 63 : 2;
+#pragma unroll
+  for (int i = 0; i < N; ++i) Q[i] = block_fix(m[i], E, n0);
+  return E;
+}
+
+// BAND: a band of a slab-decomposed grid, whose code rows beyond its edges are glo
+// and ghi ([NPOP][Nx]; NULL: the codes wrap).  moms: the moments of X, or NULL.
+// partial[4 blk + k]: the block's sums of the parameter adjoints (dt_mu, Pr, gm1,
+// epsf).
+template <int PRC>
+__global__ void __launch_bounds__(256, 2) k_adjoint_tile(const double* __restrict__ X, const double* __restrict__ Lin,
+                                                         double* Lout, double* __restrict__ partial,
+                                                         const unsigned char* __restrict__ codes,
+                                                         const double* __restrict__ moms,
+                                                         const unsigned char* __restrict__ glo,
+                                                         const unsigned char* __restrict__ ghi, Geom G, Phys P) {
+  __shared__ long long s_xs[8 * (kAdjR + 3) * kAdvPitch];
+  __shared__ int s_exp[NPOP];
+  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8;
+  const long long PL = G.plane, PT = G.pitch, cplane = (long long)G.Nx * G.Ny;
+  const double* ltile = Lin + cell_index(G, y0, x0);
+  const double* xtile = X + cell_index(G, y0, x0);
+  double* otile = Lout + cell_index(G, y0, x0);
+  const int w = __shfl_sync(0xffffffffu, (int)threadIdx.y, 0);
+  {
+    const int c0 = 25 * (w >> 2), p = 1 + (w & 3);
+    AdvTile T;
+    T.W = min(32, G.Nx - x0);
+    T.H = min(8, G.Ny - y0);
+    T.lane = threadIdx.x;
+    long long* xs = s_xs + w * ((kAdjR + 3) * kAdvPitch);
+    auto tile = [&](int pp, int q) {
+      AdvTile t = T;
+      t.fx = Lat25::backward(pp);
+      t.fy = Lat25::backward(q);
+      return t;
+    };
+    AdjointLoad V;
+    auto load = [&](int pp, int q) {
+      const int c = c0 + 5 * pp + q;
+      CodePlane C;
+      C.own = codes + c * cplane;
+      C.Nx = G.Nx;
+      C.Ny = G.Ny;
+      C.lo = glo ? glo + (long long)c * G.Nx : C.own + (cplane - G.Nx);
+      C.hi = ghi ? ghi + (long long)c * G.Nx : C.own;
+      adjoint_load(V, ltile + c * PL, PT, C, x0, y0, tile(pp, q));
+    };
+    auto out = [&](int c) { return (long long*)(otile + c * PL); };
+    load(p, 0);
+    int E = adjoint_walk<true, false>(V, [&] { load(p, 1); }, out(c0 + 5 * p), PT, tile(p, 0), P, P.kxq[p], 0, xs);
+    if (T.lane == 0) s_exp[c0 + 5 * p] = E;
+#pragma unroll 1
+    for (int q = 1; q < 5; ++q) {
+      const int c = c0 + 5 * p + q;
+      E = adjoint_walk<true, true>(V, [&] { load(q < 4 ? p : 0, q < 4 ? q + 1 : p); }, out(c), PT, tile(p, q), P,
+                                   P.kxq[p], P.kyq[q], xs);
+      if (T.lane == 0) s_exp[c] = E;
+    }
+    E = adjoint_walk<false, true>(V, [] {}, out(c0 + p), PT, tile(0, p), P, 0, P.kyq[p], xs);
+    if (T.lane == 0) s_exp[c0 + p] = E;
+    if (p == 1) {
+      if (T.lane == 0) s_exp[c0] = 0;
+      if (T.lane < T.W)
+        for (int j = 0; j < T.H; ++j) ((long long*)otile)[c0 * PL + j * PT + T.lane] = 0;
+    }
+  }
+  __syncthreads();
+  // threads beyond a ragged tile work on its last cell again and write nothing:
+  // uniform control flow keeps the planes' addresses in uniform registers
+  const bool active = x0 + (int)threadIdx.x < G.Nx && y0 + (int)threadIdx.y < G.Ny;
+  const int x = min(x0 + (int)threadIdx.x, G.Nx - 1), y = min(y0 + (int)threadIdx.y, G.Ny - 1);
+  ParamBar pb = {0, 0, 0, 0};
+  {
+    const unsigned off = ((y - y0) * (unsigned)PT + (x - x0)) * 8u;
+    double a1b = 0.0;
+    Coeffs Cb = {};
+    {
+      double cb[15], cg[6];
+      project<4>(ltile, xtile, off, PL, cb, a1b);
+      project<2>(ltile + 25 * PL, xtile + 25 * PL, off, PL, cg, a1b);
+      Cb.f00 = cb[0]; Cb.f10 = cb[1]; Cb.f01 = cb[2]; Cb.f20 = cb[3]; Cb.f11 = cb[4]; Cb.f02 = cb[5];
+      Cb.f30 = cb[6]; Cb.f21 = cb[7]; Cb.f12 = cb[8]; Cb.f03 = cb[9]; Cb.f40 = cb[10]; Cb.f31 = cb[11];
+      Cb.f22 = cb[12]; Cb.f13 = cb[13]; Cb.f04 = cb[14];
+      Cb.g00 = cg[0]; Cb.g10 = cg[1]; Cb.g01 = cg[2]; Cb.g20 = cg[3]; Cb.g11 = cg[4]; Cb.g02 = cg[5];
+    }
+    Moments m;
+    if (moms) {
+      const long long ci = (long long)y * G.Nx + x;
+      m.m00 = moms[0 * cplane + ci]; m.m10 = moms[1 * cplane + ci]; m.m01 = moms[2 * cplane + ci];
+      m.m20 = moms[3 * cplane + ci]; m.m11 = moms[4 * cplane + ci]; m.m02 = moms[5 * cplane + ci];
+      m.m30 = moms[6 * cplane + ci]; m.m21 = moms[7 * cplane + ci]; m.m12 = moms[8 * cplane + ci];
+      m.m03 = moms[9 * cplane + ci]; m.g00 = moms[10 * cplane + ci]; m.g10 = moms[11 * cplane + ci];
+      m.g01 = moms[12 * cplane + ci];
+    } else {
+      m = moments_fix<double>(xtile, off, PL);
+    }
+    Moments mb = {};
+    const double a1 = collision_coeffs_rev<PRC>(m, P, Cb, a1b, mb, pb);
+    // the pullback sum_j mbar_j dm_j/dX of population (p, q) is the polynomial
+    // sum mbar_ab xi_p^a xi_q^b, in fixed point with the flux sum taken off
+    const double mf[10] = {mb.m00, XB * mb.m10, XB * mb.m01, (XB * XB) * mb.m20, (XB * XB) * mb.m11, (XB * XB) * mb.m02,
+                           (XB * XB * XB) * mb.m30, (XB * XB * XB) * mb.m21, (XB * XB * XB) * mb.m12,
+                           (XB * XB * XB) * mb.m03};
+    const double mg[3] = {mb.g00, XB * mb.g10, XB * mb.g01};
+    long long F[10], H[3];
+    const int Ef = scale_moments(mf, F), Eg = scale_moments(mg, H);
+    // even and odd parts in x of the inner node pair
+    LimbAcc t0, u0, t1, u1, u2, v0;
+    rmac<2>(t0, F[3]);
+    rmac<1>(u0, F[1]); rmac<3>(u0, F[6]);
+    rmac<2>(t1, F[7]);
+    rmac<1>(u1, F[4]);
+    rmac<1>(u2, F[8]);
+    rmac<1>(v0, H[1]);
+    const long long eA0 = F[0] + t0.value8(), oA0 = u0.value8(), eA1 = F[2] + t1.value8(), oA1 = u1.value8(),
+                    oA2 = u2.value8(), gA = v0.value8();
+#pragma unroll 1
+    for (int p = 0; p < 5; ++p) {
+      // y-polynomial of this x-node
+      long long b0, b1, b2, g0;
+      if (p == 0) {
+        b0 = F[0]; b1 = F[2]; b2 = F[5]; g0 = H[0];
+      } else {
+        const bool inner = p <= 2;
+        const long long e0 = inner ? eA0 : F[0] + F[3], o0 = inner ? oA0 : F[1] + F[6], e1 = inner ? eA1 : F[2] + F[7],
+                        o1 = inner ? oA1 : F[4], o2 = inner ? oA2 : F[8], og = inner ? gA : H[1];
+        const bool neg = (p & 1) == 0;
+        b0 = neg ? e0 - o0 : e0 + o0;
+        b1 = neg ? e1 - o1 : e1 + o1;
+        b2 = neg ? F[5] - o2 : F[5] + o2;
+        g0 = neg ? H[0] - og : H[0] + og;
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const double* lp = ltile + (25 * k + 5 * p) * PL;
+        double* op = otile + (25 * k + 5 * p) * PL;
+        double lv[5];
+        long long W[5], t[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          lv[q] = __ldg(at(lp + q * PL, off));
+          W[q] = active ? *at((const long long*)op + q * PL, off) : 0ll;
+        }
+        if (k == 0) {
+          LimbAcc ev, od;
+          rmac<2>(ev, b2);
+          rmac<1>(od, b1); rmac<3>(od, F[9]);
+          const long long ea = b0 + ev.value8(), oa = od.value8(), eb = b0 + b2, ob = b1 + F[9];
+          t[0] = b0; t[1] = ea + oa; t[2] = ea - oa; t[3] = eb + ob; t[4] = eb - ob;
+        } else {
+          LimbAcc od;
+          rmac<1>(od, H[2]);
+          const long long oa = od.value8();
+          t[0] = g0; t[1] = g0 + oa; t[2] = g0 - oa; t[3] = g0 + H[2]; t[4] = g0 - H[2];
+        }
+        const int st = (k == 0 ? Ef : Eg) - 1;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+          const double v = collide_advect(a1, lv[q], t[q], st, W[q], s_exp[25 * k + 5 * p + q] + 3);
+          if (active) *at(op + q * PL, off) = v;
+        }
+      }
+    }
+  }
+  // block reduction of the parameter adjoints (fixed order)
+  __syncthreads();
+  double* sh = (double*)s_xs;
+  const int t = threadIdx.y * 32 + threadIdx.x;
+  if (!active) pb = {0, 0, 0, 0};
+  sh[t] = pb.dt_mu; sh[256 + t] = pb.Pr; sh[512 + t] = pb.gm1; sh[768 + t] = pb.epsf;
+  __syncthreads();
+  for (int n = 128; n > 0; n >>= 1) {
+    if (t < n)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) sh[256 * k + t] += sh[256 * k + t + n];
+    __syncthreads();
+  }
+  if (t == 0) {
+    const int b = blockIdx.y * gridDim.x + blockIdx.x;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) partial[4 * b + k] = sh[256 * k];
+  }
+}
+
 // ------------------------------------------------------------------- kernels
-// One adjoint step in two launches.
+// One adjoint step in two launches, with the branches derived from the states: a
+// general beta, or no memory for the codes.
 // k_adjoint_local: Lout = a1 Lin + sum_j mbar_j dm_j/dX (collision part) at
 // state X; per-block sums of the parameter adjoints (dt_mu, Pr, gm1, epsf)
 // into partial[blk*4 + k].
-// MOMS: the moments of X come from the recompute step (moms[k][y][x], the
-// same sums in the same order) instead of being summed again here.
-template <int PRC, bool MOMS>
+template <int PRC>
 __global__ void __launch_bounds__(256, 2) k_adjoint_local(const double* __restrict__ X, const double* __restrict__ Lin,
                                                        double* __restrict__ Lout, double* __restrict__ partial,
-                                                       const double* __restrict__ moms, Geom G, Phys P) {
+                                                       Geom G, Phys P) {
   const int x = blockIdx.x * 32 + threadIdx.x;
   const int y = blockIdx.y * 8 + threadIdx.y;
   const bool active = x < G.Nx && y < G.Ny;
@@ -566,7 +1002,7 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_local(const double* __restri
         lf[q] = __ldg(ls + (5 * p + q) * PL); lg[q] = __ldg(ls + (25 + 5 * p + q) * PL); \
         a1b = fma(lf[q], f[q], fma(lg[q], g[q], a1b));                                \
       }                                                                                \
-      if (!MOMS) accumulate_moments<p>(m, f, g);                                       \
+      accumulate_moments<p>(m, f, g);                                                  \
       accumulate_projection_fix<p>(cb, lf, lg, ELf, ELg);
       DVBM_ADJ_A(0) DVBM_ADJ_A(1) DVBM_ADJ_A(2) DVBM_ADJ_A(3) DVBM_ADJ_A(4)
 #undef DVBM_ADJ_A
@@ -580,14 +1016,6 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_local(const double* __restri
       Cb.f22 = cv(okf, cb[12 * 256], sf); Cb.f13 = cv(okf, cb[13 * 256], sf); Cb.f04 = cv(okf, cb[14 * 256], sf);
       Cb.g00 = cv(okg, cb[15 * 256], sg); Cb.g10 = cv(okg, cb[16 * 256], sg); Cb.g01 = cv(okg, cb[17 * 256], sg);
       Cb.g20 = cv(okg, cb[18 * 256], sg); Cb.g11 = cv(okg, cb[19 * 256], sg); Cb.g02 = cv(okg, cb[20 * 256], sg);
-    }
-    if (MOMS) {
-      const long long cp = (long long)G.Nx * G.Ny, ci = (long long)y * G.Nx + x;
-      m.m00 = moms[0 * cp + ci]; m.m10 = moms[1 * cp + ci]; m.m01 = moms[2 * cp + ci];
-      m.m20 = moms[3 * cp + ci]; m.m11 = moms[4 * cp + ci]; m.m02 = moms[5 * cp + ci];
-      m.m30 = moms[6 * cp + ci]; m.m21 = moms[7 * cp + ci]; m.m12 = moms[8 * cp + ci];
-      m.m03 = moms[9 * cp + ci]; m.g00 = moms[10 * cp + ci]; m.g10 = moms[11 * cp + ci];
-      m.g01 = moms[12 * cp + ci];
     }
     Moments mb = {};
     const double a1 = collision_coeffs_rev<PRC>(m, P, Cb, a1b, mb, pb);
@@ -622,18 +1050,10 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_local(const double* __restri
 }
 
 // k_adjoint_adv: Lout += -(dt/dx) v_x sum_c' Lin(c') dF_x(c')/dX(c) - (same in y),
-// one thread per (cell, population); blockIdx.z = population.  CODED: the
-// minmod branches come from the codes the recomputed forward step recorded
-// (periodic neighbours wrap), so X is not read at all.  A band of a
-// slab-decomposed grid passes the neighbouring bands' code rows next to its
-// edges (glo: the row below y = 0, ghi: the row above y = Ny - 1; [NPOP][Nx]
-// each) instead of wrapping in y (BAND).
-template <bool RAT, bool CODED, bool BAND = false>
+// one thread per (cell, population); blockIdx.z = population.
+template <bool RAT>
 __global__ void __launch_bounds__(256) k_adjoint_adv(const double* __restrict__ X, const double* __restrict__ Lin,
-                                                     double* __restrict__ Lout,
-                                                     const unsigned char* __restrict__ codes, Geom G, Phys P,
-                                                     const unsigned char* __restrict__ glo = nullptr,
-                                                     const unsigned char* __restrict__ ghi = nullptr) {
+                                                     double* __restrict__ Lout, Geom G, Phys P) {
   const int x = blockIdx.x * 32 + threadIdx.x;
   const int y = blockIdx.y * 8 + threadIdx.y;
   const int c = blockIdx.z;
@@ -645,23 +1065,7 @@ __global__ void __launch_bounds__(256) k_adjoint_adv(const double* __restrict__ 
   const double* xc = X + off;
   const double* lc = Lin + off;
   double v = Lout[off];
-  if constexpr (CODED) {
-    const unsigned char* cp = codes + (long long)c * G.Nx * G.Ny;
-    const long long row = (long long)y * G.Nx;
-    if (sx != 0) {
-      const int xm = x == 0 ? G.Nx - 1 : x - 1, xp = x == G.Nx - 1 ? 0 : x + 1;
-      const int bm = __ldg(cp + row + xm) & 3, b0 = __ldg(cp + row + x) & 3, bp = __ldg(cp + row + xp) & 3;
-      v = fma(-P.kxr[pn], adjoint_combine_rat(lc, 1, bm, b0, bp, P.lp, P.lq, sx), v);
-    }
-    if (sy != 0) {
-      const int ym = y == 0 ? G.Ny - 1 : y - 1, yp = y == G.Ny - 1 ? 0 : y + 1;
-      const unsigned char* pm = (BAND && y == 0 && glo) ? glo + (long long)c * G.Nx + x : cp + (long long)ym * G.Nx + x;
-      const unsigned char* pp =
-          (BAND && y == G.Ny - 1 && ghi) ? ghi + (long long)c * G.Nx + x : cp + (long long)yp * G.Nx + x;
-      const int bm = (__ldg(pm) >> 2) & 3, b0 = (__ldg(cp + row + x) >> 2) & 3, bp = (__ldg(pp) >> 2) & 3;
-      v = fma(-P.kyr[qn], adjoint_combine_rat(lc, G.pitch, bm, b0, bp, P.lp, P.lq, sy), v);
-    }
-  } else if constexpr (RAT) {
+  if constexpr (RAT) {
     if (sx != 0) v = fma(-P.kxr[pn], advection_adjoint_rat(xc, lc, 1, P.lp, P.lq, sx), v);
     if (sy != 0) v = fma(-P.kyr[qn], advection_adjoint_rat(xc, lc, G.pitch, P.lp, P.lq, sy), v);
   } else {
@@ -787,23 +1191,20 @@ cudaError_t launch_adjoint_step(const double* X, const double* Lin, double* Lout
                                 const unsigned char* codes, const double* moms, const Geom& G, const Phys& P,
                                 cudaStream_t st, const unsigned char* glo, const unsigned char* ghi) {
   dim3 block(32, 8), grid((G.Nx + 31) / 32, (G.Ny + 7) / 8);
-  if (moms) {
-    if (P.prc < 0) k_adjoint_local<-1, true><<<grid, block, 0, st>>>(X, Lin, Lout, partial, moms, G, P);
-    else if (P.prc > 0) k_adjoint_local<1, true><<<grid, block, 0, st>>>(X, Lin, Lout, partial, moms, G, P);
-    else k_adjoint_local<0, true><<<grid, block, 0, st>>>(X, Lin, Lout, partial, moms, G, P);
-  } else {
-    if (P.prc < 0) k_adjoint_local<-1, false><<<grid, block, 0, st>>>(X, Lin, Lout, partial, nullptr, G, P);
-    else if (P.prc > 0) k_adjoint_local<1, false><<<grid, block, 0, st>>>(X, Lin, Lout, partial, nullptr, G, P);
-    else k_adjoint_local<0, false><<<grid, block, 0, st>>>(X, Lin, Lout, partial, nullptr, G, P);
+  if (codes) {
+    if (P.prc < 0) k_adjoint_tile<-1><<<grid, block, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
+    else if (P.prc > 0) k_adjoint_tile<1><<<grid, block, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
+    else k_adjoint_tile<0><<<grid, block, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
+    return cudaGetLastError();
   }
+  if (P.prc < 0) k_adjoint_local<-1><<<grid, block, 0, st>>>(X, Lin, Lout, partial, G, P);
+  else if (P.prc > 0) k_adjoint_local<1><<<grid, block, 0, st>>>(X, Lin, Lout, partial, G, P);
+  else k_adjoint_local<0><<<grid, block, 0, st>>>(X, Lin, Lout, partial, G, P);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  dim3 grid3(grid.x, grid.y, NPOP);
-  if (P.lq > 0 && codes && (glo || ghi))
-    k_adjoint_adv<true, true, true><<<grid3, block, 0, st>>>(X, Lin, Lout, codes, G, P, glo, ghi);
-  else if (P.lq > 0 && codes) k_adjoint_adv<true, true><<<grid3, block, 0, st>>>(X, Lin, Lout, codes, G, P);
-  else if (P.lq > 0) k_adjoint_adv<true, false><<<grid3, block, 0, st>>>(X, Lin, Lout, nullptr, G, P);
-  else k_adjoint_adv<false, false><<<grid3, block, 0, st>>>(X, Lin, Lout, nullptr, G, P);
+  const dim3 grid3(grid.x, grid.y, NPOP);
+  if (P.lq > 0) k_adjoint_adv<true><<<grid3, block, 0, st>>>(X, Lin, Lout, G, P);
+  else k_adjoint_adv<false><<<grid3, block, 0, st>>>(X, Lin, Lout, G, P);
   return cudaGetLastError();
 }
 
