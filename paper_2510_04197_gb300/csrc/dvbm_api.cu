@@ -45,6 +45,7 @@ struct dvbm_ctx {
   std::vector<void*> pool;             // spare state buffers
   double* init_fields = nullptr;       // rho, ux, uy, T of the recorded dvbm_init
   double* stage = nullptr;             // 4 Nx Ny doubles staging host fields (allocated on first use)
+  cudaEvent_t ev = nullptr;            // marks the stream's end for host waits
   std::vector<void*> in_flight;        // temporaries of calls that timed out, freed by dvbm_destroy
   size_t state_bytes_dev = 0;
   // slab decomposition along y: sides whose ghost rows come from dvbm_halo_unpack
@@ -272,7 +273,8 @@ extern "C" dvbm_status dvbm_create(dvbm_ctx** out, int lattice, int Nx, int Ny, 
   }
   c->nred = 4 * sms;
   if (cudaMalloc(&c->flag, sizeof(unsigned int)) != cudaSuccess ||
-      cudaMalloc(&c->partial, sizeof(double) * 6 * c->nred) != cudaSuccess) {
+      cudaMalloc(&c->partial, sizeof(double) * 6 * c->nred) != cudaSuccess ||
+      cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     dvbm_destroy(c);
     return fail(nullptr, DVBM_ENOMEM, "cudaMalloc of work buffers failed");
@@ -290,30 +292,28 @@ extern "C" dvbm_status dvbm_create(dvbm_ctx** out, int lattice, int Nx, int Ny, 
   return DVBM_OK;
 }
 
-// stream-ordered wait with a host-side time limit
+// Stream-ordered wait with a host-side time limit.  The first two milliseconds
+// are polled (a sleep of 50 us lasts about 100: longer than a step of a small
+// grid), longer waits sleep between polls.
 static dvbm_status wait_stream(dvbm_ctx* c) {
-  cudaEvent_t ev;
-  CUDA_TRY(c, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-  cudaError_t e = cudaEventRecord(ev, c->stream);
-  if (e != cudaSuccess) { cudaEventDestroy(ev); return fail(c, DVBM_ECUDA, "cudaEventRecord: %s", cudaGetErrorString(e)); }
+  CUDA_TRY(c, cudaEventRecord(c->ev, c->stream));
   const auto t0 = std::chrono::steady_clock::now();
-  int spins = 0;
-  for (;;) {
-    e = cudaEventQuery(ev);
-    if (e == cudaSuccess) break;
-    if (e != cudaErrorNotReady) { cudaEventDestroy(ev); return fail(c, DVBM_ECUDA, "stream error: %s", cudaGetErrorString(e)); }
+  for (int spins = 0;; ++spins) {
+    const cudaError_t e = cudaEventQuery(c->ev);
+    if (e == cudaSuccess) return DVBM_OK;
+    if (e != cudaErrorNotReady) return fail(c, DVBM_ECUDA, "stream error: %s", cudaGetErrorString(e));
     const double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-    if (el > c->opts.timeout_s) { cudaEventDestroy(ev); return fail(c, DVBM_ETIMEOUT, "stream did not finish within %g s", c->opts.timeout_s); }
-    if (++spins > 64) std::this_thread::sleep_for(std::chrono::microseconds(50));
+    if (el > c->opts.timeout_s) return fail(c, DVBM_ETIMEOUT, "stream did not finish within %g s", c->opts.timeout_s);
+    if (el > 2e-3) std::this_thread::sleep_for(std::chrono::microseconds(20));
+    else if (spins > 64) std::this_thread::yield();
   }
-  cudaEventDestroy(ev);
-  return DVBM_OK;
 }
 
 // Device -> host copy under the time limit. A copy into pageable host memory returns only once
 // it has completed, i.e. once the stream has run everything queued before it, so a hung or slow
 // stream would block inside the copy, past timeout_s. The queued work is therefore waited for
-// first, under the limit; the copy then finds the stream idle.
+// first, under the limit; the copy then finds the stream idle.  Into pinned memory the copy is
+// asynchronous, so it is waited for too.
 static dvbm_status drain_then_copy(dvbm_ctx* c, void* dst, const void* src, size_t bytes) {
   dvbm_status s = wait_stream(c);
   if (s != DVBM_OK) return s;
@@ -1055,6 +1055,7 @@ extern "C" void dvbm_destroy(dvbm_ctx* c) {
   for (void* p : c->pool) cudaFree(p);
   if (c->init_fields) cudaFree(c->init_fields);
   if (c->stage) cudaFree(c->stage);
+  if (c->ev) cudaEventDestroy(c->ev);
   for (void* p : c->in_flight) cudaFree(p);
   delete c;
 }
