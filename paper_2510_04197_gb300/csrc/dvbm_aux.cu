@@ -99,43 +99,68 @@ __global__ void k_ghost(S* __restrict__ buf, Geom G, BCDev bc) {
 
 // Isothermal no-slip walls: F_G = F^eq(rho_B, 2 u_W - u_B, 2 T_W - T_B) + (F_B - F^eq(B)),
 // i.e. F_B plus the expansion of the difference of the two equilibria's
-// coefficients, in the step kernels' fixed point.  The kernel's work is small
-// and all latency, so a ghost cell has eight threads, which all form the
-// coefficients and share the populations (units of an x-node's f or g): one
-// thread a cell took 33 us of a 55 us step at 4 x 256, this takes 21.
+// coefficients, in the step kernels' fixed point.  The work is small and all
+// latency, FP64 chains first (one FP64 warp instruction occupies its scheduler's
+// pipe for 64 cycles), so a ghost cell has one thread in each of the block's
+// eight warps: warps 0 and 1 sum f and g, then form the equilibria of the mirror
+// cell and of the ghost, then bring the differences to fixed point (f, g); all
+// share the populations (units of an x-node's f or g).  At 4 x 256 one thread a
+// cell took 33 us of a 55 us step; this takes 11.
 template <class L, class S>
 __global__ void __launch_bounds__(kCta, 2) k_wall(S* __restrict__ buf, Geom G, Phys P, Macro M, BCDev bc) {
   typedef typename L::Tile LT;
-  constexpr int NQ = LT::NQ, NF = NQ * NQ;
-  __shared__ long long s_buf[LT::FIELDS * kCta];
-  const int side = blockIdx.y;
+  constexpr int NQ = LT::NQ, NF = NQ * NQ, N = LT::FIELDS;
+  __shared__ long long s_fix[N * 32];
+  __shared__ double s_m[LT::MOMS][32], s_eq[2][N][32];
+  __shared__ int s_E[2][32];
+  const int side = blockIdx.y, lane = threadIdx.x, w = threadIdx.y;
   if (bc.kind[side] != 2) return;
   const int len = side < 2 ? G.Ny : G.Nx;
-  const int t = blockIdx.x * 32 + threadIdx.x;
-  if (t >= 2 * len) return;
+  const int t = min((int)blockIdx.x * 32 + lane, 2 * len - 1);  // surplus lanes repeat the last cell
   int gx, gy, bx, by;
   ghost_cells(side, 2, 1 + t / len, t % len, G, gx, gy, bx, by);
   const long long PL = G.plane;
   S* g = buf + cell_index(G, gy, gx);
   const S* b = buf + cell_index(G, by, bx);
-  long long* slot = s_buf + threadIdx.y * 32 + threadIdx.x;
-  int Ef, Eg;
-  {
-    const CellState c = L::template state<S>(b, PL, P, M);
-    auto D = L::equilibrium(c.rho, 2.0 * bc.uw[side][0] - c.ux, 2.0 * bc.uw[side][1] - c.uy, 2.0 * bc.Tw[side] - c.T, P, M);
-    L::subtract(D, L::equilibrium(c.rho, c.ux, c.uy, c.T, P, M));
-    LT::to_smem(D, slot, Ef, Eg);
+  if (w < 2) {
+    typename LT::Mom m;
+    if (w == 0) L::template sum_f<S>(b, PL, m, P);
+    else L::template sum_g<S>(b, PL, m, P);
+    LT::put(m, w, [&](int k, double v) { s_m[k][lane] = v; });
   }
-  const FixView X{slot};
+  __syncthreads();
+  if (w < 2) {
+    typename LT::Mom m;
+    LT::get(m, [&](int k) { return s_m[k][lane]; });
+    const CellState c = L::state_of(m, P, M);
+    const auto C = w == 0 ? L::equilibrium(c.rho, c.ux, c.uy, c.T, P, M)
+                          : L::equilibrium(c.rho, 2.0 * bc.uw[side][0] - c.ux, 2.0 * bc.uw[side][1] - c.uy,
+                                           2.0 * bc.Tw[side] - c.T, P, M);
+    LT::fields(C, [&](int k, double v) { s_eq[w][k][lane] = v; });
+  }
+  __syncthreads();
+  if (w == 0) {
+    double d[LT::GFIELD];
+#pragma unroll
+    for (int k = 0; k < LT::GFIELD; ++k) d[k] = s_eq[1][k][lane] - s_eq[0][k][lane];
+    fields_to_smem<LT::GFIELD, 32>(d, s_fix + lane, s_E[0][lane]);
+  } else if (w == 1) {
+    double d[N - LT::GFIELD];
+#pragma unroll
+    for (int k = 0; k < N - LT::GFIELD; ++k) d[k] = s_eq[1][LT::GFIELD + k][lane] - s_eq[0][LT::GFIELD + k][lane];
+    fields_to_smem<N - LT::GFIELD, 32>(d, s_fix + 32 * LT::GFIELD + lane, s_E[1][lane]);
+  }
+  __syncthreads();
+  const FixViewOf<32> X{s_fix + lane};
 #pragma unroll 1
-  for (int u = threadIdx.y; u < 2 * NQ; u += 8) {
+  for (int u = w; u < 2 * NQ; u += 8) {
     const int p = u >> 1, k = u & 1;
     typename LT::NodeK K;
     LT::load_k(p, K);
     long long v[NQ];
     if (k == 0) LT::target_f(X, K, v);
     else LT::target_g(X, K, v);
-    const int sc = (k == 0 ? Ef : Eg) - 1079 - LT::kdp(p);
+    const int sc = s_E[k][lane] - 1079 - LT::kdp(p);
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const long long o = (NF * k + NQ * p + q) * PL;

@@ -467,83 +467,94 @@ __device__ __forceinline__ long long pair_sum(long long b, long long a) {
 }
 
 template <class S>
+struct FixKind {
+  static constexpr int kBias = sizeof(S) == 8 ? 1080 : 184;
+  static constexpr int kExpBits = sizeof(S) == 8 ? 20 : 23;
+  static constexpr unsigned kInf = sizeof(S) == 8 ? 0x7ff00000u : 0x7f800000u;
+  static constexpr int kTiny = sizeof(S) == 8 ? 128 : 0;  // blocks below this exponent count as zero
+};
+template <class S>
+__device__ __forceinline__ void moments_fix_f(const S* __restrict__ s, unsigned off, long long PL, Moments& m) {
+  typedef FixKind<S> K;
+  S v[25];
+  unsigned key = 0;
+#pragma unroll
+  for (int i = 0; i < 25; ++i) {
+    v[i] = __ldg(at(s + i * PL, off));
+    key = max(key, abs_key(v[i]));
+  }
+  const int E = (int)(key >> K::kExpBits);
+  const int n0 = E < K::kTiny ? 63 : 2;
+  long long M0[5], M1[5], M2[5], M3s = 0;  // y-sums of each x-node, M1, M2, M3 times 1/16, 1/64, 1/128
+#pragma unroll
+  for (int p = 0; p < 5; ++p) {
+    const long long x0 = block_fix(v[5 * p], E, n0), x1 = block_fix(v[5 * p + 1], E, n0),
+                    x2 = block_fix(v[5 * p + 2], E, n0), x3 = block_fix(v[5 * p + 3], E, n0),
+                    x4 = block_fix(v[5 * p + 4], E, n0);
+    const long long sA = x1 + x2, dA = x1 - x2, sB = x3 + x4, dB = x3 - x4;
+    M0[p] = x0 + sA + sB;
+    M1[p] = pair_sum<1>(dB, dA);
+    M2[p] = pair_sum<2>(sB, sA);
+    M3s += pair_sum<3>(dB, dA);
+  }
+  const long long a0 = M0[1] + M0[2], b0 = M0[3] + M0[4], c0 = M0[1] - M0[2], d0 = M0[3] - M0[4];
+  // second factors: the first left four spare bits
+  const long long a1 = M1[1] + M1[2], b1 = M1[3] + M1[4], c1 = M1[1] - M1[2], d1 = M1[3] - M1[4];
+  const long long a2 = M2[1] + M2[2], b2 = M2[3] + M2[4], c2 = M2[1] - M2[2], d2 = M2[3] - M2[4];
+  const int sc = E - K::kBias;
+  m.m00 = fix_to_double<true>(M0[0] + a0 + b0, sc);
+  m.m01 = fix_to_double<true>(M1[0] + a1 + b1, sc + 4);
+  m.m02 = fix_to_double<true>(M2[0] + a2 + b2, sc + 6);
+  m.m03 = fix_to_double<true>(M3s, sc + 7);
+  m.m10 = fix_to_double<true>(pair_sum<1>(d0, c0), sc + 4);
+  m.m20 = fix_to_double<true>(pair_sum<2>(b0, a0), sc + 6);
+  m.m30 = fix_to_double<true>(pair_sum<3>(d0, c0), sc + 7);
+  m.m11 = fix_to_double<true>(pair_sum<1>(d1 << 4, c1 << 4), sc + 4);
+  m.m21 = fix_to_double<true>(pair_sum<2>(b1 << 4, a1 << 4), sc + 6);
+  m.m12 = fix_to_double<true>(pair_sum<1>(d2 << 4, c2 << 4), sc + 6);
+  if (key >= K::kInf) m.m00 = __longlong_as_double(0x7ff8000000000000ll);
+}
+template <class S>
+__device__ __forceinline__ void moments_fix_g(const S* __restrict__ s, unsigned off, long long PL, Moments& m) {
+  typedef FixKind<S> K;
+  S v[25];
+  unsigned key = 0;
+#pragma unroll
+  for (int i = 0; i < 25; ++i) {
+    v[i] = __ldg(at(s + (25 + i) * PL, off));
+    key = max(key, abs_key(v[i]));
+  }
+  const int E = (int)(key >> K::kExpBits);
+  const int n0 = E < K::kTiny ? 63 : 2;
+  long long N0[5], N1s = 0;
+#pragma unroll
+  for (int p = 0; p < 5; ++p) {
+    const long long x0 = block_fix(v[5 * p], E, n0), x1 = block_fix(v[5 * p + 1], E, n0),
+                    x2 = block_fix(v[5 * p + 2], E, n0), x3 = block_fix(v[5 * p + 3], E, n0),
+                    x4 = block_fix(v[5 * p + 4], E, n0);
+    N0[p] = x0 + (x1 + x2) + (x3 + x4);
+    N1s += pair_sum<1>(x3 - x4, x1 - x2);
+  }
+  const int sc = E - K::kBias;
+  m.g00 = fix_to_double<true>(N0[0] + (N0[1] + N0[2]) + (N0[3] + N0[4]), sc);
+  m.g01 = fix_to_double<true>(N1s, sc + 4);
+  m.g10 = fix_to_double<true>(pair_sum<1>(N0[3] - N0[4], N0[1] - N0[2]), sc + 4);
+  if (key >= K::kInf) m.g00 = __longlong_as_double(0x7ff8000000000000ll);
+}
+template <class S>
 __device__ __forceinline__ Moments moments_fix(const S* __restrict__ s, unsigned off, long long PL) {
-  constexpr int kBias = sizeof(S) == 8 ? 1080 : 184;
-  constexpr int kExpBits = sizeof(S) == 8 ? 20 : 23;
-  constexpr unsigned kInf = sizeof(S) == 8 ? 0x7ff00000u : 0x7f800000u;
-  constexpr int kTiny = sizeof(S) == 8 ? 128 : 0;  // blocks below this exponent count as zero
   Moments m;
-  const double nan = __longlong_as_double(0x7ff8000000000000ll);
-  {
-    S v[25];
-    unsigned key = 0;
-#pragma unroll
-    for (int i = 0; i < 25; ++i) {
-      v[i] = __ldg(at(s + i * PL, off));
-      key = max(key, abs_key(v[i]));
-    }
-    const int E = (int)(key >> kExpBits);
-    const int n0 = E < kTiny ? 63 : 2;
-    long long M0[5], M1[5], M2[5], M3s = 0;  // y-sums of each x-node, M1, M2, M3 times 1/16, 1/64, 1/128
-#pragma unroll
-    for (int p = 0; p < 5; ++p) {
-      const long long x0 = block_fix(v[5 * p], E, n0), x1 = block_fix(v[5 * p + 1], E, n0),
-                      x2 = block_fix(v[5 * p + 2], E, n0), x3 = block_fix(v[5 * p + 3], E, n0),
-                      x4 = block_fix(v[5 * p + 4], E, n0);
-      const long long sA = x1 + x2, dA = x1 - x2, sB = x3 + x4, dB = x3 - x4;
-      M0[p] = x0 + sA + sB;
-      M1[p] = pair_sum<1>(dB, dA);
-      M2[p] = pair_sum<2>(sB, sA);
-      M3s += pair_sum<3>(dB, dA);
-    }
-    const long long a0 = M0[1] + M0[2], b0 = M0[3] + M0[4], c0 = M0[1] - M0[2], d0 = M0[3] - M0[4];
-    // second factors: the first left four spare bits
-    const long long a1 = M1[1] + M1[2], b1 = M1[3] + M1[4], c1 = M1[1] - M1[2], d1 = M1[3] - M1[4];
-    const long long a2 = M2[1] + M2[2], b2 = M2[3] + M2[4], c2 = M2[1] - M2[2], d2 = M2[3] - M2[4];
-    const int sc = E - kBias;
-    m.m00 = fix_to_double<true>(M0[0] + a0 + b0, sc);
-    m.m01 = fix_to_double<true>(M1[0] + a1 + b1, sc + 4);
-    m.m02 = fix_to_double<true>(M2[0] + a2 + b2, sc + 6);
-    m.m03 = fix_to_double<true>(M3s, sc + 7);
-    m.m10 = fix_to_double<true>(pair_sum<1>(d0, c0), sc + 4);
-    m.m20 = fix_to_double<true>(pair_sum<2>(b0, a0), sc + 6);
-    m.m30 = fix_to_double<true>(pair_sum<3>(d0, c0), sc + 7);
-    m.m11 = fix_to_double<true>(pair_sum<1>(d1 << 4, c1 << 4), sc + 4);
-    m.m21 = fix_to_double<true>(pair_sum<2>(b1 << 4, a1 << 4), sc + 6);
-    m.m12 = fix_to_double<true>(pair_sum<1>(d2 << 4, c2 << 4), sc + 6);
-    if (key >= kInf) m.m00 = nan;
-  }
-  {
-    S v[25];
-    unsigned key = 0;
-#pragma unroll
-    for (int i = 0; i < 25; ++i) {
-      v[i] = __ldg(at(s + (25 + i) * PL, off));
-      key = max(key, abs_key(v[i]));
-    }
-    const int E = (int)(key >> kExpBits);
-    const int n0 = E < kTiny ? 63 : 2;
-    long long N0[5], N1s = 0;
-#pragma unroll
-    for (int p = 0; p < 5; ++p) {
-      const long long x0 = block_fix(v[5 * p], E, n0), x1 = block_fix(v[5 * p + 1], E, n0),
-                      x2 = block_fix(v[5 * p + 2], E, n0), x3 = block_fix(v[5 * p + 3], E, n0),
-                      x4 = block_fix(v[5 * p + 4], E, n0);
-      N0[p] = x0 + (x1 + x2) + (x3 + x4);
-      N1s += pair_sum<1>(x3 - x4, x1 - x2);
-    }
-    const int sc = E - kBias;
-    m.g00 = fix_to_double<true>(N0[0] + (N0[1] + N0[2]) + (N0[3] + N0[4]), sc);
-    m.g01 = fix_to_double<true>(N1s, sc + 4);
-    m.g10 = fix_to_double<true>(pair_sum<1>(N0[3] - N0[4], N0[1] - N0[2]), sc + 4);
-    if (key >= kInf) m.g00 = nan;
-  }
+  moments_fix_f<S>(s, off, PL, m);
+  moments_fix_g<S>(s, off, PL, m);
   return m;
 }
 // moments of the FP32-deviation reference populations w rho0 (f) and w G0 (g):
 // sum w = 1, sum w xi^2 = 1 per axis, odd moments vanish
-__device__ __forceinline__ void add_reference(Moments& m, const Phys& P) {
+__device__ __forceinline__ void add_reference_f(Moments& m, const Phys& P) {
   m.m00 += P.fref0; m.m20 += P.fref0; m.m02 += P.fref0;
+}
+__device__ __forceinline__ void add_reference(Moments& m, const Phys& P) {
+  add_reference_f(m, P);
   m.g00 += P.gref0;
 }
 
@@ -792,14 +803,16 @@ static __constant__ int c_kf[5][5][2] = {
 // t at [k * kCta + t] (consecutive threads, consecutive words; registers would
 // hold 42 words across the node loop).  Field order f00, f10, f01, f20, f11,
 // f02, f30, f21, f12, f03, f40, f31, f22, f13, f04, g00, g10, g01, g20, g11, g02.
-struct FixView {
+template <int STRIDE>
+struct FixViewOf {
   const long long* b;
   __device__ __forceinline__ void mac(LimbAcc& s, int field, const int (&k)[2]) const {
-    const long long x = b[field * kCta];
+    const long long x = b[field * STRIDE];
     s.mac((int)(x >> 32), (int)x, k[0], k[1]);
   }
 };
-template <int N>
+typedef FixViewOf<kCta> FixView;
+template <int N, int STRIDE = kCta>
 __device__ __forceinline__ void fields_to_smem(const double (&f)[N], long long* b, int& E) {
   unsigned key = 0;
 #pragma unroll
@@ -807,18 +820,11 @@ __device__ __forceinline__ void fields_to_smem(const double (&f)[N], long long* 
   E = (int)(key >> 20);
   const int n0 = E < 128 ? 63 : 0;  // negligible coefficients: target 0
 #pragma unroll
-  for (int k = 0; k < N; ++k) b[k * kCta] = pack_limbs(block_fix(f[k], E, n0));
+  for (int k = 0; k < N; ++k) b[k * STRIDE] = pack_limbs(block_fix(f[k], E, n0));
 }
-__device__ __forceinline__ void coeffs_to_smem(const Coeffs& C, long long* b, int& Ef, int& Eg) {
-  const double f[15] = {C.f00, C.f10, C.f01, C.f20, C.f11, C.f02, C.f30, C.f21,
-                        C.f12, C.f03, C.f40, C.f31, C.f22, C.f13, C.f04};
-  const double g[6] = {C.g00, C.g10, C.g01, C.g20, C.g11, C.g02};
-  fields_to_smem<15>(f, b, Ef);
-  fields_to_smem<6>(g, b + 15 * kCta, Eg);
-}
-
 // h^b of x-node p: W_p sum_a C_ab He_a(xi_p)/a! (value h 2^(E - 1082 - kd(p)))
-__device__ __forceinline__ void hf_node(const FixView& X, const int (&K)[5][2], long long (&h)[5]) {
+template <class V>
+__device__ __forceinline__ void hf_node(const V& X, const int (&K)[5][2], long long (&h)[5]) {
   LimbAcc a, b, c, d, e;
   X.mac(a, 0, K[0]); X.mac(a, 1, K[1]); X.mac(a, 3, K[2]); X.mac(a, 6, K[3]); X.mac(a, 10, K[4]);
   X.mac(b, 2, K[0]); X.mac(b, 4, K[1]); X.mac(b, 7, K[2]); X.mac(b, 11, K[3]);
@@ -827,7 +833,8 @@ __device__ __forceinline__ void hf_node(const FixView& X, const int (&K)[5][2], 
   X.mac(e, 14, K[0]);
   h[0] = a.value8(); h[1] = b.value8(); h[2] = c.value8(); h[3] = d.value8(); h[4] = e.value8();
 }
-__device__ __forceinline__ void hg_node(const FixView& X, const int (&K)[5][2], long long (&h)[3]) {
+template <class V>
+__device__ __forceinline__ void hg_node(const V& X, const int (&K)[5][2], long long (&h)[3]) {
   LimbAcc a, b, c;
   X.mac(a, 15, K[0]); X.mac(a, 16, K[1]); X.mac(a, 18, K[2]);
   X.mac(b, 17, K[0]); X.mac(b, 19, K[1]);
@@ -873,26 +880,57 @@ __device__ __forceinline__ void load_kf(int p, int (&K)[5][2]) {
 }
 
 struct Lat25 {
-  static constexpr int NQ = 5, POPS = 50, FIELDS = 21;
+  static constexpr int NQ = 5, POPS = 50, FIELDS = 21, GFIELD = 15, MOMS = 13;  // GFIELD: the first field of g
   typedef Moments Mom;
   typedef int NodeK[5][2];
   __device__ static __forceinline__ bool backward(int k) { return k != 0 && (k & 1) == 0; }
   __device__ static __forceinline__ int kdp(int k) { return k == 0 ? 0 : (k <= 2 ? kd(1) : kd(3)); }
-  __device__ static __forceinline__ Mom moments(const double* s, unsigned off, long long PL) {
-    return moments_fix<double>(s, off, PL);
+  __device__ static __forceinline__ void moments_f(const double* s, unsigned off, long long PL, Mom& m) {
+    moments_fix_f<double>(s, off, PL, m);
+  }
+  __device__ static __forceinline__ void moments_g(const double* s, unsigned off, long long PL, Mom& m) {
+    moments_fix_g<double>(s, off, PL, m);
   }
   template <int PRC>
   __device__ static __forceinline__ Coeffs coeffs(const Mom& m, const Phys& P) { return collision_coeffs<PRC>(m, P); }
   __device__ static __forceinline__ void to_smem(const Coeffs& C, long long* b, int& Ef, int& Eg) {
-    coeffs_to_smem(C, b, Ef, Eg);
+    const double f[15] = {C.f00, C.f10, C.f01, C.f20, C.f11, C.f02, C.f30, C.f21,
+                          C.f12, C.f03, C.f40, C.f31, C.f22, C.f13, C.f04};
+    const double g[6] = {C.g00, C.g10, C.g01, C.g20, C.g11, C.g02};
+    fields_to_smem<15>(f, b, Ef);
+    fields_to_smem<6>(g, b + 15 * kCta, Eg);
+  }
+  // the fields in order; the moments that a sum over f (k = 0) or g yields, and back
+  template <class Put>
+  __device__ static __forceinline__ void fields(const Coeffs& C, const Put& put) {
+    const double v[21] = {C.f00, C.f10, C.f01, C.f20, C.f11, C.f02, C.f30, C.f21, C.f12, C.f03, C.f40,
+                          C.f31, C.f22, C.f13, C.f04, C.g00, C.g10, C.g01, C.g20, C.g11, C.g02};
+#pragma unroll
+    for (int k = 0; k < 21; ++k) put(k, v[k]);
+  }
+  template <class Put>
+  __device__ static __forceinline__ void put(const Mom& m, int k, const Put& put) {
+    if (k == 0) {
+      put(0, m.m00); put(1, m.m10); put(2, m.m01); put(3, m.m20); put(4, m.m11); put(5, m.m02); put(6, m.m30);
+      put(7, m.m21); put(8, m.m12); put(9, m.m03);
+    } else {
+      put(10, m.g00); put(11, m.g10); put(12, m.g01);
+    }
+  }
+  template <class Get>
+  __device__ static __forceinline__ void get(Mom& m, const Get& get) {
+    m.m00 = get(0); m.m10 = get(1); m.m01 = get(2); m.m20 = get(3); m.m11 = get(4); m.m02 = get(5); m.m30 = get(6);
+    m.m21 = get(7); m.m12 = get(8); m.m03 = get(9); m.g00 = get(10); m.g10 = get(11); m.g01 = get(12);
   }
   __device__ static __forceinline__ void load_k(int p, NodeK& K) { load_kf(p, K); }
-  __device__ static __forceinline__ void target_f(const FixView& X, const NodeK& K, long long (&t)[5]) {
+  template <class V>
+  __device__ static __forceinline__ void target_f(const V& X, const NodeK& K, long long (&t)[5]) {
     long long h[5];
     hf_node(X, K, h);
     expand_node(h, t);
   }
-  __device__ static __forceinline__ void target_g(const FixView& X, const NodeK& K, long long (&t)[5]) {
+  template <class V>
+  __device__ static __forceinline__ void target_g(const V& X, const NodeK& K, long long (&t)[5]) {
     long long h[3];
     hg_node(X, K, h);
     expand_node(h, t);
@@ -913,8 +951,8 @@ struct Lat25 {
 //    populations that move along both axes, (p, 0) along x only and (0, p) along
 //    y only, so that all eight warps have the same work; the resting population
 //    needs none.  D2Q16: the four populations of x-node w % 4.
-//  * Collision with R < 8: a cell has 8 / R threads, which all form its
-//    coefficients and share the populations (in units of an x-node's f or g).
+//  * Collision with R < 8: a cell has 8 / R threads, which share its populations
+//    (in units of an x-node's f or g).
 struct GhostKinds {
   int k[4];  // xlo, xhi, ylo, yhi: 0 periodic, 1 zero gradient, else not written here
 };
@@ -958,7 +996,7 @@ __device__ __forceinline__ void write_images(S* p, long long PL, int x, int y, c
 // CODES: also the branch codes of every population's slopes (one byte x | y << 2
 // at codes[pop][y][x]) and, unless moms is null, the cells' moments.
 template <class L, int R, int PRC, bool RAT, bool CODES>
-__global__ void __launch_bounds__(kCta, 3) k_step_tile(const double* __restrict__ src, double* dst, Geom G, Phys P,
+__global__ void __launch_bounds__(kCta, R == 8 ? 3 : 1) k_step_tile(const double* __restrict__ src, double* dst, Geom G, Phys P,
                                                        GhostKinds B, unsigned int* __restrict__ flag,
                                                        unsigned char* codes, double* __restrict__ moms) {
   __shared__ long long s_buf[L::FIELDS * kCta];  // the advection's tiles, then the collision coefficients
@@ -1036,29 +1074,59 @@ __global__ void __launch_bounds__(kCta, 3) k_step_tile(const double* __restrict_
   constexpr int NG = 8 / R;  // threads of a cell
   const int row = threadIdx.y % R, group = threadIdx.y / R;
   const int x = x0 + threadIdx.x, y = y0 + row;
-  if (x >= G.Nx || y >= G.Ny) return;
   const unsigned off = (row * (unsigned)PT + threadIdx.x) * 8u;  // this cell's byte offset in the tile
-  const typename L::Mom m = L::moments(stile, off, PL);
-  if constexpr (CODES) {
-    // the recomputing adjoint also keeps the cell's moments (13 planes of
-    // Nx * Ny doubles, Moments field order) for its collision part
-    if (moms && group == 0) {
-      const long long ci = (long long)y * G.Nx + x;
-      const double v[13] = {m.m00, m.m10, m.m01, m.m20, m.m11, m.m02, m.m30,
-                            m.m21, m.m12, m.m03, m.g00, m.g10, m.g01};
-#pragma unroll
-      for (int k = 0; k < 13; ++k) moms[k * cplane + ci] = v[k];
-    }
-  }
+  const int cell = row * 32 + threadIdx.x;
+  const FixView X{s_buf + cell};
+  const bool inside = x < G.Nx && y < G.Ny;
   int Ef, Eg;
   double a1;
-  const int tid = threadIdx.y * 32 + threadIdx.x;
-  const FixView X{s_buf + tid};
-  {
+  auto collision = [&](const typename L::Mom& m) {
+    if constexpr (CODES) {
+      // the recomputing adjoint also keeps the cell's moments (13 planes of
+      // Nx * Ny doubles, Moments field order) for its collision part
+      if (moms) {
+        const long long ci = (long long)y * G.Nx + x;
+        const double v[13] = {m.m00, m.m10, m.m01, m.m20, m.m11, m.m02, m.m30,
+                              m.m21, m.m12, m.m03, m.g00, m.g10, m.g01};
+#pragma unroll
+        for (int k = 0; k < 13; ++k) moms[k * cplane + ci] = v[k];
+      }
+    }
     const auto C = L::template coeffs<PRC>(m, P);
     if (C.bad) atomicOr(flag, 1u);
-    L::to_smem(C, s_buf + tid, Ef, Eg);
+    L::to_smem(C, s_buf + cell, Ef, Eg);
     a1 = C.a1;
+  };
+  if constexpr (NG == 1) {
+    if (!inside) return;
+    typename L::Mom m;
+    L::moments_f(stile, off, PL, m);
+    L::moments_g(stile, off, PL, m);
+    collision(m);
+  } else {
+    // the first group sums f and forms the coefficients, the second sums g: all
+    // groups doing all of it would share the FP64 pipe (64^2: 22.6 -> 16.4 us)
+    __shared__ double s_share[4][32 * R];
+    __shared__ int s_block[2][32 * R];
+    typename L::Mom m;
+    if (inside && group == 0) L::moments_f(stile, off, PL, m);
+    if (inside && group == 1) {
+      L::moments_g(stile, off, PL, m);
+      s_share[0][cell] = m.g00; s_share[1][cell] = m.g10; s_share[2][cell] = m.g01;
+    }
+    __syncthreads();
+    if (inside && group == 0) {
+      m.g00 = s_share[0][cell]; m.g10 = s_share[1][cell]; m.g01 = s_share[2][cell];
+      collision(m);
+      s_share[3][cell] = a1;
+      s_block[0][cell] = Ef;
+      s_block[1][cell] = Eg;
+    }
+    __syncthreads();
+    if (!inside) return;
+    a1 = s_share[3][cell];
+    Ef = s_block[0][cell];
+    Eg = s_block[1][cell];
   }
 #pragma unroll 1
   for (int p0 = 0; p0 < NQ; p0 += NG > 2 ? NG / 2 : 1) {

@@ -25,7 +25,8 @@ inline GhostKinds ghost_kinds(const BCDev& bc) {
 // 2 rows on a full chip); while the grid's tiles are fewer than the SMs, lower
 // tiles shorten the step by spreading it over more of them, as long as each
 // SM gets no more than one.  Measured, D2Q25, us a step with 8 / 4 / 2 rows: 64^2
-// 41 / 29 / 23, 128^2 41 / 31 / 33, 192^2 42 / 41 / 54, 256^2 60 / 69 / 84.
+// 41 / 29 / 23 (16 since the low tiles share a cell's coefficients), 128^2
+// 41 / 31 / 33 (23 with 4 rows), 192^2 42 / 41 / 54, 256^2 60 / 69 / 84.
 inline int tile_rows(const Geom& G) {
   const long long tiles = (long long)((G.Nx + 31) / 32) * ((G.Ny + 7) / 8);
   return 4 * tiles <= 152 ? 2 : 2 * tiles <= 152 ? 4 : 8;

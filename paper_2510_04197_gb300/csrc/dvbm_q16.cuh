@@ -161,45 +161,41 @@ __device__ __forceinline__ long long pair_sum16(long long b, long long a) {
   return s.value();
 }
 
-// moments in block fixed point, as moments_fix for D2Q25
-__device__ __forceinline__ Mom moments_fix16(const double* __restrict__ s, unsigned off, long long PL) {
-  Mom m;
+// moments in block fixed point, as moments_fix for D2Q25: of f (k = 0) or g (k = 1)
+template <int k>
+__device__ __forceinline__ void moments_fix16(const double* __restrict__ s, unsigned off, long long PL, Mom& m) {
+  double v[16];
+  unsigned key = 0;
 #pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    double v[16];
-    unsigned key = 0;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      v[i] = __ldg(at(s + (16 * k + i) * PL, off));
-      key = max(key, abs_key(v[i]));
-    }
-    const int E = (int)(key >> 20);
-    const int n0 = E < 128 ? 63 : 2;
-    const int sc = E - 1080;
-    long long M0[4], M1[4], M2s = 0;  // y-sums of each x-node, M1 and M2 times 1/16, 1/32
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const long long x0 = block_fix(v[4 * p], E, n0), x1 = block_fix(v[4 * p + 1], E, n0),
-                      x2 = block_fix(v[4 * p + 2], E, n0), x3 = block_fix(v[4 * p + 3], E, n0);
-      const long long sA = x0 + x1, dA = x0 - x1, sB = x2 + x3, dB = x2 - x3;
-      M0[p] = sA + sB;
-      M1[p] = pair_sum16<1>(dB, dA);
-      if (k == 0) M2s += pair_sum16<2>(sB, sA);
-    }
-    const long long a0 = M0[0] + M0[1], b0 = M0[2] + M0[3], c0 = M0[0] - M0[1], d0 = M0[2] - M0[3];
-    const double s00 = key < 0x7ff00000u ? fix_to_double<true>(a0 + b0, sc) : __longlong_as_double(0x7ff8000000000000ll);
-    const double s10 = fix_to_double<true>(pair_sum16<1>(d0, c0), sc + 4);
-    const double s01 = fix_to_double<true>((M1[0] + M1[1]) + (M1[2] + M1[3]), sc + 4);
-    if (k == 0) {
-      m.m00 = s00; m.m10 = s10; m.m01 = s01;
-      m.m20 = fix_to_double<true>(pair_sum16<2>(b0, a0), sc + 5);
-      m.m02 = fix_to_double<true>(M2s, sc + 5);
-      m.m11 = fix_to_double<true>(pair_sum16<1>((M1[2] - M1[3]) << 4, (M1[0] - M1[1]) << 4), sc + 4);
-    } else {
-      m.g00 = s00; m.g10 = s10; m.g01 = s01;
-    }
+  for (int i = 0; i < 16; ++i) {
+    v[i] = __ldg(at(s + (16 * k + i) * PL, off));
+    key = max(key, abs_key(v[i]));
   }
-  return m;
+  const int E = (int)(key >> 20);
+  const int n0 = E < 128 ? 63 : 2;
+  const int sc = E - 1080;
+  long long M0[4], M1[4], M2s = 0;  // y-sums of each x-node, M1 and M2 times 1/16, 1/32
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const long long x0 = block_fix(v[4 * p], E, n0), x1 = block_fix(v[4 * p + 1], E, n0),
+                    x2 = block_fix(v[4 * p + 2], E, n0), x3 = block_fix(v[4 * p + 3], E, n0);
+    const long long sA = x0 + x1, dA = x0 - x1, sB = x2 + x3, dB = x2 - x3;
+    M0[p] = sA + sB;
+    M1[p] = pair_sum16<1>(dB, dA);
+    if (k == 0) M2s += pair_sum16<2>(sB, sA);
+  }
+  const long long a0 = M0[0] + M0[1], b0 = M0[2] + M0[3], c0 = M0[0] - M0[1], d0 = M0[2] - M0[3];
+  const double s00 = key < 0x7ff00000u ? fix_to_double<true>(a0 + b0, sc) : __longlong_as_double(0x7ff8000000000000ll);
+  const double s10 = fix_to_double<true>(pair_sum16<1>(d0, c0), sc + 4);
+  const double s01 = fix_to_double<true>((M1[0] + M1[1]) + (M1[2] + M1[3]), sc + 4);
+  if (k == 0) {
+    m.m00 = s00; m.m10 = s10; m.m01 = s01;
+    m.m20 = fix_to_double<true>(pair_sum16<2>(b0, a0), sc + 5);
+    m.m02 = fix_to_double<true>(M2s, sc + 5);
+    m.m11 = fix_to_double<true>(pair_sum16<1>((M1[2] - M1[3]) << 4, (M1[0] - M1[1]) << 4), sc + 4);
+  } else {
+    m.g00 = s00; m.g10 = s10; m.g01 = s01;
+  }
 }
 template <int k, int n>
 __device__ __forceinline__ void kqmac(LimbAcc& s, const Limbs& x) {
@@ -208,13 +204,16 @@ __device__ __forceinline__ void kqmac(LimbAcc& s, const Limbs& x) {
 }  // namespace q16
 
 struct Lat16 {
-  static constexpr int NQ = 4, POPS = 32, FIELDS = 16;
+  static constexpr int NQ = 4, POPS = 32, FIELDS = 16, GFIELD = 10, MOMS = 9;
   typedef q16::Mom Mom;
   typedef int NodeK[4][2];
   __device__ static __forceinline__ bool backward(int k) { return (k & 1) != 0; }
   __device__ static __forceinline__ int kdp(int k) { return q16::kdq(k); }
-  __device__ static __forceinline__ Mom moments(const double* s, unsigned off, long long PL) {
-    return q16::moments_fix16(s, off, PL);
+  __device__ static __forceinline__ void moments_f(const double* s, unsigned off, long long PL, Mom& m) {
+    q16::moments_fix16<0>(s, off, PL, m);
+  }
+  __device__ static __forceinline__ void moments_g(const double* s, unsigned off, long long PL, Mom& m) {
+    q16::moments_fix16<1>(s, off, PL, m);
   }
   template <int PRC>
   __device__ static __forceinline__ q16::Co coeffs(const Mom& m, const Phys& P) { return q16::coeffs<PRC>(m, P); }
@@ -225,6 +224,26 @@ struct Lat16 {
     fields_to_smem<10>(f, b, Ef);
     fields_to_smem<6>(g, b + 10 * kCta, Eg);
   }
+  template <class Put>
+  __device__ static __forceinline__ void fields(const q16::Co& C, const Put& put) {
+    const double v[16] = {C.f00, C.f10, C.f01, C.f20, C.f11, C.f02, C.f30, C.f21,
+                          C.f12, C.f03, C.g00, C.g10, C.g01, C.g20, C.g11, C.g02};
+#pragma unroll
+    for (int k = 0; k < 16; ++k) put(k, v[k]);
+  }
+  template <class Put>
+  __device__ static __forceinline__ void put(const Mom& m, int k, const Put& put) {
+    if (k == 0) {
+      put(0, m.m00); put(1, m.m10); put(2, m.m01); put(3, m.m20); put(4, m.m11); put(5, m.m02);
+    } else {
+      put(6, m.g00); put(7, m.g10); put(8, m.g01);
+    }
+  }
+  template <class Get>
+  __device__ static __forceinline__ void get(Mom& m, const Get& get) {
+    m.m00 = get(0); m.m10 = get(1); m.m01 = get(2); m.m20 = get(3); m.m11 = get(4); m.m02 = get(5);
+    m.g00 = get(6); m.g10 = get(7); m.g01 = get(8);
+  }
   __device__ static __forceinline__ void load_k(int p, NodeK& K) {
 #pragma unroll
     for (int n = 0; n < 4; ++n) {
@@ -232,7 +251,8 @@ struct Lat16 {
       K[n][1] = q16::c_kqf[p][n][1];
     }
   }
-  __device__ static __forceinline__ void target_f(const FixView& X, const NodeK& K, long long (&t)[4]) {
+  template <class V>
+  __device__ static __forceinline__ void target_f(const V& X, const NodeK& K, long long (&t)[4]) {
     LimbAcc a, b, c, d;
     X.mac(a, 0, K[0]); X.mac(a, 1, K[1]); X.mac(a, 3, K[2]); X.mac(a, 6, K[3]);
     X.mac(b, 2, K[0]); X.mac(b, 4, K[1]); X.mac(b, 7, K[2]);
@@ -247,7 +267,8 @@ struct Lat16 {
     t[0] = ea.value() + oa.value(); t[1] = ea.value() - oa.value();
     t[2] = eb.value() + ob.value(); t[3] = eb.value() - ob.value();
   }
-  __device__ static __forceinline__ void target_g(const FixView& X, const NodeK& K, long long (&t)[4]) {
+  template <class V>
+  __device__ static __forceinline__ void target_g(const V& X, const NodeK& K, long long (&t)[4]) {
     LimbAcc a, b, c;
     X.mac(a, 10, K[0]); X.mac(a, 11, K[1]); X.mac(a, 13, K[2]);
     X.mac(b, 12, K[0]); X.mac(b, 14, K[1]);

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kCta, 1024 / kCta) k_step32(const float* __res
   __shared__ long long s_fix[Lat25::FIELDS * kCta];
   const int tid = threadIdx.y * 32 + threadIdx.x;
   int Ef, Eg;
-  coeffs_to_smem(C, s_fix + tid, Ef, Eg);
+  Lat25::to_smem(C, s_fix + tid, Ef, Eg);
   const FixView X{s_fix + tid};
   node_update32<true>(0, s, d, G, X, Ef, Eg, P, a1f);
 #pragma unroll 1
