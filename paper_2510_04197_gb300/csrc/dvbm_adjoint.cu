@@ -525,11 +525,13 @@ __device__ __forceinline__ double advection_adjoint_rat(const double* __restrict
 // ------------------------------------------------- the coded adjoint step over tiles
 // One adjoint step in one launch, with the branch codes of the recomputed forward
 // step, in the forward step's two phases (k_step_tile): first one population per
-// warp over a 32 x 8 tile, then one cell per thread.  512^2: 0.47 ms for the two
+// warp over a 32 x R tile, then one cell per thread.  512^2: 0.47 ms for the two
 // kernels it replaces (one thread per cell and population in the advection, 64-bit
 // high products in the projection) -> 0.36 ms.  Bound by the FP64 pipe (54 % busy, about
 // 460 instructions a cell, half of them the reverse pass over the collision
-// coefficients) and by latency at 16 warps an SM.
+// coefficients) and by latency at 16 warps an SM.  100^2, all latency, with 4-row
+// tiles and the parts of a cell on several threads: 110 -> 75 us a step with the
+// recompute.
 
 // a code's multipliers 4 lq d(sigma)/d(first argument), /d(second), as a byte table
 // indexed by the code (lp and lq are coprime and lq <= 64, so 2 lp <= 254 fits)
@@ -540,11 +542,11 @@ __device__ __forceinline__ unsigned code_factor(unsigned table, unsigned code) {
 // What a warp reads of one population: the adjoint state at its lane's column in
 // stream rows -1 .. R + 1, one cell of the x-halo, the branch codes of its
 // column in rows -1 .. R (packed: x bits of rows 0 .., y bits of rows -1 ..)
-// and, lanes 0 .. 15, of the cells before and behind row lane % 8.
-constexpr int kAdjR = 8;
+// and, lanes 0 .. 2 R - 1, of the cells before and behind row lane % R.
+template <int R>
 struct AdjointLoad {
-  double v[kAdjR + 3], h;
-  unsigned char code[kAdjR + 2], edge;
+  double v[R + 3], h;
+  unsigned char code[R + 2], edge;
 };
 struct CodePlane {
   const unsigned char *own, *lo, *hi;  // [Ny][Nx]; the rows below y = 0 and above y = Ny - 1
@@ -553,23 +555,24 @@ struct CodePlane {
     return y < 0 ? lo : y >= Ny ? hi : own + (long long)y * Nx;
   }
 };
-__device__ __forceinline__ void adjoint_load(AdjointLoad& L, const double* __restrict__ plane, long long PT,
+template <int R>
+__device__ __forceinline__ void adjoint_load(AdjointLoad<R>& L, const double* __restrict__ plane, long long PT,
                                              const CodePlane& C, int x0, int y0, const AdvTile& T) {
   const int i = min(T.lane, T.W - 1);
   const int cx = T.fx ? T.W - 1 - i : i;
   const long long sy = T.fy ? -PT : PT;
   const double* row0 = plane + (T.fy ? (T.H - 1) * PT : 0);
 #pragma unroll
-  for (int j = -1; j <= kAdjR + 1; ++j) L.v[j + 1] = __ldg(at(row0 + min(j, T.H + 1) * sy, (unsigned)cx * 8u));
-  const int hr = min(T.lane & 7, T.H - 1), hc = T.lane >> 3;  // stream columns -1, W, W + 1 (or 0)
-  const int h = hc == 0 ? -1 : hc == 3 ? 0 : T.W - 1 + hc;
+  for (int j = -1; j <= R + 1; ++j) L.v[j + 1] = __ldg(at(row0 + min(j, T.H + 1) * sy, (unsigned)cx * 8u));
+  const int hr = min(T.lane % R, T.H - 1), hc = T.lane / R;  // stream columns -1, W, W + 1 (or 0)
+  const int h = hc == 0 ? -1 : hc > 2 ? 0 : T.W - 1 + hc;
   L.h = __ldg(row0 + hr * sy + (T.fx ? T.W - 1 - h : h));
 #pragma unroll
-  for (int j = -1; j <= kAdjR; ++j) {
+  for (int j = -1; j <= R; ++j) {
     const int y = y0 + (T.fy ? T.H - 1 - min(j, T.H) : min(j, T.H));
     L.code[j + 1] = __ldg(C.row(y) + x0 + cx);
   }
-  const int he = T.lane < 8 ? -1 : T.W;
+  const int he = T.lane < R ? -1 : T.W;
   int xe = x0 + (T.fx ? T.W - 1 - he : he);
   xe = xe < 0 ? C.Nx - 1 : xe >= C.Nx ? 0 : xe;
   L.edge = __ldg(C.own + (long long)(y0 + (T.fy ? T.H - 1 - hr : hr)) * C.Nx + xe);
@@ -581,10 +584,9 @@ __device__ __forceinline__ void adjoint_load(AdjointLoad& L, const double* __res
 // cell i gets k (Dbar_i - Dbar_{i+1}), subtracted from its adjoint.  Writes the
 // sums over both axes as integers in units of 2^(E - 1076), returns E.  Walked
 // against an axis, the codes' arguments are swapped (tables t1, t2).
-template <bool MX, bool MY, class Next>
-__device__ __forceinline__ int adjoint_walk(const AdjointLoad& L, const Next& next, long long* out, long long PT,
+template <int R, bool MX, bool MY, class Next>
+__device__ __forceinline__ int adjoint_walk(const AdjointLoad<R>& L, const Next& next, long long* out, long long PT,
                                             const AdvTile& T, const Phys& P, long long kx, long long ky, long long* xs) {
-  constexpr int R = kAdjR;
   const int lane = T.lane;
   const bool in = lane < T.W;
   const unsigned lx = in ? (unsigned)(T.fx ? T.W - 1 - lane : lane) : 0u;
@@ -600,7 +602,7 @@ __device__ __forceinline__ int adjoint_walk(const AdjointLoad& L, const Next& ne
   __syncwarp();
 #pragma unroll
   for (int j = J0; j <= J1; ++j) xs[(j + 1) * kAdvPitch + lane + 1] = block_fix(L.v[j + 1], E, n0);
-  const int hr = lane & 7, hc = lane >> 3;
+  const int hr = lane % R, hc = lane / R;
   if (MX) {
     __syncwarp();
     if (hc < 3 && hr < T.H) xs[(hr + 1) * kAdvPitch + (hc == 0 ? 0 : T.W + hc)] = block_fix(L.h, E, n0);
@@ -619,7 +621,7 @@ __device__ __forceinline__ int adjoint_walk(const AdjointLoad& L, const Next& ne
   if (MX) {
     // Dbar of column W, one row per lane, kept in column W + 1
     const unsigned last = __shfl_sync(0xffffffffu, xb, T.W - 1);  // codes of column W - 1
-    const unsigned be = __shfl_sync(0xffffffffu, edge, 8 + (lane & 7));
+    const unsigned be = __shfl_sync(0xffffffffu, edge, R + lane % R);
     if (lane < T.H) {
       long long* r = xs + (lane + 1) * kAdvPitch + T.W;  // column W - 1
       const long long a = r[0] - r[1], b = r[1] - r[2];
@@ -783,35 +785,39 @@ __device__ __forceinline__ int scale_moments(const double (&m)[N], long long (&Q
 // and ghi ([NPOP][Nx]; NULL: the codes wrap).  moms: the moments of X, or NULL.
 // partial[4 blk + k]: the block's sums of the parameter adjoints (dt_mu, Pr, gm1,
 // epsf).
-template <int PRC>
-__global__ void __launch_bounds__(256, 2) k_adjoint_tile(const double* __restrict__ X, const double* __restrict__ Lin,
+// R: tile height, as in k_step_tile; with R < 8 a cell has 8 / R threads: the first
+// projects f and forms the moment adjoints, the second projects g, all share the
+// populations.
+template <int R, int PRC>
+__global__ void __launch_bounds__(256, R == 8 ? 2 : 1) k_adjoint_tile(const double* __restrict__ X,
+                                                         const double* __restrict__ Lin,
                                                          double* Lout, double* __restrict__ partial,
                                                          const unsigned char* __restrict__ codes,
                                                          const double* __restrict__ moms,
                                                          const unsigned char* __restrict__ glo,
                                                          const unsigned char* __restrict__ ghi, Geom G, Phys P) {
-  __shared__ long long s_xs[8 * (kAdjR + 3) * kAdvPitch];
+  __shared__ long long s_xs[8 * (R + 3) * kAdvPitch];
   __shared__ int s_exp[NPOP];
-  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8;
+  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * R;
   const long long PL = G.plane, PT = G.pitch, cplane = (long long)G.Nx * G.Ny;
   const double* ltile = Lin + cell_index(G, y0, x0);
   const double* xtile = X + cell_index(G, y0, x0);
   double* otile = Lout + cell_index(G, y0, x0);
-  const int w = __shfl_sync(0xffffffffu, (int)threadIdx.y, 0);
   {
+    const int w = __shfl_sync(0xffffffffu, (int)threadIdx.y, 0);
     const int c0 = 25 * (w >> 2), p = 1 + (w & 3);
     AdvTile T;
     T.W = min(32, G.Nx - x0);
-    T.H = min(8, G.Ny - y0);
+    T.H = min(R, G.Ny - y0);
     T.lane = threadIdx.x;
-    long long* xs = s_xs + w * ((kAdjR + 3) * kAdvPitch);
+    long long* xs = s_xs + w * ((R + 3) * kAdvPitch);
     auto tile = [&](int pp, int q) {
       AdvTile t = T;
       t.fx = Lat25::backward(pp);
       t.fy = Lat25::backward(q);
       return t;
     };
-    AdjointLoad V;
+    AdjointLoad<R> V;
     auto load = [&](int pp, int q) {
       const int c = c0 + 5 * pp + q;
       CodePlane C;
@@ -820,20 +826,20 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_tile(const double* __restric
       C.Ny = G.Ny;
       C.lo = glo ? glo + (long long)c * G.Nx : C.own + (cplane - G.Nx);
       C.hi = ghi ? ghi + (long long)c * G.Nx : C.own;
-      adjoint_load(V, ltile + c * PL, PT, C, x0, y0, tile(pp, q));
+      adjoint_load<R>(V, ltile + c * PL, PT, C, x0, y0, tile(pp, q));
     };
     auto out = [&](int c) { return (long long*)(otile + c * PL); };
     load(p, 0);
-    int E = adjoint_walk<true, false>(V, [&] { load(p, 1); }, out(c0 + 5 * p), PT, tile(p, 0), P, P.kxq[p], 0, xs);
+    int E = adjoint_walk<R, true, false>(V, [&] { load(p, 1); }, out(c0 + 5 * p), PT, tile(p, 0), P, P.kxq[p], 0, xs);
     if (T.lane == 0) s_exp[c0 + 5 * p] = E;
 #pragma unroll 1
     for (int q = 1; q < 5; ++q) {
       const int c = c0 + 5 * p + q;
-      E = adjoint_walk<true, true>(V, [&] { load(q < 4 ? p : 0, q < 4 ? q + 1 : p); }, out(c), PT, tile(p, q), P,
-                                   P.kxq[p], P.kyq[q], xs);
+      E = adjoint_walk<R, true, true>(V, [&] { load(q < 4 ? p : 0, q < 4 ? q + 1 : p); }, out(c), PT, tile(p, q), P,
+                                      P.kxq[p], P.kyq[q], xs);
       if (T.lane == 0) s_exp[c] = E;
     }
-    E = adjoint_walk<false, true>(V, [] {}, out(c0 + p), PT, tile(0, p), P, 0, P.kyq[p], xs);
+    E = adjoint_walk<R, false, true>(V, [] {}, out(c0 + p), PT, tile(0, p), P, 0, P.kyq[p], xs);
     if (T.lane == 0) s_exp[c0 + p] = E;
     if (p == 1) {
       if (T.lane == 0) s_exp[c0] = 0;
@@ -842,24 +848,25 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_tile(const double* __restric
     }
   }
   __syncthreads();
+  constexpr int NG = 8 / R;
+  const int row = threadIdx.y % R, group = threadIdx.y / R;
   // threads beyond a ragged tile work on its last cell again and write nothing:
   // uniform control flow keeps the planes' addresses in uniform registers
-  const bool active = x0 + (int)threadIdx.x < G.Nx && y0 + (int)threadIdx.y < G.Ny;
-  const int x = min(x0 + (int)threadIdx.x, G.Nx - 1), y = min(y0 + (int)threadIdx.y, G.Ny - 1);
+  const bool active = x0 + (int)threadIdx.x < G.Nx && y0 + row < G.Ny;
+  const int x = min(x0 + (int)threadIdx.x, G.Nx - 1), y = min(y0 + row, G.Ny - 1);
+  const unsigned off = ((y - y0) * (unsigned)PT + (x - x0)) * 8u;
   ParamBar pb = {0, 0, 0, 0};
-  {
-    const unsigned off = ((y - y0) * (unsigned)PT + (x - x0)) * 8u;
-    double a1b = 0.0;
+  // the moment adjoints of the collision (from the projections cb, cg and sum lambda X)
+  // as fixed-point polynomials: f at exponent Ef, g at Eg
+  double a1;
+  long long F[10], H[3];
+  int Ef, Eg;
+  auto pull_back = [&](const double (&cb)[15], const double (&cg)[6], double a1b) {
     Coeffs Cb = {};
-    {
-      double cb[15], cg[6];
-      project<4>(ltile, xtile, off, PL, cb, a1b);
-      project<2>(ltile + 25 * PL, xtile + 25 * PL, off, PL, cg, a1b);
-      Cb.f00 = cb[0]; Cb.f10 = cb[1]; Cb.f01 = cb[2]; Cb.f20 = cb[3]; Cb.f11 = cb[4]; Cb.f02 = cb[5];
-      Cb.f30 = cb[6]; Cb.f21 = cb[7]; Cb.f12 = cb[8]; Cb.f03 = cb[9]; Cb.f40 = cb[10]; Cb.f31 = cb[11];
-      Cb.f22 = cb[12]; Cb.f13 = cb[13]; Cb.f04 = cb[14];
-      Cb.g00 = cg[0]; Cb.g10 = cg[1]; Cb.g01 = cg[2]; Cb.g20 = cg[3]; Cb.g11 = cg[4]; Cb.g02 = cg[5];
-    }
+    Cb.f00 = cb[0]; Cb.f10 = cb[1]; Cb.f01 = cb[2]; Cb.f20 = cb[3]; Cb.f11 = cb[4]; Cb.f02 = cb[5];
+    Cb.f30 = cb[6]; Cb.f21 = cb[7]; Cb.f12 = cb[8]; Cb.f03 = cb[9]; Cb.f40 = cb[10]; Cb.f31 = cb[11];
+    Cb.f22 = cb[12]; Cb.f13 = cb[13]; Cb.f04 = cb[14];
+    Cb.g00 = cg[0]; Cb.g10 = cg[1]; Cb.g01 = cg[2]; Cb.g20 = cg[3]; Cb.g11 = cg[4]; Cb.g02 = cg[5];
     Moments m;
     if (moms) {
       const long long ci = (long long)y * G.Nx + x;
@@ -872,15 +879,57 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_tile(const double* __restric
       m = moments_fix<double>(xtile, off, PL);
     }
     Moments mb = {};
-    const double a1 = collision_coeffs_rev<PRC>(m, P, Cb, a1b, mb, pb);
+    a1 = collision_coeffs_rev<PRC>(m, P, Cb, a1b, mb, pb);
     // the pullback sum_j mbar_j dm_j/dX of population (p, q) is the polynomial
     // sum mbar_ab xi_p^a xi_q^b, in fixed point with the flux sum taken off
     const double mf[10] = {mb.m00, XB * mb.m10, XB * mb.m01, (XB * XB) * mb.m20, (XB * XB) * mb.m11, (XB * XB) * mb.m02,
                            (XB * XB * XB) * mb.m30, (XB * XB * XB) * mb.m21, (XB * XB * XB) * mb.m12,
                            (XB * XB * XB) * mb.m03};
     const double mg[3] = {mb.g00, XB * mb.g10, XB * mb.g01};
-    long long F[10], H[3];
-    const int Ef = scale_moments(mf, F), Eg = scale_moments(mg, H);
+    Ef = scale_moments(mf, F);
+    Eg = scale_moments(mg, H);
+  };
+  if constexpr (NG == 1) {
+    double cb[15], cg[6], a1b = 0.0;
+    project<4>(ltile, xtile, off, PL, cb, a1b);
+    project<2>(ltile + 25 * PL, xtile + 25 * PL, off, PL, cg, a1b);
+    pull_back(cb, cg, a1b);
+  } else {
+    __shared__ double s_g[7][32 * R], s_a1[32 * R];
+    __shared__ long long s_p[13][32 * R];
+    __shared__ int s_e[2][32 * R];
+    const int cell = row * 32 + threadIdx.x;
+    double cb[15], cg[6], a1b = 0.0;
+    if (group == 0) project<4>(ltile, xtile, off, PL, cb, a1b);
+    if (group == 1) {
+      project<2>(ltile + 25 * PL, xtile + 25 * PL, off, PL, cg, a1b);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) s_g[k][cell] = cg[k];
+      s_g[6][cell] = a1b;
+    }
+    __syncthreads();
+    if (group == 0) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) cg[k] = s_g[k][cell];
+      pull_back(cb, cg, a1b + s_g[6][cell]);
+#pragma unroll
+      for (int k = 0; k < 10; ++k) s_p[k][cell] = F[k];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) s_p[10 + k][cell] = H[k];
+      s_a1[cell] = a1;
+      s_e[0][cell] = Ef;
+      s_e[1][cell] = Eg;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 10; ++k) F[k] = s_p[k][cell];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) H[k] = s_p[10 + k][cell];
+    a1 = s_a1[cell];
+    Ef = s_e[0][cell];
+    Eg = s_e[1][cell];
+  }
+  {
     // even and odd parts in x of the inner node pair
     LimbAcc t0, u0, t1, u1, u2, v0;
     rmac<2>(t0, F[3]);
@@ -892,7 +941,9 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_tile(const double* __restric
     const long long eA0 = F[0] + t0.value8(), oA0 = u0.value8(), eA1 = F[2] + t1.value8(), oA1 = u1.value8(),
                     oA2 = u2.value8(), gA = v0.value8();
 #pragma unroll 1
-    for (int p = 0; p < 5; ++p) {
+    for (int p0 = 0; p0 < 5; p0 += NG > 2 ? NG / 2 : 1) {
+      const int p = NG > 2 ? p0 + (group >> 1) : p0;  // as in k_step_tile
+      if (NG > 2 && p >= 5) break;
       // y-polynomial of this x-node
       long long b0, b1, b2, g0;
       if (p == 0) {
@@ -909,6 +960,7 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_tile(const double* __restric
       }
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
+        if (NG > 1 && k != (group & 1)) continue;
         const double* lp = ltile + (25 * k + 5 * p) * PL;
         double* op = otile + (25 * k + 5 * p) * PL;
         double lv[5];
@@ -943,7 +995,7 @@ __global__ void __launch_bounds__(256, 2) k_adjoint_tile(const double* __restric
   __syncthreads();
   double* sh = (double*)s_xs;
   const int t = threadIdx.y * 32 + threadIdx.x;
-  if (!active) pb = {0, 0, 0, 0};
+  if (!active || group != 0) pb = {0, 0, 0, 0};
   sh[t] = pb.dt_mu; sh[256 + t] = pb.Pr; sh[512 + t] = pb.gm1; sh[768 + t] = pb.epsf;
   __syncthreads();
   for (int n = 128; n > 0; n >>= 1) {
@@ -1157,7 +1209,11 @@ __global__ void __launch_bounds__(256) k_adjoint_init(const double* __restrict__
 }
 
 // ------------------------------------------------------------------ wrappers
-int adjoint_blocks(const Geom& G) { return ((G.Nx + 31) / 32) * ((G.Ny + 7) / 8); }
+// partial-sum slots of a launch: the coded step's blocks, at least those of the 8-row kernels
+int adjoint_blocks(const Geom& G) {
+  const int R = tile_rows(G);
+  return ((G.Nx + 31) / 32) * ((G.Ny + R - 1) / R);
+}
 
 // Branch-code rows next to a band's edges: unpack = 0 copies rows y = 0 (to
 // lo) and y = Ny - 1 (to hi) of every population's codes, unpack = 1 copies
@@ -1187,14 +1243,25 @@ cudaError_t launch_code_rows(unsigned char* codes, void* lo, void* hi, unsigned 
   return cudaGetLastError();
 }
 
+template <int R>
+static void launch_adjoint_tile(const double* X, const double* Lin, double* Lout, double* partial,
+                                const unsigned char* codes, const double* moms, const unsigned char* glo,
+                                const unsigned char* ghi, const Geom& G, const Phys& P, cudaStream_t st) {
+  const dim3 b(32, 8), g((G.Nx + 31) / 32, (G.Ny + R - 1) / R);
+  if (P.prc < 0) k_adjoint_tile<R, -1><<<g, b, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
+  else if (P.prc > 0) k_adjoint_tile<R, 1><<<g, b, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
+  else k_adjoint_tile<R, 0><<<g, b, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
+}
+
 cudaError_t launch_adjoint_step(const double* X, const double* Lin, double* Lout, double* partial,
                                 const unsigned char* codes, const double* moms, const Geom& G, const Phys& P,
                                 cudaStream_t st, const unsigned char* glo, const unsigned char* ghi) {
   dim3 block(32, 8), grid((G.Nx + 31) / 32, (G.Ny + 7) / 8);
   if (codes) {
-    if (P.prc < 0) k_adjoint_tile<-1><<<grid, block, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
-    else if (P.prc > 0) k_adjoint_tile<1><<<grid, block, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
-    else k_adjoint_tile<0><<<grid, block, 0, st>>>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P);
+    const int R = tile_rows(G);
+    if (R == 8) launch_adjoint_tile<8>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P, st);
+    else if (R == 4) launch_adjoint_tile<4>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P, st);
+    else launch_adjoint_tile<2>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P, st);
     return cudaGetLastError();
   }
   if (P.prc < 0) k_adjoint_local<-1><<<grid, block, 0, st>>>(X, Lin, Lout, partial, G, P);
