@@ -87,6 +87,7 @@ __device__ __forceinline__ void ghost_cells(int side, int kind, int k, int j, co
 // periodic and zero-gradient sides, one thread per (side, layer, position, population)
 template <class S>
 __global__ void k_ghost(S* __restrict__ buf, Geom G, BCDev bc) {
+  buf = chain_wait(buf);
   const int side = blockIdx.y, kind = bc.kind[side], pop = blockIdx.z;
   if (kind > 1) return;
   const int len = side < 2 ? G.Ny : G.Nx;
@@ -113,6 +114,7 @@ __global__ void __launch_bounds__(kCta, 2) k_wall(S* __restrict__ buf, Geom G, P
   __shared__ long long s_fix[N * 32];
   __shared__ double s_m[LT::MOMS][32], s_eq[2][N][32];
   __shared__ int s_E[2][32];
+  buf = chain_wait(buf);
   const int side = blockIdx.y, lane = threadIdx.x, w = threadIdx.y;
   if (bc.kind[side] != 2) return;
   const int len = side < 2 ? G.Ny : G.Nx;
@@ -124,8 +126,8 @@ __global__ void __launch_bounds__(kCta, 2) k_wall(S* __restrict__ buf, Geom G, P
   const S* b = buf + cell_index(G, by, bx);
   if (w < 2) {
     typename LT::Mom m;
-    if (w == 0) L::template sum_f<S>(b, PL, m, P);
-    else L::template sum_g<S>(b, PL, m, P);
+    if (w == 0) L::template sum_f<S, false>(b, PL, m, P);
+    else L::template sum_g<S, false>(b, PL, m, P);
     LT::put(m, w, [&](int k, double v) { s_m[k][lane] = v; });
   }
   __syncthreads();
@@ -337,14 +339,14 @@ cudaError_t launch_ghost(int lattice, int storage, void* buf, const Geom& G, con
   }
   if (copies) {
     const dim3 b(128), g((2 * len + 127) / 128, 4, lattice == 1 ? L16::NPOP : L25::NPOP);
-    if (storage == 0) k_ghost<double><<<g, b, 0, st>>>((double*)buf, G, bc);
-    else k_ghost<float><<<g, b, 0, st>>>((float*)buf, G, bc);
+    if (storage == 0) launch_chained(k_ghost<double>, g, b, st, (double*)buf, G, bc);
+    else launch_chained(k_ghost<float>, g, b, st, (float*)buf, G, bc);
   }
   if (walls) {
     const dim3 b(32, 8), g((2 * len + 31) / 32, 4);
-    if (lattice == 1) k_wall<L16, double><<<g, b, 0, st>>>((double*)buf, G, P, M, bc);
-    else if (storage == 0) k_wall<L25, double><<<g, b, 0, st>>>((double*)buf, G, P, M, bc);
-    else k_wall<L25, float><<<g, b, 0, st>>>((float*)buf, G, P, M, bc);
+    if (lattice == 1) launch_chained(k_wall<L16, double>, g, b, st, (double*)buf, G, P, M, bc);
+    else if (storage == 0) launch_chained(k_wall<L25, double>, g, b, st, (double*)buf, G, P, M, bc);
+    else launch_chained(k_wall<L25, float>, g, b, st, (float*)buf, G, P, M, bc);
   }
   return cudaGetLastError();
 }

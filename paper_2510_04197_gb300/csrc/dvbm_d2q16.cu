@@ -10,9 +10,13 @@ template <int R, bool RAT>
 static void launch_tile16(const double* s, double* d, const Geom& G, const Phys& P, const GhostKinds& B,
                           unsigned int* flag, cudaStream_t st) {
   const dim3 block(32, 8), grid((G.Nx + 31) / 32, (G.Ny + R - 1) / R);
-  if (P.prc < 0) k_step_tile<Lat16, R, -1, RAT, false><<<grid, block, 0, st>>>(s, d, G, P, B, flag, nullptr, nullptr);
-  else if (P.prc > 0) k_step_tile<Lat16, R, 1, RAT, false><<<grid, block, 0, st>>>(s, d, G, P, B, flag, nullptr, nullptr);
-  else k_step_tile<Lat16, R, 0, RAT, false><<<grid, block, 0, st>>>(s, d, G, P, B, flag, nullptr, nullptr);
+  const auto k = P.prc < 0   ? k_step_tile<Lat16, R, -1, RAT, false>
+                 : P.prc > 0 ? k_step_tile<Lat16, R, 1, RAT, false>
+                             : k_step_tile<Lat16, R, 0, RAT, false>;
+  unsigned char* codes = nullptr;
+  double* moms = nullptr;
+  if (R < 8) launch_chained(k, grid, block, st, s, d, G, P, B, flag, codes, moms);
+  else k<<<grid, block, 0, st>>>(s, d, G, P, B, flag, codes, moms);
 }
 
 cudaError_t launch_step16(const void* src, void* dst, const Geom& G, const Phys& P, const BCDev& bc, unsigned int* flag,

@@ -11,6 +11,21 @@ struct BCDev {
   double Tw[4];         // wall temperature
 };
 
+// launch of a kernel that begins with chain_wait
+template <class... P, class... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, (P)args...);  // an error is left for cudaGetLastError, as by <<<>>>
+}
+
 struct Macro {          // constants needed to turn moments into physical fields
   double c, T_ref, R, gamma;
 };

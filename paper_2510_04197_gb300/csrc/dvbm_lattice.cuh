@@ -21,14 +21,14 @@ struct L25 {
   static constexpr int NPOP = 50;
   typedef Lat25 Tile;
   // the sums over f and over g of one cell
-  template <class S>
+  template <class S, bool NC = true>
   __device__ static void sum_f(const S* p, long long PL, Moments& m, const Phys& P) {
-    moments_fix_f<S>(p, 0u, PL, m);
+    moments_fix_f<S, NC>(p, 0u, PL, m);
     if constexpr (sizeof(S) == 4) add_reference_f(m, P);
   }
-  template <class S>
+  template <class S, bool NC = true>
   __device__ static void sum_g(const S* p, long long PL, Moments& m, const Phys& P) {
-    moments_fix_g<S>(p, 0u, PL, m);
+    moments_fix_g<S, NC>(p, 0u, PL, m);
     if constexpr (sizeof(S) == 4) m.g00 += P.gref0;
   }
   __device__ static CellState state_of(const Moments& m, const Phys& P, const Macro& M) {
@@ -55,14 +55,14 @@ struct L25 {
 struct L16 {
   static constexpr int NPOP = 32;
   typedef Lat16 Tile;
-  template <class S>
+  template <class S, bool NC = true>
   __device__ static void sum_f(const S* p, long long PL, q16::Mom& m, const Phys&) {
     static_assert(sizeof(S) == 8, "the D2Q16 / split I model has FP64 storage only");
-    q16::moments_fix16<0>(p, 0u, PL, m);
+    q16::moments_fix16<0, NC>(p, 0u, PL, m);
   }
-  template <class S>
+  template <class S, bool NC = true>
   __device__ static void sum_g(const S* p, long long PL, q16::Mom& m, const Phys&) {
-    q16::moments_fix16<1>(p, 0u, PL, m);
+    q16::moments_fix16<1, NC>(p, 0u, PL, m);
   }
   __device__ static CellState state_of(const q16::Mom& m, const Phys& P, const Macro& M) {
     CellState c;

@@ -162,13 +162,13 @@ __device__ __forceinline__ long long pair_sum16(long long b, long long a) {
 }
 
 // moments in block fixed point, as moments_fix for D2Q25: of f (k = 0) or g (k = 1)
-template <int k>
+template <int k, bool NC = true>
 __device__ __forceinline__ void moments_fix16(const double* __restrict__ s, unsigned off, long long PL, Mom& m) {
   double v[16];
   unsigned key = 0;
 #pragma unroll
   for (int i = 0; i < 16; ++i) {
-    v[i] = __ldg(at(s + (16 * k + i) * PL, off));
+    v[i] = load<NC>(at(s + (16 * k + i) * PL, off));
     key = max(key, abs_key(v[i]));
   }
   const int E = (int)(key >> 20);
@@ -209,11 +209,13 @@ struct Lat16 {
   typedef int NodeK[4][2];
   __device__ static __forceinline__ bool backward(int k) { return (k & 1) != 0; }
   __device__ static __forceinline__ int kdp(int k) { return q16::kdq(k); }
+  template <bool NC>
   __device__ static __forceinline__ void moments_f(const double* s, unsigned off, long long PL, Mom& m) {
-    q16::moments_fix16<0>(s, off, PL, m);
+    q16::moments_fix16<0, NC>(s, off, PL, m);
   }
+  template <bool NC>
   __device__ static __forceinline__ void moments_g(const double* s, unsigned off, long long PL, Mom& m) {
-    q16::moments_fix16<1>(s, off, PL, m);
+    q16::moments_fix16<1, NC>(s, off, PL, m);
   }
   template <int PRC>
   __device__ static __forceinline__ q16::Co coeffs(const Mom& m, const Phys& P) { return q16::coeffs<PRC>(m, P); }

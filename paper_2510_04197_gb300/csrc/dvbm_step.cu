@@ -111,9 +111,11 @@ template <int R, bool RAT, bool CODES>
 static void launch_tile(const double* s, double* d, const Geom& G, const Phys& P, const GhostKinds& B, unsigned int* flag,
                         unsigned char* codes, double* moms, cudaStream_t st) {
   const dim3 block(32, 8), grid((G.Nx + 31) / 32, (G.Ny + R - 1) / R);
-  if (P.prc < 0) k_step_tile<Lat25, R, -1, RAT, CODES><<<grid, block, 0, st>>>(s, d, G, P, B, flag, codes, moms);
-  else if (P.prc > 0) k_step_tile<Lat25, R, 1, RAT, CODES><<<grid, block, 0, st>>>(s, d, G, P, B, flag, codes, moms);
-  else k_step_tile<Lat25, R, 0, RAT, CODES><<<grid, block, 0, st>>>(s, d, G, P, B, flag, codes, moms);
+  const auto k = P.prc < 0   ? k_step_tile<Lat25, R, -1, RAT, CODES>
+                 : P.prc > 0 ? k_step_tile<Lat25, R, 1, RAT, CODES>
+                             : k_step_tile<Lat25, R, 0, RAT, CODES>;
+  if (R < 8) launch_chained(k, grid, block, st, s, d, G, P, B, flag, codes, moms);
+  else k<<<grid, block, 0, st>>>(s, d, G, P, B, flag, codes, moms);
 }
 template <bool RAT, bool CODES>
 static void launch_tiles(const double* s, double* d, const Geom& G, const Phys& P, const GhostKinds& B,
