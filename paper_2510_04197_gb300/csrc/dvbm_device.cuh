@@ -141,6 +141,15 @@ __device__ __forceinline__ double recip(double x) {
   return fma(r, fma(e, e, e), r);
 }
 
+// v > 0 and |v| < 1e300 (false for NaN) on the bit patterns: a comparison of doubles
+// takes a slot of the FP64 pipe
+__device__ __forceinline__ bool is_positive(double v) {
+  return (unsigned long long)__double_as_longlong(v) - 1ull < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool is_bounded(double v) {
+  return (__double_as_longlong(v) & 0x7fffffffffffffffll) < 0x7e37e43c8800759cll;
+}
+
 // Collision coefficients from the moments (Sec. II.C relaxation times,
 // Table I split-II quasi-equilibria).  PRC selects the Prandtl case at
 // compile time: -1 (Pr < 1), 0 (Pr = 1), +1 (Pr > 1).
@@ -164,7 +173,7 @@ __device__ __forceinline__ Coeffs collision_coeffs(const Moments& m, const Phys&
   const double Et = fma(0.5, m.m20 + m.m02, m.g00 * P.inv_c2);        // E / c^2
   const double theta = P.gm1 * fma(-0.5, fma(ux, ux, uy * uy), Et * irho);
   const double s = theta - 1.0;
-  C.bad = !(rho > 0.0) || !(theta > 0.0) || !(fabs(Et) < 1e300);
+  C.bad = !is_positive(rho) || !is_positive(theta) || !is_bounded(Et);
   const double rt = rho * theta;                                         // p / c^2
   const double kp = (P.dt_mu * P.c2) * rt;                               // dt p / mu
   const double k1 = PRC <= 0 ? kp : kp * P.Pr;                           // dt/tau1
