@@ -46,6 +46,18 @@ struct L25 {
     sum_g<S>(p, PL, m, P);
     return state_of(m, P, M);
   }
+  // the same in units of c and T_ref, and its equilibrium coefficients
+  __device__ static void reduced_state(const Moments& m, const Phys& P, double& rho, double& ux, double& uy,
+                                       double& theta) {
+    rho = m.m00;
+    const double irho = recip(rho);
+    ux = m.m10 * irho;
+    uy = m.m01 * irho;
+    theta = P.gm1 * fma(-0.5, fma(ux, ux, uy * uy), fma(0.5, m.m20 + m.m02, m.g00 * P.inv_c2) * irho);
+  }
+  __device__ static Coeffs reduced_equilibrium(double rho, double ux, double uy, double theta, const Phys& P) {
+    return equilibrium_coeffs(rho, ux, uy, theta, P);
+  }
   // equilibrium coefficients of (rho, u, T) (Sec. III.A.3 initial conditions)
   __device__ static Coeffs equilibrium(double rho, double ux, double uy, double T, const Phys& P, const Macro& M) {
     return equilibrium_coeffs(rho, ux / M.c, uy / M.c, T / M.T_ref, P);
@@ -78,6 +90,17 @@ struct L16 {
     sum_f<S>(p, PL, m, P);
     sum_g<S>(p, PL, m, P);
     return state_of(m, P, M);
+  }
+  __device__ static void reduced_state(const q16::Mom& m, const Phys& P, double& rho, double& ux, double& uy,
+                                       double& theta) {
+    rho = m.m00;
+    const double irho = recip(rho);
+    ux = m.m10 * irho;
+    uy = m.m01 * irho;
+    theta = P.gm1 * fma(-0.5, fma(ux, ux, uy * uy), m.g00 * P.inv_c2 * irho);
+  }
+  __device__ static q16::Co reduced_equilibrium(double rho, double ux, double uy, double theta, const Phys& P) {
+    return q16::equilibrium(rho, ux, uy, theta, P);
   }
   __device__ static q16::Co equilibrium(double rho, double ux, double uy, double T, const Phys& P, const Macro& M) {
     return q16::equilibrium(rho, ux / M.c, uy / M.c, T / M.T_ref, P);

@@ -117,7 +117,7 @@ __device__ __forceinline__ Co equilibrium(double rho, double ux, double uy, doub
   Co C;
   const Eq3 e = eq_f3(rho, ux, uy, theta - 1.0);
   const double pRT = rho * P.c2 * theta;
-  const double E = rho * P.c2 * (theta / P.gm1 + 0.5 * fma(ux, ux, uy * uy));
+  const double E = rho * P.c2 * (theta * recip(P.gm1) + 0.5 * fma(ux, ux, uy * uy));
   const EqG q = eq_g1(E, pRT, ux, uy, theta);
   C.f00 = e.a00; C.f10 = e.a10; C.f01 = e.a01; C.f20 = e.a20; C.f11 = e.a11; C.f02 = e.a02;
   C.f30 = e.a30; C.f21 = e.a21; C.f12 = e.a12; C.f03 = e.a03;
