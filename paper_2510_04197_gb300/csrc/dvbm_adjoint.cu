@@ -1211,7 +1211,7 @@ __global__ void __launch_bounds__(256) k_adjoint_init(const double* __restrict__
 // ------------------------------------------------------------------ wrappers
 // partial-sum slots of a launch: the coded step's blocks, at least those of the 8-row kernels
 int adjoint_blocks(const Geom& G) {
-  const int R = tile_rows(G);
+  const int R = adjoint_tile_rows(G);
   return ((G.Nx + 31) / 32) * ((G.Ny + R - 1) / R);
 }
 
@@ -1258,7 +1258,7 @@ cudaError_t launch_adjoint_step(const double* X, const double* Lin, double* Lout
                                 cudaStream_t st, const unsigned char* glo, const unsigned char* ghi) {
   dim3 block(32, 8), grid((G.Nx + 31) / 32, (G.Ny + 7) / 8);
   if (codes) {
-    const int R = tile_rows(G);
+    const int R = adjoint_tile_rows(G);
     if (R == 8) launch_adjoint_tile<8>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P, st);
     else if (R == 4) launch_adjoint_tile<4>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P, st);
     else launch_adjoint_tile<2>(X, Lin, Lout, partial, codes, moms, glo, ghi, G, P, st);

@@ -1,5 +1,5 @@
-// dvbm_cellmom.cuh -- moments of the 50 populations of one cell (used by the
-// auxiliary and adjoint kernels; the step kernel accumulates them inline).
+// dvbm_cellmom.cuh -- moments of the 50 populations of one cell in FP64, for
+// the adjoint kernels.
 #pragma once
 #include "dvbm_device.cuh"
 

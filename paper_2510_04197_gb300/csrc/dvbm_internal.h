@@ -37,13 +37,24 @@ inline GhostKinds ghost_kinds(const BCDev& bc) {
   return B;
 }
 // Tile height of the FP64 step.  8 rows share their halo best (2.2 times the rate of
-// 2 rows on a full chip); while the grid's tiles are fewer than the SMs, lower
-// tiles shorten the step by spreading it over more of them, as long as each
-// SM gets no more than one.  Measured, D2Q25, us a step with 8 / 4 / 2 rows: 64^2
-// 41 / 29 / 23 (16 since the low tiles share a cell's coefficients), 128^2
-// 41 / 31 / 33 (23 with 4 rows), 192^2 42 / 41 / 54, 256^2 60 / 69 / 84.
+// 2 rows on a full chip); lower tiles spread a small grid over more SMs and shorten
+// a tile's serial chain.  4 rows as long as the 8-row tiles fit in one wave (three
+// CTAs on each of 152 SMs), 2 rows as long as each SM gets one of them.  Measured,
+// periodic, us a step with 2 / 4 / 8 rows.  D2Q25: 64^2 15.7 / 20.6 / 37.4, 96^2
+// 16.6 / 20.8 / 37.8, 128^2 30.3 / 21.0 / 37.9, 192^2 58 / 31.6 / 39.3, 224^2
+// 81 / 45.7 / 56.5, 288^2 - / 70.4 / 76.4, 352^2 - / 96.4 / 96.8, 416^2 - / 123 / 118,
+// 512^2 - / 184 / 160.  D2Q16: 64^2 11.2 / 15.0 / 27.4, 128^2 14.8 / 15.3 / 27.6, 192^2
+// 28.0 / 21.6 / 27.4, 288^2 - / 50.1 / 53.8, 352^2 - / 67.7 / 66.4, 512^2 - / 131 / 108.
+inline long long tiles8(const Geom& G) { return (long long)((G.Nx + 31) / 32) * ((G.Ny + 7) / 8); }
 inline int tile_rows(const Geom& G) {
-  const long long tiles = (long long)((G.Nx + 31) / 32) * ((G.Ny + 7) / 8);
+  const long long tiles = tiles8(G);
+  return 4 * tiles <= 152 ? 2 : tiles <= 3 * 152 ? 4 : 8;
+}
+// Tile height of the coded adjoint step: 4 rows only while each SM gets one of
+// them (the low tiles' kernel has one CTA of 214 registers on an SM, the 8-row
+// kernel two of 128).
+inline int adjoint_tile_rows(const Geom& G) {
+  const long long tiles = tiles8(G);
   return 4 * tiles <= 152 ? 2 : 2 * tiles <= 152 ? 4 : 8;
 }
 // Does the step kernel write the ghost layers of periodic and zero-gradient sides?

@@ -30,7 +30,6 @@ constexpr int NP = 32;
 __host__ __device__ constexpr double xi(int k) { return k == 0 ? YA : k == 1 ? -YA : k == 2 ? YB : -YB; }
 __host__ __device__ constexpr double w(int k) { return k < 2 ? VA : VB; }
 __host__ __device__ constexpr int sgn(int k) { return (k % 2 == 0) ? 1 : -1; }
-__host__ __device__ constexpr double khq(int k, int n) { return w(k) * he(n, xi(k)) * inv_fact(n); }
 
 struct Mom { double m00, m10, m01, m20, m11, m02, g00, g10, g01; };
 struct Co {

@@ -1,10 +1,10 @@
 // dvbm_step.cu -- the fused time step (Sec. III.A.1, Eq. finalDiscretePDE):
 //     F_new = (1 - dt/tau1) F + W W sum C He He - (dt/dx) v_x dF_x - (dt/dy) v_y dF_y
-// over 32 x 8-cell tiles: moments, combined collision coefficients, the
+// over tiles of cells: moments, combined collision coefficients, the
 // collision target of every population (sum-factorised Grad expansion) and its
 // upwind-limited flux differences.  GB300 has two FP64 lanes per SM, so FP64
 // storage does all of this but the collision coefficients in fixed point on the
-// integer pipes (k_step64); FP32-deviation storage keeps float deviations from
+// integer pipes (k_step_tile); FP32-deviation storage keeps float deviations from
 // a reference state, with the advection in float (k_step32).
 #include "dvbm_device.cuh"
 #include "dvbm_internal.h"

@@ -23,7 +23,7 @@ def D():
 
 
 # tiles of 2, 4 and 8 rows, ragged along both axes
-@pytest.mark.parametrize("Nx,Ny", [(5, 7), (63, 61), (130, 75), (331, 97)])
+@pytest.mark.parametrize("Nx,Ny", [(5, 7), (63, 61), (130, 75), (331, 97), (352, 385)])
 @pytest.mark.parametrize("kind", ["periodic", "open"])
 @pytest.mark.parametrize("lattice,storage", [(0, 0), (0, 1), (1, 0)])
 def test_back_to_back_steps_equal_single_steps(D, Nx, Ny, kind, lattice, storage):
