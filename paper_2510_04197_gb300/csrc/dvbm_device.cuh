@@ -112,8 +112,9 @@ __device__ __forceinline__ EqF eq_f(double rho, double ux, double uy, double s) 
   e.a20 = fma(e.a10, ux, rs);
   e.a11 = e.a10 * uy;
   e.a02 = fma(e.a01, uy, rs);
-  e.a30 = fma(e.a20, ux, 2.0 * s * e.a10);
-  e.a03 = fma(e.a02, uy, 2.0 * s * e.a01);
+  const double rs2 = rs + rs;
+  e.a30 = ux * (e.a20 + rs2);
+  e.a03 = uy * (e.a02 + rs2);
   e.a21 = e.a20 * uy;
   e.a12 = e.a02 * ux;
   e.a40 = fma(e.a30, ux, 3.0 * s * e.a20);
