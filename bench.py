@@ -548,7 +548,7 @@ def main():
     roofline = {"bound": "hbm", "achieved": ach_gbs, "peak": hbm_peak, "unit": "GB/s",
                 "frac": ach_gbs / hbm_peak, "frac_of_8tbs": ach_gbs / NOMINAL_HBM_GBS,
                 "traffic": (tr["dram_bytes_per_cell"] * N * N if tr else None),
-                "kernel": "k_step<double> (FP64 storage, D2Q25 split II)",
+                "kernel": "k_step_tile (FP64 storage, D2Q25 split II)",
                 "what": "algorithmic 800 B per cell update x cells / step-kernel time (CUDA events); peak = "
                         + ("MEASURED_PEAKS.json hbm_gbs (of measured)" if peak_kind == "measured"
                            else "fallback 6.8 TB/s (of fallback)")}

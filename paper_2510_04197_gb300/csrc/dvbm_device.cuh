@@ -1029,10 +1029,10 @@ __device__ __forceinline__ void write_images(S* p, long long PL, int x, int y, c
 }
 
 // What bounds it: the integer ALU (about two thirds busy) beside the FP64 pipe
-// (about half) and the latency between them; DRAM is at a fifth of its rate.
-// D2Q25: 12.4 k instructions and 186 FP64 ones a cell, against 26.8 k and 407 of a
+// (57 %) and the latency between them; DRAM is at 38 % of its rate (the flux sums
+// leave L2 in part: 1571 B a cell).  D2Q25: 13.2 k instructions and 186 FP64 ones a cell, against 26.8 k and 407 of a
 // thread per cell with its own stencils: 15.5 -> 8.4 ms a step at 4096^2, 1.02 ->
-// 0.54 ms at 1024^2.  D2Q16: 10.5 -> 6.0 ms and 0.70 -> 0.39 ms.  Three CTAs of 80
+// 0.54 ms at 1024^2.  D2Q16: 10.5 -> 5.6 ms and 0.70 -> 0.37 ms.  Three CTAs of 80
 // registers; four of 64 measured 1 % slower.
 // L: the lattice (Lat25, Lat16).  PRC: Prandtl branch; RAT: rational limiter;
 // CODES: also the branch codes of every population's slopes (one byte x | y << 2
