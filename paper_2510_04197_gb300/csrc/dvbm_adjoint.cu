@@ -598,14 +598,14 @@ __device__ __forceinline__ int adjoint_walk(const AdjointLoad<R>& L, const Next&
   if (MX) key = max(key, ((unsigned)__double2hiint(L.h) + 0x100000u) & 0x7fffffffu);
   key = __reduce_max_sync(0xffffffffu, key);
   const int E = (int)(key >> 20) - 1;
-  const int n0 = E < 128 ? 63 : P.advn + 3;
+  const BlockScale B(E, P.advn + 3);
   __syncwarp();
 #pragma unroll
-  for (int j = J0; j <= J1; ++j) xs[(j + 1) * kAdvPitch + lane + 1] = block_fix(L.v[j + 1], E, n0);
+  for (int j = J0; j <= J1; ++j) xs[(j + 1) * kAdvPitch + lane + 1] = block_fix(L.v[j + 1], B);
   const int hr = lane % R, hc = lane / R;
   if (MX) {
     __syncwarp();
-    if (hc < 3 && hr < T.H) xs[(hr + 1) * kAdvPitch + (hc == 0 ? 0 : T.W + hc)] = block_fix(L.h, E, n0);
+    if (hc < 3 && hr < T.H) xs[(hr + 1) * kAdvPitch + (hc == 0 ? 0 : T.W + hc)] = block_fix(L.h, B);
   }
   unsigned xb = 0, yb = 0;  // codes of rows 0 .. R - 1 (x), -1 .. R (y), two bits each
 #pragma unroll
@@ -699,16 +699,16 @@ __device__ __forceinline__ void project(const double* __restrict__ lam, const do
     key = max(key, ((unsigned)__double2hiint(v[i]) + 0x100000u) & 0x7fffffffu);
   }
   const int E = (int)(key >> 20) - 1;
-  const int n0 = E < 128 ? 63 : 2;
+  const BlockScale B(E, 2);
   long long c[N + 1], s[2][N + 1], d[2][N + 1];  // y-projections: centre node, sums and differences of the node pairs
 #pragma unroll
   for (int p = 0; p < 5; ++p) {
     long long h[N + 1];
 #pragma unroll
     for (int q = 0; q < 5; ++q) a1b = fma(v[5 * p + q], __ldg(at(X + (5 * p + q) * PL, off)), a1b);
-    const long long l0 = block_fix(v[5 * p], E, n0), l1 = block_fix(v[5 * p + 1], E, n0),
-                    l2 = block_fix(v[5 * p + 2], E, n0), l3 = block_fix(v[5 * p + 3], E, n0),
-                    l4 = block_fix(v[5 * p + 4], E, n0);
+    const long long l0 = block_fix(v[5 * p], B), l1 = block_fix(v[5 * p + 1], B),
+                    l2 = block_fix(v[5 * p + 2], B), l3 = block_fix(v[5 * p + 3], B),
+                    l4 = block_fix(v[5 * p + 4], B);
     const Limbs z(l0), sA(l1 + l2), dA(l1 - l2), sB(l3 + l4), dB(l3 - l4);
     LimbAcc a0, a1, a2;
     k0mac<0, 0>(a0, z); k0mac<1, 0>(a0, sA); k0mac<2, 0>(a0, sB);
@@ -774,11 +774,10 @@ __device__ __forceinline__ int scale_moments(const double (&m)[N], long long (&Q
   unsigned key = 0;
 #pragma unroll
   for (int i = 0; i < N; ++i) key = max(key, abs_key(m[i]));
-  const int E = (int)(key >> 20);
-  const int n0 = E < 128 ? 63 : 2;
+  const BlockScale B((int)(key >> 20), 2);
 #pragma unroll
-  for (int i = 0; i < N; ++i) Q[i] = block_fix(m[i], E, n0);
-  return E;
+  for (int i = 0; i < N; ++i) Q[i] = block_fix(m[i], B);
+  return max(B.E, 128);  // as in fields_to_smem
 }
 
 // BAND: a band of a slab-decomposed grid, whose code rows beyond its edges are glo

@@ -440,26 +440,35 @@ __device__ __forceinline__ long long pack_limbs(long long x) { return x + ((x & 
 __device__ __forceinline__ unsigned abs_key(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 __device__ __forceinline__ unsigned abs_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 
+// How a block of largest exponent E enters fixed point.  Below 2^-895 (E < 128) the
+// block is negligible: its integers' units would leave the range of doubles, so that
+// every value of it, of either sign, has to become exactly 0 (an integer of one unit
+// scaled below the smallest exponent wraps into numbers near 2^1000).
+struct BlockScale {
+  int E, n0, sign;  // exponent, dropped bits (63: all), mask of the values' signs
+  __device__ __forceinline__ BlockScale(int E_, int bits, int tiny = 128)
+      : E(E_), n0(E_ < tiny ? 63 : bits), sign(E_ < tiny ? 0 : -1) {}
+};
 // Value v as an integer of 60 - n0 bits at the block exponent E (n0 >= 0):
 // v = X 2^(E - 1082 + n0); magnitudes are truncated, negative values are the
 // ones' complement of theirs (one unit more).  A value of larger exponent than
-// E (only non-finite ones are left out of the block maximum) gives 0.
-__device__ __forceinline__ long long block_fix(double v, int E, int n0) {
+// E (only non-finite ones are left out of the block maximum) gives 0 or -1.
+__device__ __forceinline__ long long block_fix(double v, const BlockScale& B) {
   const int hi = __double2hiint(v);
   const unsigned lo = (unsigned)__double2loint(v);
   const int e = (hi >> 20) & 0x7ff;
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
   const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 7;
-  const unsigned n = min((unsigned)(E - e + n0), 63u);
-  return (long long)(m >> n) ^ (long long)(hi >> 31);
+  const unsigned n = min((unsigned)(B.E - e + B.n0), 63u);
+  return (long long)(m >> n) ^ (long long)((hi >> 31) & B.sign);
 }
 // the same for a float: v = X 2^(E - 186 + n0)
-__device__ __forceinline__ long long block_fix(float v, int E, int n0) {
+__device__ __forceinline__ long long block_fix(float v, const BlockScale& B) {
   const int u = __float_as_int(v);
   const int e = (u >> 23) & 0xff;
   const unsigned mh = (((unsigned)u & 0x7fffffu) | 0x800000u) << 4;
-  const unsigned n = min((unsigned)(E - e + n0), 63u);
-  return (long long)(((unsigned long long)mh << 32) >> n) ^ (long long)(u >> 31);
+  const unsigned n = min((unsigned)(B.E - e + B.n0), 63u);
+  return (long long)(((unsigned long long)mh << 32) >> n) ^ (long long)((u >> 31) & B.sign);
 }
 
 // int64 -> double by bit manipulation, value F 2^scale: one count of leading
@@ -524,13 +533,13 @@ __device__ __forceinline__ void moments_fix_f(const S* __restrict__ s, unsigned 
     key = max(key, abs_key(v[i]));
   }
   const int E = (int)(key >> K::kExpBits);
-  const int n0 = E < K::kTiny ? 63 : 2;
+  const BlockScale B(E, 2, K::kTiny);
   long long M0[5], M1[5], M2[5], M3s = 0;  // y-sums of each x-node, M1, M2, M3 times 1/16, 1/64, 1/128
 #pragma unroll
   for (int p = 0; p < 5; ++p) {
-    const long long x0 = block_fix(v[5 * p], E, n0), x1 = block_fix(v[5 * p + 1], E, n0),
-                    x2 = block_fix(v[5 * p + 2], E, n0), x3 = block_fix(v[5 * p + 3], E, n0),
-                    x4 = block_fix(v[5 * p + 4], E, n0);
+    const long long x0 = block_fix(v[5 * p], B), x1 = block_fix(v[5 * p + 1], B),
+                    x2 = block_fix(v[5 * p + 2], B), x3 = block_fix(v[5 * p + 3], B),
+                    x4 = block_fix(v[5 * p + 4], B);
     const long long sA = x1 + x2, dA = x1 - x2, sB = x3 + x4, dB = x3 - x4;
     M0[p] = x0 + sA + sB;
     M1[p] = pair_sum<1>(dB, dA);
@@ -565,13 +574,13 @@ __device__ __forceinline__ void moments_fix_g(const S* __restrict__ s, unsigned 
     key = max(key, abs_key(v[i]));
   }
   const int E = (int)(key >> K::kExpBits);
-  const int n0 = E < K::kTiny ? 63 : 2;
+  const BlockScale B(E, 2, K::kTiny);
   long long N0[5], N1s = 0;
 #pragma unroll
   for (int p = 0; p < 5; ++p) {
-    const long long x0 = block_fix(v[5 * p], E, n0), x1 = block_fix(v[5 * p + 1], E, n0),
-                    x2 = block_fix(v[5 * p + 2], E, n0), x3 = block_fix(v[5 * p + 3], E, n0),
-                    x4 = block_fix(v[5 * p + 4], E, n0);
+    const long long x0 = block_fix(v[5 * p], B), x1 = block_fix(v[5 * p + 1], B),
+                    x2 = block_fix(v[5 * p + 2], B), x3 = block_fix(v[5 * p + 3], B),
+                    x4 = block_fix(v[5 * p + 4], B);
     N0[p] = x0 + (x1 + x2) + (x3 + x4);
     N1s += pair_sum<1>(x3 - x4, x1 - x2);
   }
@@ -743,13 +752,13 @@ __device__ __forceinline__ int advect_tile(AdvLoad<R>& L, const Next& next, long
   if (MX) key = max(key, ((unsigned)__double2hiint(vh) + 0x100000u) & 0x7fffffffu);
   key = __reduce_max_sync(0xffffffffu, key);
   const int E = (int)(key >> 20) - 1;
-  const int n0 = E < 128 ? 63 : P.advn;  // a block of negligible values has no flux
+  const BlockScale B(E, P.advn);  // a block of negligible values has no flux
   __syncwarp();                          // the previous population's reads of xs are done
 #pragma unroll
-  for (int j = J0; j <= J1; ++j) xs[(j + 2) * kAdvPitch + lane + 2] = block_fix(v[j - J0], E, n0);
+  for (int j = J0; j <= J1; ++j) xs[(j + 2) * kAdvPitch + lane + 2] = block_fix(v[j - J0], B);
   if (MX) {
     __syncwarp();  // column W of a ragged tile is written twice: the halo value last
-    if (hin) xs[(hr + 2) * kAdvPitch + (hc == 2 ? T.W + 2 : hc)] = block_fix(vh, E, n0);
+    if (hin) xs[(hr + 2) * kAdvPitch + (hc == 2 ? T.W + 2 : hc)] = block_fix(vh, B);
   }
   next();
   __syncwarp();
@@ -857,10 +866,10 @@ __device__ __forceinline__ void fields_to_smem(const double (&f)[N], long long* 
   unsigned key = 0;
 #pragma unroll
   for (int k = 0; k < N; ++k) key = max(key, abs_key(f[k]));
-  E = (int)(key >> 20);
-  const int n0 = E < 128 ? 63 : 0;  // negligible coefficients: target 0
+  const BlockScale B((int)(key >> 20), 0);  // negligible coefficients: target 0
 #pragma unroll
-  for (int k = 0; k < N; ++k) b[k * STRIDE] = pack_limbs(block_fix(f[k], E, n0));
+  for (int k = 0; k < N; ++k) b[k * STRIDE] = pack_limbs(block_fix(f[k], B));
+  E = max(B.E, 128);  // a zero target's exponent too lies where collide_advect's result is normal
 }
 // h^b of x-node p: W_p sum_a C_ab He_a(xi_p)/a! (value h 2^(E - 1082 - kd(p)))
 template <class V>

@@ -178,13 +178,13 @@ __device__ __forceinline__ void moments_fix16(const double* __restrict__ s, unsi
     key = max(key, abs_key(v[i]));
   }
   const int E = (int)(key >> 20);
-  const int n0 = E < 128 ? 63 : 2;
+  const BlockScale B(E, 2);
   const int sc = E - 1080;
   long long M0[4], M1[4], M2s = 0;  // y-sums of each x-node, M1 and M2 times 1/16, 1/32
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
-    const long long x0 = block_fix(v[4 * p], E, n0), x1 = block_fix(v[4 * p + 1], E, n0),
-                    x2 = block_fix(v[4 * p + 2], E, n0), x3 = block_fix(v[4 * p + 3], E, n0);
+    const long long x0 = block_fix(v[4 * p], B), x1 = block_fix(v[4 * p + 1], B),
+                    x2 = block_fix(v[4 * p + 2], B), x3 = block_fix(v[4 * p + 3], B);
     const long long sA = x0 + x1, dA = x0 - x1, sB = x2 + x3, dB = x2 - x3;
     M0[p] = sA + sB;
     M1[p] = pair_sum16<1>(dB, dA);
