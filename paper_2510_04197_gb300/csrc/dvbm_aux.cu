@@ -228,8 +228,13 @@ __global__ void __launch_bounds__(256) k_speed(const double* __restrict__ rho, c
   double mx = 0.0, bad = 0.0, pm = 0.0;
   // The FP64 square roots (about 50 instructions of the FP64 pipe) are taken
   // only where a single-precision estimate (relative error below 2^-21) could
-  // exceed the maximum so far; the input tests compare bit patterns.
-  const float gR = (float)(M.gamma * M.R), R = (float)M.R;
+  // exceed the maximum so far; the input tests compare bit patterns.  What a
+  // product or a conversion loses below the smallest float stays under 2^-60 of
+  // the estimate (factors gamma R, R within 2^+-30, rho and T below 2^60 for the
+  // pressure), so it is used against maxima above 2^-30 only: otherwise mxf, pmf
+  // are 0 and every cell is evaluated in FP64.
+  const float gR = (float)(M.gamma * M.R), R = (float)M.R, lowest = 0x1p-30f, highest = 0x1p30f;
+  const bool est = gR > lowest && gR < highest && R > lowest && R < highest;
   const unsigned long long big = (unsigned long long)__double_as_longlong(1e300);
   auto positive = [&](double v) { return (unsigned long long)__double_as_longlong(v) - 1ull < big - 1ull; };
   auto bounded = [&](double v) { return ((unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull) < big; };
@@ -243,11 +248,12 @@ __global__ void __launch_bounds__(256) k_speed(const double* __restrict__ rho, c
     const float af = (float)a, bf = (float)b, tf = (float)t;
     if (!((sqrtf(af * af + bf * bf) + sqrtf(gR * tf)) * 1.000001f < mxf)) {
       mx = fmax(mx, sqrt(a * a + b * b) + sqrt(M.gamma * M.R * t));
-      mxf = (float)mx;
+      mxf = est && (float)mx > lowest ? (float)mx : 0.f;
     }
-    if (!((float)r * R * tf * 1.000001f < pmf)) {
+    const float rf = (float)r;
+    if (!(rf * R * tf * 1.000001f < pmf) || fmaxf(rf, tf) >= 0x1p60f) {
       pm = fmax(pm, r * M.R * t);
-      pmf = (float)pm;
+      pmf = est && (float)pm > lowest ? (float)pm : 0.f;
     }
   }
   __shared__ double sm[256], sb[256], sp[256];
