@@ -275,6 +275,15 @@ dvbm_status dvbm_halo_unpack(dvbm_ctx* ctx, const void* lo, const void* hi);
  * run that has stepped). */
 dvbm_status dvbm_set_dt(dvbm_ctx* ctx, double dt);
 
+/* Rows of the whole grid that this context holds a band of (default: its own
+ * Ny).  The step and adjoint kernels work on tiles of 32 x 2, 4 or 8 cells,
+ * chosen by the grid's size, whose cells share a block exponent; with the whole
+ * grid's rows set in every band, bands that begin and end on multiples of 8 rows
+ * (the last one ends with the grid) give bitwise the undecomposed run.  Without
+ * it they agree to rounding.  Errors: EINVAL (rows < Ny), ESTATE (a stepwise
+ * adjoint in progress or a recorded run that has stepped, and rows differs). */
+dvbm_status dvbm_set_grid_rows(dvbm_ctx* ctx, int rows);
+
 /* Time step size fixed at dvbm_init (0 before). */
 double dvbm_dt(const dvbm_ctx* ctx);
 

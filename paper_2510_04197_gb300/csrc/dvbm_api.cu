@@ -229,6 +229,7 @@ extern "C" dvbm_status dvbm_create(dvbm_ctx** out, int lattice, int Nx, int Ny, 
   c->G.xoff = align;
   c->G.pitch = ((Nx + align + 2 + align - 1) / align) * align;
   c->G.plane = (long long)(Ny + 4) * c->G.pitch;
+  c->G.grid_rows = Ny;
   const double c2 = o.R * o.T_ref;
   c->M.c = std::sqrt(c2); c->M.T_ref = o.T_ref; c->M.R = o.R; c->M.gamma = gamma;
   c->P.c2 = c2; c->P.inv_c2 = 1.0 / c2;
@@ -670,6 +671,18 @@ extern "C" dvbm_status dvbm_set_dt(dvbm_ctx* c, double dt) {
   if (s != DVBM_OK) return s;
   c->dt = dt;
   set_step_factors(c);
+  return DVBM_OK;
+}
+
+extern "C" dvbm_status dvbm_set_grid_rows(dvbm_ctx* c, int rows) {
+  if (!c) return DVBM_EINVAL;
+  if (rows < c->Ny) return fail(c, DVBM_EINVAL, "a grid of %d rows cannot hold this band of %d", rows, c->Ny);
+  if (rows == c->G.grid_rows) return DVBM_OK;
+  // the adjoint recomputes the recorded run with the context's tiles, and a pass in
+  // progress has sized its partial sums by them
+  if (c->adj.active || (c->recorded && c->steps > 0))
+    return fail(c, DVBM_ESTATE, "the recorded run has taken steps: the grid's rows cannot change now");
+  c->G.grid_rows = rows;
   return DVBM_OK;
 }
 

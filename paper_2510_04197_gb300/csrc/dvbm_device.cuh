@@ -50,6 +50,7 @@ struct Geom {
   int pitch;             // elements per row (ghost columns included)
   int xoff;              // element offset of x = 0 inside a row
   long long plane;       // elements per population plane = (Ny + 4) * pitch
+  int grid_rows;         // rows of the whole grid (Ny, or more for a band of it): fixes the tile heights
 };
 
 struct Phys {

@@ -45,7 +45,11 @@ inline GhostKinds ghost_kinds(const BCDev& bc) {
 // 81 / 45.7 / 56.5, 288^2 - / 70.4 / 76.4, 352^2 - / 96.4 / 96.8, 416^2 - / 123 / 118,
 // 512^2 - / 184 / 160.  D2Q16: 64^2 11.2 / 15.0 / 27.4, 128^2 14.8 / 15.3 / 27.6, 192^2
 // 28.0 / 21.6 / 27.4, 288^2 - / 50.1 / 53.8, 352^2 - / 67.7 / 66.4, 512^2 - / 131 / 108.
-inline long long tiles8(const Geom& G) { return (long long)((G.Nx + 31) / 32) * ((G.Ny + 7) / 8); }
+// A band counts the tiles of the whole grid: a tile's cells share a block exponent,
+// so bands of whole 8-row tiles are bitwise the undecomposed run only with its tiles
+// (a band of 192 rows of 192 columns then takes 39.3 us a step instead of 31.6 where
+// the whole grid has 8-row tiles).
+inline long long tiles8(const Geom& G) { return (long long)((G.Nx + 31) / 32) * ((G.grid_rows + 7) / 8); }
 inline int tile_rows(const Geom& G) {
   const long long tiles = tiles8(G);
   return 4 * tiles <= 152 ? 2 : tiles <= 3 * 152 ? 4 : 8;

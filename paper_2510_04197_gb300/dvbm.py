@@ -69,6 +69,7 @@ SIGNATURES = {
     "dvbm_halo_pack": (_CI, [_VP, _VP, _VP]),
     "dvbm_halo_unpack": (_CI, [_VP, _VP, _VP]),
     "dvbm_set_dt": (_CI, [_VP, _CD]),
+    "dvbm_set_grid_rows": (_CI, [_VP, _CI]),
     "dvbm_cfl_dt_noalloc": (_CI, [_VP, _VP, _VP, _VP, ctypes.c_longlong, _CD, _CD, _CD, _CD, _VP, _DP]),
 }
 
@@ -348,6 +349,11 @@ class Simulation:
 
     def set_dt(self, dt: float):
         _check(lib().dvbm_set_dt(self._h, float(dt)), self._h)
+        return self
+
+    def set_grid_rows(self, rows: int):
+        """Rows of the whole grid this context is a band of (its tile heights)."""
+        _check(lib().dvbm_set_grid_rows(self._h, int(rows)), self._h)
         return self
 
     @property

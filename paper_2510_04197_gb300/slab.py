@@ -48,9 +48,9 @@ def neighbours(rank: int, world: int, periodic: bool):
 
 def split_rows(Ny: int, parts: int, align: int = 8) -> List[int]:
     """Band heights summing to Ny: multiples of ``align`` where possible (the
-    step kernel's tile height, so that bands tile the grid exactly as the
-    undecomposed run does), the remainder on the last band; every band keeps
-    at least 4 rows."""
+    largest tile height of the step kernels, so that bands that know the whole
+    grid's rows (``dvbm_set_grid_rows``) tile it exactly as the undecomposed run
+    does), the remainder on the last band; every band keeps at least 4 rows."""
     if parts < 1 or Ny < 4 * parts:
         raise ValueError(f"cannot split {Ny} rows into {parts} bands of >= 4 rows")
     base = max(align * (Ny // (parts * align)), 4) if align > 0 else Ny // parts
@@ -119,7 +119,7 @@ class LocalSlabs:
         for k, h in enumerate(self.heights):
             bk, self.periodic = band_bcs(bcs, k, len(self.heights))
             self.sims.append(D.Simulation(self.Nx, h, Pr, gamma, mu, bcs=bk, storage=storage, lattice=lattice,
-                                          Lx=Lx, Ly=dy * h, **opts))
+                                          Lx=Lx, Ly=dy * h, **opts).set_grid_rows(self.Ny))
         n = len(self.sims)
         self.nb = [neighbours(k, n, self.periodic) for k in range(n)]
         self.out_lo = [s.halo_buffer() for s in self.sims]
@@ -224,8 +224,8 @@ class LocalSlabs:
 
 class RankSlab:
     """Band ``rank`` of a grid split over ``world`` processes (one GPU each),
-    halos exchanged with ``exchange`` (NCCL), dt and totals reduced over the
-    process group."""
+    halos exchanged with ``exchange`` (NCCL), dt, the grid's rows (at ``init``)
+    and totals reduced over the process group."""
 
     def __init__(self, dist, Nx: int, Ny_band: int, Pr: float, gamma: float, mu: float, bcs=None,
                  storage: int = D.FP64, lattice: int = D.D2Q25_SPLIT_II, **opts):
@@ -249,6 +249,9 @@ class RankSlab:
 
     def init(self, rho, ux, uy, T):
         import torch
+        rows = torch.tensor([self.sim.Ny], dtype=torch.int64, device=self.sim.device)
+        self.dist.all_reduce(rows, op=self.dist.ReduceOp.SUM)
+        self.sim.set_grid_rows(int(rows.item()))
         self.sim.init(rho, ux, uy, T)
         if not self.fixed_dt:
             t = torch.tensor([self.sim.dt], dtype=torch.float64, device=self.sim.device)
