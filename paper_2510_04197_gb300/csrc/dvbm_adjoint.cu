@@ -737,13 +737,13 @@ __device__ __forceinline__ void project(const double* __restrict__ lam, const do
   [&] {                                                                                         \
     LimbAcc t;                                                                                  \
     k0mac<0, a>(t, Limbs(c[b])); k0mac<1, a>(t, Limbs(s[0][b])); k0mac<2, a>(t, Limbs(s[1][b])); \
-    return fix_to_double<true>(t.value8(), sc);                                                 \
+    return fix_to_double(t.value8(), sc);                                                 \
   }()
 #define DVBM_ODD(a, b)                                                \
   [&] {                                                               \
     LimbAcc t;                                                        \
     k0mac<1, a>(t, Limbs(d[0][b])); k0mac<2, a>(t, Limbs(d[1][b]));   \
-    return fix_to_double<true>(t.value8(), sc);                       \
+    return fix_to_double(t.value8(), sc);                       \
   }()
   if constexpr (N == 4) {
     // f00, f10, f01, f20, f11, f02, f30, f21, f12, f03, f40, f31, f22, f13, f04

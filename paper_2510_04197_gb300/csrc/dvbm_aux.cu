@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kCta, 3) k_init(S* __restrict__ dst, const dou
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
         S* o = d + (NF * k + NQ * p + q) * PL;
-        if constexpr (sizeof(S) == 8) *o = fix_to_double<true>(t[q], sc - LT::kdp(q));
+        if constexpr (sizeof(S) == 8) *o = fix_to_double(t[q], sc - LT::kdp(q));
         else *o = ll_to_float_rn(t[q], sc - LT::kdp(q));
       }
     }
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kCta, 2) k_wall(S* __restrict__ buf, Geom G, P
 #pragma unroll
     for (int q = 0; q < NQ; ++q) {
       const long long o = (NF * k + NQ * p + q) * PL;
-      g[o] = (S)((double)b[o] + fix_to_double<true>(v[q], sc - LT::kdp(q)));
+      g[o] = (S)((double)b[o] + fix_to_double(v[q], sc - LT::kdp(q)));
     }
   }
 }

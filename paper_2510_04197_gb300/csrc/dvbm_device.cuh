@@ -143,8 +143,8 @@ __device__ __forceinline__ double recip(double x) {
   return fma(r, fma(e, e, e), r);
 }
 
-// v > 0 and |v| < 1e300 (false for NaN) on the bit patterns: a comparison of doubles
-// takes a slot of the FP64 pipe
+// v > 0 (true for +inf, false for NaN) and |v| < 1e300 (false for NaN) on the bit
+// patterns: a comparison of doubles takes a slot of the FP64 pipe
 __device__ __forceinline__ bool is_positive(double v) {
   return (unsigned long long)__double_as_longlong(v) - 1ull < 0x7ff0000000000000ull;
 }
@@ -376,10 +376,10 @@ __device__ __forceinline__ T* at(T* base, unsigned off) {
 // The short kernels of a step (tiles below 8 rows, ghost layers, walls) are
 // launched while the kernel before them in the stream still runs
 // (launch_chained), and wait here until it has completed and its writes are
-// visible: 64^2 17.8 -> 16.5 us a step, 4 x 256 with walls 29.4 -> 27.7.  Their own
-// successor is let in after that, so that at most one waits.  p: the kernel's input, which later loads then depend on; the data
-// changes after the kernel's start, so it is read by plain loads (load), never
-// by the read-only path.
+// visible, which spares 1.3 us of a 64^2 step and 1.7 us of one on 4 x 256 with walls.
+// Their own successor is let in after that, so that at most one waits.  p: the
+// kernel's input, which later loads then depend on; the data changes after the
+// kernel's start, so it is read by plain loads (load), never by the read-only path.
 template <class T>
 __device__ __forceinline__ T* chain_wait(T* p) {
   asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" : "+l"(p) : : "memory");
@@ -473,11 +473,9 @@ __device__ __forceinline__ long long block_fix(float v, const BlockScale& B) {
 }
 
 // int64 -> double by bit manipulation, value F 2^scale: one count of leading
-// zeros on the word that holds the leading one.  RN rounds to nearest (ties
-// away), otherwise the bits below 2^-52 of the value are dropped; a negative F
-// counts one unit less in magnitude (see block_fix).  The value's exponent must
-// lie in the normal range.
-template <bool RN>
+// zeros on the word that holds the leading one, rounded to nearest (ties away); a
+// negative F counts one unit less in magnitude (see block_fix).  The value's
+// exponent must lie in the normal range.
 __device__ __forceinline__ double fix_to_double(long long F, int scale) {
   const int s = (int)(F >> 63);
   const unsigned hi = (unsigned)(int)(F >> 32) ^ (unsigned)s, lo = (unsigned)F ^ (unsigned)s;
@@ -487,7 +485,7 @@ __device__ __forceinline__ double fix_to_double(long long F, int scale) {
   // leading one at bit 62 (|F| < 2^62); a carry out of the rounded significand
   // goes into the exponent below, which is exactly right
   const unsigned long long norm = ((((unsigned long long)hi) << 32) | lo) << ((n - 1) & 63);
-  const unsigned long long r = (norm + (RN ? 0x200u : 0u)) >> 10;
+  const unsigned long long r = (norm + 0x200u) >> 10;
   const unsigned rh = (unsigned)(r >> 32) + ((unsigned)(1023 + 62 - n + scale) << 20);
   const double v = __hiloint2double((int)(rh | ((unsigned)s & 0x80000000u)), (int)(unsigned)r);
   return top == 0u ? 0.0 : v;
@@ -552,16 +550,16 @@ __device__ __forceinline__ void moments_fix_f(const S* __restrict__ s, unsigned 
   const long long a1 = M1[1] + M1[2], b1 = M1[3] + M1[4], c1 = M1[1] - M1[2], d1 = M1[3] - M1[4];
   const long long a2 = M2[1] + M2[2], b2 = M2[3] + M2[4], c2 = M2[1] - M2[2], d2 = M2[3] - M2[4];
   const int sc = E - K::kBias;
-  m.m00 = fix_to_double<true>(M0[0] + a0 + b0, sc);
-  m.m01 = fix_to_double<true>(M1[0] + a1 + b1, sc + 4);
-  m.m02 = fix_to_double<true>(M2[0] + a2 + b2, sc + 6);
-  m.m03 = fix_to_double<true>(M3s, sc + 7);
-  m.m10 = fix_to_double<true>(pair_sum<1>(d0, c0), sc + 4);
-  m.m20 = fix_to_double<true>(pair_sum<2>(b0, a0), sc + 6);
-  m.m30 = fix_to_double<true>(pair_sum<3>(d0, c0), sc + 7);
-  m.m11 = fix_to_double<true>(pair_sum<1>(d1 << 4, c1 << 4), sc + 4);
-  m.m21 = fix_to_double<true>(pair_sum<2>(b1 << 4, a1 << 4), sc + 6);
-  m.m12 = fix_to_double<true>(pair_sum<1>(d2 << 4, c2 << 4), sc + 6);
+  m.m00 = fix_to_double(M0[0] + a0 + b0, sc);
+  m.m01 = fix_to_double(M1[0] + a1 + b1, sc + 4);
+  m.m02 = fix_to_double(M2[0] + a2 + b2, sc + 6);
+  m.m03 = fix_to_double(M3s, sc + 7);
+  m.m10 = fix_to_double(pair_sum<1>(d0, c0), sc + 4);
+  m.m20 = fix_to_double(pair_sum<2>(b0, a0), sc + 6);
+  m.m30 = fix_to_double(pair_sum<3>(d0, c0), sc + 7);
+  m.m11 = fix_to_double(pair_sum<1>(d1 << 4, c1 << 4), sc + 4);
+  m.m21 = fix_to_double(pair_sum<2>(b1 << 4, a1 << 4), sc + 6);
+  m.m12 = fix_to_double(pair_sum<1>(d2 << 4, c2 << 4), sc + 6);
   if (key >= K::kInf) m.m00 = __longlong_as_double(0x7ff8000000000000ll);
 }
 template <class S, bool NC = true>
@@ -586,9 +584,9 @@ __device__ __forceinline__ void moments_fix_g(const S* __restrict__ s, unsigned 
     N1s += pair_sum<1>(x3 - x4, x1 - x2);
   }
   const int sc = E - K::kBias;
-  m.g00 = fix_to_double<true>(N0[0] + (N0[1] + N0[2]) + (N0[3] + N0[4]), sc);
-  m.g01 = fix_to_double<true>(N1s, sc + 4);
-  m.g10 = fix_to_double<true>(pair_sum<1>(N0[3] - N0[4], N0[1] - N0[2]), sc + 4);
+  m.g00 = fix_to_double(N0[0] + (N0[1] + N0[2]) + (N0[3] + N0[4]), sc);
+  m.g01 = fix_to_double(N1s, sc + 4);
+  m.g10 = fix_to_double(pair_sum<1>(N0[3] - N0[4], N0[1] - N0[2]), sc + 4);
   if (key >= K::kInf) m.g00 = __longlong_as_double(0x7ff8000000000000ll);
 }
 template <class S>
@@ -640,7 +638,9 @@ __device__ __forceinline__ long long to_block_fixed52(double v, int E) {
 // The update's flux differences (Sec. III.A.2) of one population over a tile of
 // up to 32 x R cells, by one warp, in block fixed point: the tile's cells and
 // its upwind halo share one exponent, so every value is converted once (a
-// per-cell stencil converts eight values per cell), differences are exact, and
+// per-cell stencil converts eight values per cell), to integers in units of
+// 2^-(58 - L) of the largest (L: Phys::advn - 1; 2^-55 at beta = 6/5): exact for
+// values within 2^(6 - L) of it, truncated below.  Differences are exact, and
 // each limited slope is computed once and handed to the neighbour (along x by
 // a warp shuffle, along y in registers while the warp walks the rows).
 //
@@ -997,7 +997,7 @@ struct Lat25 {
 // population in fixed point, and the update with the flux sum (collide_advect).
 // Low tiles (R < 8, small grids) also write the periodic and zero-gradient ghost
 // images of the cells next to the grid's edge, so that a step without walls is
-// one launch (64^2: 25 -> 21 us).  In the 8-row kernel the same code costs 6 %: its
+// one launch (4 us less at 64^2).  In the 8-row kernel the same code costs 6 %: its
 // divergent tail keeps the compiler off the uniform registers for addresses.
 //  * Advection: warp w does f (w < 4) or g.  D2Q25: x-node p = 1 + w % 4, its four
 //    populations that move along both axes, (p, 0) along x only and (0, p) along
@@ -1040,9 +1040,9 @@ __device__ __forceinline__ void write_images(S* p, long long PL, int x, int y, c
 
 // What bounds it: the integer ALU (about two thirds busy) beside the FP64 pipe
 // (57 %) and the latency between them; DRAM is at 38 % of its rate (the flux sums
-// leave L2 in part: 1571 B a cell).  D2Q25: 13.2 k instructions and 186 FP64 ones a cell, against 26.8 k and 407 of a
-// thread per cell with its own stencils: 15.5 -> 8.4 ms a step at 4096^2, 1.02 ->
-// 0.54 ms at 1024^2.  D2Q16: 10.5 -> 5.6 ms and 0.70 -> 0.37 ms.  Three CTAs of 80
+// leave L2 in part: about 1.6 kB a cell).  D2Q25: 13.2 k instructions and 186 FP64 ones
+// a cell (conversions counted), against 26.8 k and 407 of a thread per cell with its
+// own stencils: 15.5 -> 8.4 ms a step at 4096^2, 1.02 -> 0.54 ms at 1024^2.  D2Q16: 10.5 -> 5.6 ms and 0.70 -> 0.37 ms.  Three CTAs of 80
 // registers; four of 64 measured 1 % slower.
 // L: the lattice (Lat25, Lat16).  PRC: Prandtl branch; RAT: rational limiter;
 // CODES: also the branch codes of every population's slopes (one byte x | y << 2
@@ -1158,7 +1158,7 @@ __global__ void __launch_bounds__(kCta, R == 8 ? 3 : 1) k_step_tile(const double
     collision(m);
   } else {
     // the first group sums f and forms the coefficients, the second sums g: all
-    // groups doing all of it would share the FP64 pipe (64^2: 22.6 -> 16.4 us)
+    // groups doing all of it would share the FP64 pipe (6 us more at 64^2)
     __shared__ double s_share[4][32 * R];
     __shared__ int s_block[2][32 * R];
     typename L::Mom m;

@@ -191,14 +191,14 @@ __device__ __forceinline__ void moments_fix16(const double* __restrict__ s, unsi
     if (k == 0) M2s += pair_sum16<2>(sB, sA);
   }
   const long long a0 = M0[0] + M0[1], b0 = M0[2] + M0[3], c0 = M0[0] - M0[1], d0 = M0[2] - M0[3];
-  const double s00 = key < 0x7ff00000u ? fix_to_double<true>(a0 + b0, sc) : __longlong_as_double(0x7ff8000000000000ll);
-  const double s10 = fix_to_double<true>(pair_sum16<1>(d0, c0), sc + 4);
-  const double s01 = fix_to_double<true>((M1[0] + M1[1]) + (M1[2] + M1[3]), sc + 4);
+  const double s00 = key < 0x7ff00000u ? fix_to_double(a0 + b0, sc) : __longlong_as_double(0x7ff8000000000000ll);
+  const double s10 = fix_to_double(pair_sum16<1>(d0, c0), sc + 4);
+  const double s01 = fix_to_double((M1[0] + M1[1]) + (M1[2] + M1[3]), sc + 4);
   if (k == 0) {
     m.m00 = s00; m.m10 = s10; m.m01 = s01;
-    m.m20 = fix_to_double<true>(pair_sum16<2>(b0, a0), sc + 5);
-    m.m02 = fix_to_double<true>(M2s, sc + 5);
-    m.m11 = fix_to_double<true>(pair_sum16<1>((M1[2] - M1[3]) << 4, (M1[0] - M1[1]) << 4), sc + 4);
+    m.m20 = fix_to_double(pair_sum16<2>(b0, a0), sc + 5);
+    m.m02 = fix_to_double(M2s, sc + 5);
+    m.m11 = fix_to_double(pair_sum16<1>((M1[2] - M1[3]) << 4, (M1[0] - M1[1]) << 4), sc + 4);
   } else {
     m.g00 = s00; m.g10 = s10; m.g01 = s01;
   }

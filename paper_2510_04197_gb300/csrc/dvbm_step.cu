@@ -15,11 +15,6 @@ namespace dvbm {
 // One thread per cell: moments and coefficients as above, the collision target
 // of each population rounded to float, the upwind-limited flux differences in
 // float on the deviations from L1-cached neighbours.
-// The ten populations (f and g, y-nodes q = 0..4) of x-node p; CENTER: p = 0
-// (xi_x = 0, no x-flux), otherwise p = 1..4 at run time, so that one copy of
-// this body serves the four moving x-nodes and the kernel's code stays small
-// enough for the instruction cache.  The y-node loop stays unrolled (1754 vs
-// 1722 MLUPS rolled at 4096^2).
 // the five targets t_q 2^(scale - kd(q)) of an x-node as floats: the hardware's
 // conversion (one slot of the FP64 pipe, which this kernel does not fill, for
 // about fifteen integer instructions) and two exact power-of-two factors
@@ -31,6 +26,11 @@ __device__ __forceinline__ void to_floats(const long long (&t)[5], int scale, fl
   for (int q = 0; q < 5; ++q) f[q] = (__ll2float_rn(t[q]) * m1) * (m2 * (1.0f / (float)(1 << kd(q))));
 }
 
+// The ten populations (f and g, y-nodes q = 0..4) of x-node p; CENTER: p = 0
+// (xi_x = 0, no x-flux), otherwise p = 1..4 at run time, so that one copy of
+// this body serves the four moving x-nodes and the kernel's code stays small
+// enough for the instruction cache.  The y-node loop stays unrolled (rolled it
+// measured 2 % slower at 4096^2).
 template <bool CENTER>
 __device__ __forceinline__ void node_update32(int p, const float* __restrict__ s, float* __restrict__ d, const Geom& G,
                                               const FixView& X, int Ef, int Eg, const Phys& P, float a1f) {
