@@ -442,19 +442,26 @@ __device__ __forceinline__ unsigned abs_key(double v) { return (unsigned)__doubl
 __device__ __forceinline__ unsigned abs_key(float v) { return __float_as_uint(v) & 0x7fffffffu; }
 
 // How a block of largest exponent E enters fixed point.  Below 2^-895 (E < 128) the
-// block is negligible: its integers' units would leave the range of doubles, so that
-// every value of it, of either sign, has to become exactly 0 (an integer of one unit
-// scaled below the smallest exponent wraps into numbers near 2^1000).
-struct BlockScale {
+// block is negligible: its integers' units would leave the range of doubles, and an
+// integer of one unit scaled below the smallest exponent wraps into numbers near
+// 2^1000.  Its values become 0, negative ones -1; Signed keeps them from that (exactly 0
+// for either sign) where the result is to be 0.  The forward step's kernels do
+// without the mask, which costs a 64^2 step 1.6 % and one on 4 x 256 with walls 2.6 %:
+// they scale at least at exponent 128, where a unit is below 1e-285.
+template <bool Signed>
+struct BlockScaleOf {
   int E, n0, sign;  // exponent, dropped bits (63: all), mask of the values' signs
-  __device__ __forceinline__ BlockScale(int E_, int bits, int tiny = 128)
-      : E(E_), n0(E_ < tiny ? 63 : bits), sign(E_ < tiny ? 0 : -1) {}
+  __device__ __forceinline__ BlockScaleOf(int E_, int bits, int tiny = 128)
+      : E(E_), n0(E_ < tiny ? 63 : bits), sign(Signed && E_ < tiny ? 0 : -1) {}
 };
+typedef BlockScaleOf<true> BlockScale;
+typedef BlockScaleOf<false> FlowScale;
 // Value v as an integer of 60 - n0 bits at the block exponent E (n0 >= 0):
 // v = X 2^(E - 1082 + n0); magnitudes are truncated, negative values are the
 // ones' complement of theirs (one unit more).  A value of larger exponent than
 // E (only non-finite ones are left out of the block maximum) gives 0 or -1.
-__device__ __forceinline__ long long block_fix(double v, const BlockScale& B) {
+template <bool Signed>
+__device__ __forceinline__ long long block_fix(double v, const BlockScaleOf<Signed>& B) {
   const int hi = __double2hiint(v);
   const unsigned lo = (unsigned)__double2loint(v);
   const int e = (hi >> 20) & 0x7ff;
@@ -464,7 +471,8 @@ __device__ __forceinline__ long long block_fix(double v, const BlockScale& B) {
   return (long long)(m >> n) ^ (long long)((hi >> 31) & B.sign);
 }
 // the same for a float: v = X 2^(E - 186 + n0)
-__device__ __forceinline__ long long block_fix(float v, const BlockScale& B) {
+template <bool Signed>
+__device__ __forceinline__ long long block_fix(float v, const BlockScaleOf<Signed>& B) {
   const int u = __float_as_int(v);
   const int e = (u >> 23) & 0xff;
   const unsigned mh = (((unsigned)u & 0x7fffffu) | 0x800000u) << 4;
@@ -532,7 +540,7 @@ __device__ __forceinline__ void moments_fix_f(const S* __restrict__ s, unsigned 
     key = max(key, abs_key(v[i]));
   }
   const int E = (int)(key >> K::kExpBits);
-  const BlockScale B(E, 2, K::kTiny);
+  const FlowScale B(E, 2, K::kTiny);
   long long M0[5], M1[5], M2[5], M3s = 0;  // y-sums of each x-node, M1, M2, M3 times 1/16, 1/64, 1/128
 #pragma unroll
   for (int p = 0; p < 5; ++p) {
@@ -549,7 +557,7 @@ __device__ __forceinline__ void moments_fix_f(const S* __restrict__ s, unsigned 
   // second factors: the first left four spare bits
   const long long a1 = M1[1] + M1[2], b1 = M1[3] + M1[4], c1 = M1[1] - M1[2], d1 = M1[3] - M1[4];
   const long long a2 = M2[1] + M2[2], b2 = M2[3] + M2[4], c2 = M2[1] - M2[2], d2 = M2[3] - M2[4];
-  const int sc = E - K::kBias;
+  const int sc = max(E, K::kTiny) - K::kBias;
   m.m00 = fix_to_double(M0[0] + a0 + b0, sc);
   m.m01 = fix_to_double(M1[0] + a1 + b1, sc + 4);
   m.m02 = fix_to_double(M2[0] + a2 + b2, sc + 6);
@@ -573,7 +581,7 @@ __device__ __forceinline__ void moments_fix_g(const S* __restrict__ s, unsigned 
     key = max(key, abs_key(v[i]));
   }
   const int E = (int)(key >> K::kExpBits);
-  const BlockScale B(E, 2, K::kTiny);
+  const FlowScale B(E, 2, K::kTiny);
   long long N0[5], N1s = 0;
 #pragma unroll
   for (int p = 0; p < 5; ++p) {
@@ -583,7 +591,7 @@ __device__ __forceinline__ void moments_fix_g(const S* __restrict__ s, unsigned 
     N0[p] = x0 + (x1 + x2) + (x3 + x4);
     N1s += pair_sum<1>(x3 - x4, x1 - x2);
   }
-  const int sc = E - K::kBias;
+  const int sc = max(E, K::kTiny) - K::kBias;
   m.g00 = fix_to_double(N0[0] + (N0[1] + N0[2]) + (N0[3] + N0[4]), sc);
   m.g01 = fix_to_double(N1s, sc + 4);
   m.g10 = fix_to_double(pair_sum<1>(N0[3] - N0[4], N0[1] - N0[2]), sc + 4);
@@ -728,7 +736,7 @@ __device__ __forceinline__ void advect_load(AdvLoad<R>& L, const double* __restr
 
 // out: the plane (at the tile's lowest cell, row pitch PT) where the tile's flux
 // sums go, kx (x-face difference) + ky (y-face difference) as integers W in
-// units of 2^(E - 1079), E the returned block exponent; MX, MY: the population
+// units of 2^(E - 1079), E the returned block exponent (at least 128); MX, MY: the population
 // moves along x, along y; kx, ky: flux factors (Phys::kxq, kyq); xs: this warp's
 // [R + 3][kAdvPitch] words of shared memory; code: (CODES) this population's
 // branch codes at the tile's lowest cell, row pitch cpitch; next: starts the
@@ -753,8 +761,8 @@ __device__ __forceinline__ int advect_tile(AdvLoad<R>& L, const Next& next, long
   if (MX) key = max(key, ((unsigned)__double2hiint(vh) + 0x100000u) & 0x7fffffffu);
   key = __reduce_max_sync(0xffffffffu, key);
   const int E = (int)(key >> 20) - 1;
-  const BlockScale B(E, P.advn);  // a block of negligible values has no flux
-  __syncwarp();                          // the previous population's reads of xs are done
+  const FlowScale B(E, P.advn);
+  __syncwarp();  // the previous population's reads of xs are done
 #pragma unroll
   for (int j = J0; j <= J1; ++j) xs[(j + 2) * kAdvPitch + lane + 2] = block_fix(v[j - J0], B);
   if (MX) {
@@ -817,7 +825,7 @@ __device__ __forceinline__ int advect_tile(AdvLoad<R>& L, const Next& next, long
     orow += sy;
     if (CODES) crow += csy;
   }
-  return E;
+  return max(E, 128);
 }
 
 // a1 F + target - flux sum of one population: the target t 2^(st - 1079) and
@@ -867,10 +875,10 @@ __device__ __forceinline__ void fields_to_smem(const double (&f)[N], long long* 
   unsigned key = 0;
 #pragma unroll
   for (int k = 0; k < N; ++k) key = max(key, abs_key(f[k]));
-  const BlockScale B((int)(key >> 20), 0);  // negligible coefficients: target 0
+  const FlowScale B((int)(key >> 20), 0);
 #pragma unroll
   for (int k = 0; k < N; ++k) b[k * STRIDE] = pack_limbs(block_fix(f[k], B));
-  E = max(B.E, 128);  // a zero target's exponent too lies where collide_advect's result is normal
+  E = max(B.E, 128);  // also where collide_advect's result of a zero target is normal
 }
 // h^b of x-node p: W_p sum_a C_ab He_a(xi_p)/a! (value h 2^(E - 1082 - kd(p)))
 template <class V>

@@ -178,8 +178,8 @@ __device__ __forceinline__ void moments_fix16(const double* __restrict__ s, unsi
     key = max(key, abs_key(v[i]));
   }
   const int E = (int)(key >> 20);
-  const BlockScale B(E, 2);
-  const int sc = E - 1080;
+  const FlowScale B(E, 2);
+  const int sc = max(E, 128) - 1080;
   long long M0[4], M1[4], M2s = 0;  // y-sums of each x-node, M1 and M2 times 1/16, 1/32
 #pragma unroll
   for (int p = 0; p < 4; ++p) {

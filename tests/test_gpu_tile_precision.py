@@ -83,3 +83,24 @@ def test_density_scaled_by_a_power_of_two(D, k, lattice, Pr):
         assert np.abs(a[s] - b[s]).max() <= 30 * 2.0 ** -53 * np.abs(a[s]).max()
     for q in ("ux", "uy", "T"):
         assert float((ma[q] - mb[q]).abs().max()) <= 60 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("Nx,Ny", [(64, 64), (128, 96), (640, 192)])
+@pytest.mark.parametrize("tiny", [-0.0, -1e-300, 1e-300, -3e-277])
+def test_negligible_populations_stay_negligible(D, Nx, Ny, tiny):
+    """gamma = 2 has no internal non-translational energy: g is zero.  Populations of g
+    below every block's range, of either sign, leave f as it is and stay below 1e-270."""
+    F = I.random_smooth(Nx, Ny, seed=5, amp=0.1, Ma=0.4)
+    dt = 0.3 * min(F.Lx / Nx, F.Ly / Ny) / 2.857
+    sim = D.Simulation(Nx, Ny, 0.71, 2.0, 8.0 * dt, Lx=F.Lx, Ly=F.Ly, dt=dt)
+    sim.init(*(torch.tensor(a) for a in (F.rho, F.ux, F.uy, F.T)))
+    st = sim.get_state()
+    sim.step(4)
+    clean = sim.populations().clone()
+    assert float(clean[25:].abs().max()) < 1e-270
+    sim.populations(st)[25:] = tiny
+    sim.set_state(st)
+    sim.step(4)
+    got = sim.populations()
+    assert torch.equal(got[:25], clean[:25])
+    assert float(got[25:].abs().max()) < 1e-270
