@@ -527,9 +527,9 @@ __device__ __forceinline__ double advection_adjoint_rat(const double* __restrict
 // step, in the forward step's two phases (k_step_tile): first one population per
 // warp over a 32 x R tile, then one cell per thread.  512^2: 0.47 ms for the two
 // kernels it replaces (one thread per cell and population in the advection, 64-bit
-// high products in the projection) -> 0.36 ms.  Bound by the FP64 pipe (54 % busy, about
-// 460 instructions a cell, half of them the reverse pass over the collision
-// coefficients) and by latency at 16 warps an SM.  100^2, all latency, with 4-row
+// high products in the projection) -> 0.36 ms.  Bound by the FP64 pipe (53 % busy, 436
+// instructions a cell, about half of them the reverse pass over the collision
+// coefficients) and by latency at 15 warps an SM.  100^2, all latency, with 4-row
 // tiles and the parts of a cell on several threads: 110 -> 75 us a step with the
 // recompute.
 
