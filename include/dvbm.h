@@ -280,7 +280,7 @@ dvbm_status dvbm_set_dt(dvbm_ctx* ctx, double dt);
  * chosen by the grid's size, whose cells share a block exponent; with the whole
  * grid's rows set in every band, bands that begin and end on multiples of 8 rows
  * (the last one ends with the grid) give bitwise the undecomposed run.  Without
- * it they agree to rounding.  Errors: EINVAL (rows < Ny), ESTATE (a stepwise
+ * it they agree to rounding.  Errors: EINVAL (rows < Ny or > 2^30), ESTATE (a stepwise
  * adjoint in progress or a recorded run that has stepped, and rows differs). */
 dvbm_status dvbm_set_grid_rows(dvbm_ctx* ctx, int rows);
 

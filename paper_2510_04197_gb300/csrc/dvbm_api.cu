@@ -677,6 +677,7 @@ extern "C" dvbm_status dvbm_set_dt(dvbm_ctx* c, double dt) {
 extern "C" dvbm_status dvbm_set_grid_rows(dvbm_ctx* c, int rows) {
   if (!c) return DVBM_EINVAL;
   if (rows < c->Ny) return fail(c, DVBM_EINVAL, "a grid of %d rows cannot hold this band of %d", rows, c->Ny);
+  if (rows > (1 << 30)) return fail(c, DVBM_EINVAL, "a grid of %d rows is out of range", rows);
   if (rows == c->G.grid_rows) return DVBM_OK;
   // the adjoint recomputes the recorded run with the context's tiles, and a pass in
   // progress has sized its partial sums by them

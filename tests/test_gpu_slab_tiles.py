@@ -62,9 +62,10 @@ def test_adjoint_bitwise(D, Nx, Ny, parts, Pr):
 def test_contract(D):
     F = I.random_smooth(32, 16, seed=2, amp=0.1, Ma=0.5)
     sim = D.Simulation(32, 16, 0.71, 1.4, 2e-3, dt=2e-4, Lx=F.Lx, Ly=F.Ly)
-    with pytest.raises(D.DVBMError) as e:  # fewer rows than the context's own
-        sim.set_grid_rows(15)
-    assert e.value.status == D.EINVAL
+    for rows in (15, 2 ** 31 - 1):  # fewer than the context's own; out of range
+        with pytest.raises(D.DVBMError) as e:
+            sim.set_grid_rows(rows)
+        assert e.value.status == D.EINVAL
     sim.set_grid_rows(4096).set_grid_rows(16)
     sim.record(2)
     sim.init(*(torch.tensor(v) for v in (F.rho, F.ux, F.uy, F.T)))
